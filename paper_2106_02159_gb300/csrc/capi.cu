@@ -80,7 +80,7 @@ struct eh_ctx {
   // work arrays (it is stepped inside the batch's own context)
   bool static_only = false;
   // a merged batch's context: the sizes its arrays were allocated for
-  int64_t cap_n = 0, cap_nnz = 0, cap_bnd = 0;
+  int64_t cap_n = 0, cap_nnz = 0, cap_bnd = 0, cap_bp = 0;
   int64_t rec_n = 0;  // nodes the record array was allocated for
 };
 
@@ -368,32 +368,31 @@ eh_status setup_instances(eh_ctx *c, int ninst, const int64_t *off, const double
   return EH_OK;
 }
 
-// Device arrays of the static mesh data for (up to) n nodes, nnz entries and
-// n_bnd boundary nodes; sets the MeshView pointers (contents not written).
-eh_status alloc_static(eh_ctx *c, int64_t n, int64_t nnz, int64_t n_bnd) {
+// Device arrays of the static mesh data for (up to) n nodes, nnz entries,
+// n_bnd boundary nodes and n_bp edges between two of them; sets the MeshView
+// pointers (contents not written).
+eh_status alloc_static(eh_ctx *c, int64_t n, int64_t nnz, int64_t n_bnd, int64_t n_bp) {
   const int dim = c->cfg.dim, S = S_of(c);
   MeshView &m = c->mv;
   eh_status st;
   int64_t *row = nullptr;
-  int32_t *col = nullptr, *tr = nullptr, *bidx = nullptr, *bnode = nullptr, *bkind = nullptr;
-  double *cij = nullptr, *cn = nullptr, *cinv = nullptr, *betat = nullptr, *mi = nullptr, *imi = nullptr,
+  int32_t *col = nullptr, *tr = nullptr, *bidx = nullptr, *bnode = nullptr, *bkind = nullptr, *bprow = nullptr,
+          *bppos = nullptr;
+  double *betat = nullptr, *mi = nullptr, *imi = nullptr,
          *relax = nullptr, *lam = nullptr, *bnorm = nullptr, *bstate = nullptr;
   unsigned char *isb = nullptr;
   if ((st = dalloc(c, &row, (size_t)n + 1)) || (st = dalloc(c, &col, (size_t)nnz)) ||
-      (st = dalloc(c, &tr, (size_t)nnz)) || (st = dalloc(c, &cij, (size_t)dim * nnz)) ||
-      (st = dalloc(c, &cn, (size_t)nnz)) || (st = dalloc(c, &cinv, (size_t)nnz)) ||
+      (st = dalloc(c, &tr, (size_t)nnz)) ||
       (st = dalloc(c, &betat, (size_t)nnz)) || (st = dalloc(c, &mi, (size_t)n)) || (st = dalloc(c, &imi, (size_t)n)) ||
       (st = dalloc(c, &relax, (size_t)n)) || (st = dalloc(c, &lam, (size_t)n)) || (st = dalloc(c, &isb, (size_t)n)) ||
       (st = dalloc(c, &bidx, (size_t)n)) || (st = dalloc(c, &bnode, (size_t)n_bnd)) ||
       (st = dalloc(c, &bkind, (size_t)n_bnd)) || (st = dalloc(c, &bnorm, (size_t)dim * n_bnd)) ||
-      (st = dalloc(c, &bstate, (size_t)S * n_bnd)))
+      (st = dalloc(c, &bstate, (size_t)S * n_bnd)) || (st = dalloc(c, &bprow, (size_t)n_bp)) ||
+      (st = dalloc(c, &bppos, (size_t)n_bp)))
     return st;
   m.row_ptr = row;
   m.col = col;
   m.tr = tr;
-  m.cij = cij;
-  m.cn = cn;
-  m.cinv = cinv;
   m.betat = betat;
   m.mi = mi;
   m.inv_mi = imi;
@@ -405,18 +404,14 @@ eh_status alloc_static(eh_ctx *c, int64_t n, int64_t nnz, int64_t n_bnd) {
   m.bnd_kind = bkind;
   m.bnd_normal = bnorm;
   m.bnd_state = bstate;
-  m.vcij = cij;
-  m.vcn = cn;
-  m.vcinv = cinv;
-  if (mixed(c)) {  // FP32 c_ij, |c_ij|, 1/|c_ij|
-    float *fc = nullptr, *fn = nullptr, *fi = nullptr;
-    if ((st = dalloc(c, &fc, (size_t)dim * nnz)) || (st = dalloc(c, &fn, (size_t)nnz)) ||
-        (st = dalloc(c, &fi, (size_t)nnz)))
-      return st;
-    m.vcij = fc;
-    m.vcn = fn;
-    m.vcinv = fi;
-  }
+  m.bp_row = bprow;
+  m.bp_pos = bppos;
+  const size_t vsz = mixed(c) ? sizeof(float) : sizeof(double);
+  char *geo = nullptr, *ginv = nullptr;
+  if ((st = dalloc(c, &geo, 4 * vsz * (size_t)nnz))) return st;
+  if (dim == 3 && (st = dalloc(c, &ginv, vsz * (size_t)nnz))) return st;
+  m.geo = geo;
+  m.geo_inv = ginv;
   return EH_OK;
 }
 
@@ -459,29 +454,25 @@ eh_status alloc_work(eh_ctx *c, int64_t n, int64_t nnz) {
     static_assert(EdgeLayout<2, float>::packed && EdgeLayout<3, float>::packed, "FP32 edge slots are packed");
     constexpr int spw_f = EdgeLayout<2, float>::SPW;
     ALLOC(f_w, (size_t)nnz * spw_f);
-    w.va = nullptr;
+    w.vad = nullptr;
     w.vrec = f_rec;
     w.vw = f_w;
-    w.vd = nullptr;
     w.vFH = f_fh;
     ALLOC(w.G64, (size_t)n * SP);
   } else {
     ALLOC(w.FH, (size_t)n * SP);
-    double *d_a = nullptr;
+    double *d_ad = nullptr;
     if (dim == 3) {  // packed slots [w (5), a, d, 0]
       constexpr int spw3 = EdgeLayout<3, double>::SPW;
       ALLOC(w.w, (size_t)nnz * spw3);
-      w.d = nullptr;
     } else {
       constexpr int spw2 = EdgeLayout<2, double>::SPW;
       ALLOC(w.w, (size_t)nnz * spw2);
-      ALLOC(w.d, nnz);
-      ALLOC(d_a, nnz);
+      ALLOC(d_ad, 2 * (size_t)nnz);
     }
-    w.va = d_a;
+    w.vad = d_ad;
     w.vrec = w.rec;
     w.vw = w.w;
-    w.vd = w.d;
     w.vFH = w.FH;
     w.G64 = w.FH;
   }
@@ -635,7 +626,7 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
     // 512 rows in flight per SM on k_pass, which kept a 27-entry row's lines
     // of P in L1 while its second walk still re-read all of them)
     c->tpb[EH_KERNEL_PREP] = 64;
-    c->tpb[EH_KERNEL_VISC] = 64;
+    c->tpb[EH_KERNEL_VISC] = 128;
     c->tpb[EH_KERNEL_LOW] = 64;
     c->tpb[EH_KERNEL_LIM1] = 128;
     c->tpb[EH_KERNEL_PASS] = 256;
@@ -648,6 +639,7 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
     for (int k = 0; k < EH_KERNEL_COUNT; ++k)
       if (k != EH_KERNEL_TAU) c->tpb[k] = 64;
     c->tpb[EH_KERNEL_LSEARCH] = 128;
+    c->tpb[EH_KERNEL_VISC] = 128;
   }
   Params &p = c->prm;
   p.gamma = cfg->gamma;
@@ -659,6 +651,9 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
   p.inv_z = 1.0 / p.z;
   p.kshock = (cfg->gamma + 1.0) / (2.0 * cfg->gamma);
   p.inv_gm1 = 1.0 / (cfg->gamma - 1.0);
+  p.gm1_f = (float)p.gm1;
+  p.inv_z_f = (float)p.inv_z;
+  p.kshock_f = (float)p.kshock;
   *out = c;
   return EH_OK;
 }
@@ -712,14 +707,29 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
       tr[k] = (int32_t)(row_ptr[j] + (f - b));
     }
   }
-  std::vector<double> cn(nnz), cinv(nnz), betat(nnz);
+  // c_ij, |c_ij|, 1/|c_ij| per entry in the viscosity precision (MeshView::geo)
+  std::vector<double> betat(nnz), geo64, ginv64;
+  std::vector<float> geo32, ginv32;
+  if (mixed(c)) geo32.resize(4 * (size_t)nnz); else geo64.resize(4 * (size_t)nnz);
+  if (dim == 3) {
+    if (mixed(c)) ginv32.resize(nnz); else ginv64.resize(nnz);
+  }
   for (int i = 0; i < n; ++i) {
     for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
       double s2 = 0.0;
       for (int d = 0; d < dim; ++d) s2 += cij[(int64_t)d * nnz + k] * cij[(int64_t)d * nnz + k];
-      cn[k] = std::sqrt(s2);
-      cinv[k] = cn[k] > 0.0 ? 1.0 / cn[k] : 0.0;
-      if (col[k] != i && !(cn[k] > 0.0)) return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry");
+      const double cn = std::sqrt(s2), cinv = cn > 0.0 ? 1.0 / cn : 0.0;
+      if (col[k] != i && !(cn > 0.0)) return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry");
+      double g[5];
+      for (int d = 0; d < dim; ++d) g[d] = cij[(int64_t)d * nnz + k];
+      g[dim] = cn;
+      g[dim + 1] = cinv;
+      for (int q = 0; q < 4; ++q) {
+        if (mixed(c)) geo32[4 * k + q] = (float)g[q]; else geo64[4 * k + q] = g[q];
+      }
+      if (dim == 3) {
+        if (mixed(c)) ginv32[k] = (float)cinv; else ginv64[k] = cinv;
+      }
       // the consistent mass matrix is symmetric (m_ij = int phi_i phi_j);
       // k_lim1 relies on it, with the mean of the two entries
       const double a = mij[k], b = mij[tr[k]];
@@ -748,9 +758,17 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
     isb[i] = 1;
     bidx[i] = b;
   }
+  std::vector<int32_t> bprow, bppos;  // edges between two boundary nodes, from the smaller one's row
+  for (int i = 0; i < n; ++i)
+    if (isb[i])
+      for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k)
+        if (col[k] > i && isb[col[k]]) {
+          bprow.push_back(i);
+          bppos.push_back((int32_t)k);
+        }
   // ---- device arrays ----
   eh_status st;
-  if ((st = alloc_static(c, n, nnz, n_bnd)) != EH_OK) {
+  if ((st = alloc_static(c, n, nnz, n_bnd, (int64_t)bprow.size())) != EH_OK) {
     free_mesh(c);
     return st;
   }
@@ -763,9 +781,12 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   if (e == cudaSuccess) e = up(m.row_ptr, row_ptr, sizeof(int64_t) * (n + 1));
   if (e == cudaSuccess) e = up(m.col, col, sizeof(int32_t) * nnz);
   if (e == cudaSuccess) e = up(m.tr, tr.data(), sizeof(int32_t) * nnz);
-  if (e == cudaSuccess) e = up(m.cij, cij, sizeof(double) * dim * nnz);
-  if (e == cudaSuccess) e = up(m.cn, cn.data(), sizeof(double) * nnz);
-  if (e == cudaSuccess) e = up(m.cinv, cinv.data(), sizeof(double) * nnz);
+  if (e == cudaSuccess) {
+    const size_t v = mixed(c) ? sizeof(float) : sizeof(double);
+    e = up(m.geo, mixed(c) ? (const void *)geo32.data() : (const void *)geo64.data(), 4 * v * nnz);
+    if (e == cudaSuccess && dim == 3)
+      e = up(m.geo_inv, mixed(c) ? (const void *)ginv32.data() : (const void *)ginv64.data(), v * nnz);
+  }
   if (e == cudaSuccess) e = up(m.betat, betat.data(), sizeof(double) * nnz);
   if (e == cudaSuccess) e = up(m.mi, mi, sizeof(double) * n);
   if (e == cudaSuccess) e = up(m.inv_mi, inv_mi.data(), sizeof(double) * n);
@@ -777,16 +798,8 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   if (e == cudaSuccess) e = up(m.bnd_kind, bnd_kind, sizeof(int32_t) * n_bnd);
   if (e == cudaSuccess) e = up(m.bnd_normal, bnd_normal, sizeof(double) * dim * n_bnd);
   if (e == cudaSuccess && bnd_state) e = up(m.bnd_state, bnd_state, sizeof(double) * S * n_bnd);
-  if (e == cudaSuccess && mixed(c)) {
-    std::vector<float> tmp((size_t)dim * nnz);
-    for (size_t q = 0; q < tmp.size(); ++q) tmp[q] = (float)cij[q];
-    e = up(m.vcij, tmp.data(), sizeof(float) * tmp.size());
-    tmp.resize(nnz);
-    for (int64_t k = 0; e == cudaSuccess && k < nnz; ++k) tmp[k] = (float)cn[k];
-    if (e == cudaSuccess) e = up(m.vcn, tmp.data(), sizeof(float) * nnz);
-    for (int64_t k = 0; e == cudaSuccess && k < nnz; ++k) tmp[k] = (float)cinv[k];
-    if (e == cudaSuccess) e = up(m.vcinv, tmp.data(), sizeof(float) * nnz);
-  }
+  if (e == cudaSuccess) e = up(m.bp_row, bprow.data(), sizeof(int32_t) * bprow.size());
+  if (e == cudaSuccess) e = up(m.bp_pos, bppos.data(), sizeof(int32_t) * bppos.size());
   if (e != cudaSuccess) {
     free_mesh(c);
     return fail(c, EH_ERR_CUDA, "mesh upload: %s", cudaGetErrorString(e));
@@ -794,6 +807,7 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   m.n = n;
   m.nnz = nnz;
   m.n_bnd = n_bnd;
+  m.n_bp = (int)bprow.size();
   m.n_nonreflecting = 0;
   for (int b = 0; b < n_bnd; ++b)
     if (bnd_kind[b] == EH_BC_CHARACTERISTIC || bnd_kind[b] == EH_BC_GODUNOV) ++m.n_nonreflecting;
@@ -1520,8 +1534,8 @@ eh_status eh_trace(eh_ctx *c, int what, double *host_out, int64_t count) {
         for (int64_t k = 0; k < nnz; ++k) host_out[k] = buf[k * spw + dpos];
         return EH_OK;
       }
-      if ((st = vcopy(c->wk.vd, nnz, buf))) return st;
-      std::copy(buf.begin(), buf.end(), host_out);
+      if ((st = vcopy(c->wk.vad, 2 * nnz, buf))) return st;  // [a, d] pairs
+      for (int64_t k = 0; k < nnz; ++k) host_out[k] = buf[2 * k + 1];
       return EH_OK;
     case EH_TRACE_ALPHA:  // stored halved
       if ((st = plain(c->wk.alpha, n))) return st;
@@ -1608,24 +1622,27 @@ eh_status assemble(eh_ctx *uni, eh_ctx *const *parts, int count, const double *t
   CUDA_TRY(uni, cudaSetDevice(uni->device));
   CUDA_TRY(uni, cudaStreamSynchronize(uni->stream));
   const int dim = uni->cfg.dim, S = S_of(uni);
-  int64_t N = 0, NNZ = 0, NB = 0;
+  int64_t N = 0, NNZ = 0, NB = 0, NBP = 0;
   for (int k = 0; k < count; ++k) {
     N += parts[k]->n;
+    NBP += parts[k]->mv.n_bp;
     NNZ += parts[k]->nnz;
     NB += parts[k]->n_bnd;
   }
   if (N > INT32_MAX || NNZ >= ((int64_t)1 << 31)) return fail(uni, EH_ERR_INVALID_ARG, "merged batch too large");
   eh_status st;
-  if (!uni->have_mesh || N > uni->cap_n || NNZ > uni->cap_nnz || NB > uni->cap_bnd) {
+  if (!uni->have_mesh || N > uni->cap_n || NNZ > uni->cap_nnz || NB > uni->cap_bnd ||
+      NBP > uni->cap_bp) {
     free_mesh(uni);
     // room to grow: the next arrivals are placed without reallocating
     uni->cap_n = std::min<int64_t>(INT32_MAX, N + N / 4 + 1024);
     uni->cap_nnz = std::min<int64_t>(((int64_t)1 << 31) - 1, NNZ + NNZ / 4 + 16384);
     uni->cap_bnd = NB + NB / 4 + 256;
-    if ((st = alloc_static(uni, uni->cap_n, uni->cap_nnz, uni->cap_bnd)) ||
+    uni->cap_bp = NBP + NBP / 4 + 256;
+    if ((st = alloc_static(uni, uni->cap_n, uni->cap_nnz, uni->cap_bnd, uni->cap_bp)) ||
         (st = alloc_work(uni, uni->cap_n, uni->cap_nnz))) {
       free_mesh(uni);
-      uni->cap_n = uni->cap_nnz = uni->cap_bnd = 0;
+      uni->cap_n = uni->cap_nnz = uni->cap_bnd = uni->cap_bp = 0;
       return st;
     }
   }
@@ -1635,7 +1652,7 @@ eh_status assemble(eh_ctx *uni, eh_ctx *const *parts, int count, const double *t
     if (bytes) cudaMemcpyAsync(const_cast<void *>(dst), src, bytes, cudaMemcpyDeviceToDevice, s);
   };
   const size_t vsz = mixed(uni) ? sizeof(float) : sizeof(double);
-  int64_t ro = 0, eo = 0, bo = 0;
+  int64_t ro = 0, eo = 0, bo = 0, po = 0;
   int nonrefl = 0;
   for (int k = 0; k < count; ++k) {
     const eh_ctx *p = parts[k];
@@ -1644,18 +1661,9 @@ eh_status assemble(eh_ctx *uni, eh_ctx *const *parts, int count, const double *t
     launch_offset_copy<int64_t>(const_cast<int64_t *>(m.row_ptr) + ro, pm.row_ptr, n, eo, false, s);
     launch_offset_copy<int32_t>(const_cast<int32_t *>(m.col) + eo, pm.col, nnz, (int32_t)ro, false, s);
     launch_offset_copy<int32_t>(const_cast<int32_t *>(m.tr) + eo, pm.tr, nnz, (int32_t)eo, false, s);
-    for (int q = 0; q < dim; ++q) {
-      cp(m.cij + (int64_t)q * NNZ + eo, pm.cij + (int64_t)q * nnz, sizeof(double) * nnz);
-      cp((const char *)m.vcij + vsz * ((int64_t)q * NNZ + eo), (const char *)pm.vcij + vsz * (int64_t)q * nnz,
-         vsz * nnz);
-    }
-    cp(m.cn + eo, pm.cn, sizeof(double) * nnz);
-    cp(m.cinv + eo, pm.cinv, sizeof(double) * nnz);
+    cp((const char *)m.geo + 4 * vsz * eo, pm.geo, 4 * vsz * nnz);
+    if (dim == 3) cp((const char *)m.geo_inv + vsz * eo, pm.geo_inv, vsz * nnz);
     cp(m.betat + eo, pm.betat, sizeof(double) * nnz);
-    if (mixed(uni)) {
-      cp((const char *)m.vcn + vsz * eo, pm.vcn, vsz * nnz);
-      cp((const char *)m.vcinv + vsz * eo, pm.vcinv, vsz * nnz);
-    }
     cp(m.mi + ro, pm.mi, sizeof(double) * n);
     cp(m.inv_mi + ro, pm.inv_mi, sizeof(double) * n);
     cp(m.relax + ro, pm.relax, sizeof(double) * n);
@@ -1667,10 +1675,13 @@ eh_status assemble(eh_ctx *uni, eh_ctx *const *parts, int count, const double *t
     for (int q = 0; q < dim; ++q) cp(m.bnd_normal + (int64_t)q * NB + bo, pm.bnd_normal + (int64_t)q * nb, 8 * nb);
     for (int c = 0; c < S; ++c) cp(m.bnd_state + (int64_t)c * NB + bo, pm.bnd_state + (int64_t)c * nb, 8 * nb);
     for (int c = 0; c < S; ++c) cp(uni->U + (int64_t)c * N + ro, p->U + (int64_t)c * n, 8 * n);
+    launch_offset_copy<int32_t>(const_cast<int32_t *>(m.bp_row) + po, pm.bp_row, pm.n_bp, (int32_t)ro, false, s);
+    launch_offset_copy<int32_t>(const_cast<int32_t *>(m.bp_pos) + po, pm.bp_pos, pm.n_bp, (int32_t)eo, false, s);
     nonrefl += pm.n_nonreflecting;
     ro += n;
     eo += nnz;
     bo += nb;
+    po += pm.n_bp;
   }
   CUDA_TRY(uni, cudaGetLastError());
   CUDA_TRY(uni, cudaMemcpyAsync(const_cast<int64_t *>(m.row_ptr) + N, &NNZ, sizeof(int64_t), cudaMemcpyHostToDevice, s));
@@ -1678,6 +1689,7 @@ eh_status assemble(eh_ctx *uni, eh_ctx *const *parts, int count, const double *t
   m.n = (int)N;
   m.nnz = NNZ;
   m.n_bnd = (int)NB;
+  m.n_bp = (int)NBP;
   m.n_nonreflecting = nonrefl;
   uni->n = (int)N;
   uni->nnz = NNZ;

@@ -69,59 +69,126 @@ __device__ __forceinline__ double abs_bits(double x) {
 }
 __device__ __forceinline__ float abs_bits(float x) { return fabsf(x); }
 
+// 256-bit accesses (sm_100 on): a lane's 32-byte sector in one instruction.
+// Lanes of a row kernel read sectors of different lines (rows are 64 to 288
+// bytes apart), so L1 serves one lane's line at a time whatever the width:
+// with 8-byte loads and stores the viscosity kernel ran its L1 at 74-81 % and
+// wrote five times the sectors it had values for. The loads are of data that
+// the kernel does not write.
+__device__ __forceinline__ void ld4(const double *p, double &a, double &b, double &c, double &d) {
+  asm("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
+}
+__device__ __forceinline__ void ld4(const float *p, float &a, float &b, float &c, float &d) {
+  const float4 v = *reinterpret_cast<const float4 *>(p);
+  a = v.x;
+  b = v.y;
+  c = v.z;
+  d = v.w;
+}
+__device__ __forceinline__ void st4(double *p, double a, double b, double c, double d) {
+  asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+}
+__device__ __forceinline__ void ld8(const float *p, float *v) {
+  asm("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+__device__ __forceinline__ void st8(float *p, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]),
+               "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void ld2(const double *p, double &a, double &b) {
+  const double2 v = *reinterpret_cast<const double2 *>(p);
+  a = v.x;
+  b = v.y;
+}
+// a state vector of stride Layout::SP (2D: one sector; 3D: 48 bytes)
+template <int DIM> __device__ __forceinline__ void load_vec(const double *p, double *v) {
+  if constexpr (DIM == 2) {
+    ld4(p, v[0], v[1], v[2], v[3]);
+  } else {
+    ld2(p, v[0], v[1]);
+    ld2(p + 2, v[2], v[3]);
+    v[4] = p[4];
+  }
+}
+template <int DIM> __device__ __forceinline__ void store_vec(double *p, const double *v) {
+  if constexpr (DIM == 2) {
+    st4(p, v[0], v[1], v[2], v[3]);
+  } else {
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+    p[4] = v[4];
+  }
+}
+// the state of a node from its FP64 record
+template <int DIM> __device__ __forceinline__ void load_rec_state(const double *R, double *u) {
+  ld4(R, u[0], u[1], u[2], u[3]);
+  if constexpr (DIM == 3) u[4] = R[4];
+}
+
 // the per-entry viscosity quantities (layout: EdgeLayout)
 template <int DIM, typename T> __device__ __forceinline__ T *w_slot(const Work &w, int64_t k) {
   return (T *)w.vw + k * EdgeLayout<DIM, T>::SPW;
 }
 template <int DIM, typename T> __device__ __forceinline__ T *d_ptr(const Work &w, int64_t k) {
-  return EdgeLayout<DIM, T>::packed ? w_slot<DIM, T>(w, k) + EdgeLayout<DIM, T>::D : (T *)w.vd + k;
+  return EdgeLayout<DIM, T>::packed ? w_slot<DIM, T>(w, k) + EdgeLayout<DIM, T>::D : (T *)w.vad + 2 * k + 1;
 }
-template <int DIM, typename T> __device__ __forceinline__ T *a_ptr(const Work &w, int64_t k) {
-  return EdgeLayout<DIM, T>::packed ? w_slot<DIM, T>(w, k) + EdgeLayout<DIM, T>::A : (T *)w.va + k;
-}
-// one packed slot [w (S), a, d, 0...] of 8 values in whole-sector vector stores
-template <int S> __device__ __forceinline__ void store_slot(double *p, const double *wv, double a, double d) {
-  double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+// w_ij (S values), a_ij and d_ij of entry k
+template <int DIM, typename T>
+__device__ __forceinline__ void store_edge(const Work &w, int64_t k, const T *wv, T a, T d) {
+  constexpr int S = DIM + 2;
+  if constexpr (sizeof(T) == 4) {
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-  for (int s = 0; s < S; ++s) v[s] = wv[s];
-  v[S] = a;
-  v[S + 1] = d;
-  double2 *q = reinterpret_cast<double2 *>(p);
+    for (int s = 0; s < S; ++s) v[s] = wv[s];
+    v[S] = a;
+    v[S + 1] = d;
+    st8(w_slot<DIM, T>(w, k), v);
+  } else if constexpr (DIM == 3) {
+    st4(w_slot<DIM, T>(w, k), wv[0], wv[1], wv[2], wv[3]);
+    st4(w_slot<DIM, T>(w, k) + 4, wv[S - 1], a, d, 0.0);
+  } else {
+    st4(w_slot<DIM, T>(w, k), wv[0], wv[1], wv[2], wv[3]);
+    reinterpret_cast<double2 *>(w.vad)[k] = make_double2(a, d);
+  }
+}
+template <int DIM, typename T>
+__device__ __forceinline__ void load_edge(const Work &w, int64_t k, T *wv, T &a, T &d) {
+  constexpr int S = DIM + 2;
+  if constexpr (sizeof(T) == 4) {
+    float v[8];
+    ld8(w_slot<DIM, T>(w, k), v);
 #pragma unroll
-  for (int h = 0; h < 4; ++h) q[h] = make_double2(v[2 * h], v[2 * h + 1]);
+    for (int s = 0; s < S; ++s) wv[s] = v[s];
+    a = v[S];
+    d = v[S + 1];
+  } else if constexpr (DIM == 3) {
+    double z;
+    ld4(w_slot<DIM, T>(w, k), wv[0], wv[1], wv[2], wv[3]);
+    ld4(w_slot<DIM, T>(w, k) + 4, wv[S - 1], a, d, z);
+  } else {
+    ld4(w_slot<DIM, T>(w, k), wv[0], wv[1], wv[2], wv[3]);
+    ld2((const double *)w.vad + 2 * k, a, d);
+  }
 }
-// one 32-byte sector of FP64 values
-__device__ __forceinline__ void store_sector(double *p, double x0, double x1, double x2, double x3) {
-  double2 *q = reinterpret_cast<double2 *>(p);
-  q[0] = make_double2(x0, x1);
-  q[1] = make_double2(x2, x3);
-}
-template <int S> __device__ __forceinline__ void store_slot(float *p, const float *wv, float a, float d) {
-  float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int s = 0; s < S; ++s) v[s] = wv[s];
-  v[S] = a;
-  v[S + 1] = d;
-  float4 *q = reinterpret_cast<float4 *>(p);
-  q[0] = make_float4(v[0], v[1], v[2], v[3]);
-  q[1] = make_float4(v[4], v[5], v[6], v[7]);
-}
-
 // the entry k of an edge between equal states: w = 0, a = 0, and d
 template <int DIM, typename T> __device__ __forceinline__ void store_zero_edge(const Work &w, int64_t k, T d) {
-  constexpr int S = DIM + 2;
-  if constexpr (!EdgeLayout<DIM, T>::packed) {
-    store_sector((double *)w_slot<DIM, T>(w, k), 0.0, 0.0, 0.0, 0.0);
-    *a_ptr<DIM, T>(w, k) = T(0);
-    *d_ptr<DIM, T>(w, k) = d;
-  } else if constexpr (sizeof(T) == 8) {  // FP64 3D: two sectors [w0..w3], [w4, a, d, 0]
-    store_sector((double *)w_slot<DIM, T>(w, k), 0.0, 0.0, 0.0, 0.0);
-    store_sector((double *)w_slot<DIM, T>(w, k) + 4, 0.0, 0.0, (double)d, 0.0);
-  } else {
-    T z[S];
+  T z[DIM + 2];
 #pragma unroll
-    for (int s = 0; s < S; ++s) z[s] = T(0);
-    store_slot<S>(w_slot<DIM, T>(w, k), z, T(0), d);
+  for (int s = 0; s < DIM + 2; ++s) z[s] = T(0);
+  store_edge<DIM, T>(w, k, z, T(0), d);
+}
+// c_ij, |c_ij| and 1/|c_ij| of entry k (MeshView::geo)
+template <int DIM, typename T>
+__device__ __forceinline__ void load_geo(const MeshView &m, int64_t k, T *c, T &cn, T &ci) {
+  const T *g = (const T *)m.geo + 4 * k;
+  if constexpr (DIM == 2) {
+    ld4(g, c[0], c[1], cn, ci);
+  } else {
+    ld4(g, c[0], c[1], c[2], cn);
+    ci = ((const T *)m.geo_inv)[k];
   }
 }
 
@@ -200,6 +267,113 @@ __device__ __forceinline__ T lambda_max(const Params &p, T unl, T pl, T al, T az
   T lam1 = unl - al * sl;
   T lam3 = unr + ar * sr;
   return max_nonneg(pos_part(-lam1), pos_part(lam3));
+}
+
+// x rounded towards zero to FP32 on the integer units (relative error 2^-23;
+// 0 below 2^-126, +-inf from 2^127 on and for NaN): an FP64 -> FP32 conversion
+// instruction takes part of an FP64 issue slot, this takes none
+__device__ __forceinline__ float trunc_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu, sg = hi & 0x80000000u;
+  unsigned r = ((__funnelshift_l(lo, hi, 3) - (384u << 23)) & 0x7fffffffu) | sg;
+  if (e < 897u) r = sg;
+  if (e > 1149u) r = sg | 0x7f800000u;
+  return __uint_as_float(r);
+}
+
+// a and p of a node as an FP32 pair in one FP64 slot of its record (Rec::F32),
+// for lambda_max_sel; a = NaN when a, p or a p^-z could leave FP32's range
+__device__ __forceinline__ double pack_f32(double a, double pr, double az) {
+  const bool ok = gt_pos(a, 1e-15) && lt_pos(a, 1e15) && gt_pos(pr, 1e-25) && lt_pos(pr, 1e25) && gt_pos(az, 1e-25) &&
+                  lt_pos(az, 1e25);
+  const float af = ok ? __double2float_rn(a) : __int_as_float(0x7fffffff);
+  return __hiloint2double(__float_as_int(__double2float_rn(pr)), __float_as_int(af));
+}
+__device__ __forceinline__ float2 unpack_f32(double x) {
+  return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x)));
+}
+
+// lambda_max in FP64, evaluated only where it can matter; the value is that of
+// lambda_max above, bit for bit. The result is the larger of two outer speeds
+// (a_l s_l - u_l and u_r + a_r s_r), each with s = 1 unless p_tr exceeds that
+// side's pressure. FP32 intervals around both decide, where they are clear,
+// which speed is the larger (the other side's root is not evaluated) and
+// whether p_tr stays below the pressure there (then neither p_tr -- a division
+// and a power -- nor a root is). An FP64 instruction costs 76 FP32 ones on this
+// part, and neighbouring rows agree on their decisions, so the intervals cost
+// little against the ~25 of 64 FP64 issue slots an edge that they save.
+// Errors, u = 2^-24: a and p are rounded (u), a p^-z, v.c and 1/|c| truncated
+// (2u); normal velocities 5u; the numerator of p_tr 6u of its terms'
+// magnitudes (gamma <= 5/3); the quotient 8u more; the seventh power (or exp2
+// of inv_z log2) multiplies the relative error by 7 (inv_z). Anything unclear,
+// or out of FP32's range (a = NaN), takes the full evaluation.
+__device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, double vcr, double ci, double pl, double al,
+                                                 double azl, double ipl, float2 fl, double pr, double ar, double azr,
+                                                 double ipr, float2 fr) {
+  constexpr float u = 5.9604645e-8f;  // 2^-24
+  const float cif = trunc_f32(ci);
+  const float ulf = trunc_f32(vcl) * cif, urf = trunc_f32(vcr) * cif;
+  const float num_f = fl.x + fr.x - 0.5f * p.gm1_f * (urf - ulf);
+  const float mag = fl.x + fr.x + fabsf(ulf) + fabsf(urf);
+  const float en = __fdividef(6.0f * u * mag, num_f);  // relative error of the numerator
+  const float xf = __fdividef(num_f, trunc_f32(azl) + trunc_f32(azr));
+  float ptr_f, rel;
+  if (p.gamma75) {
+    const float x2 = xf * xf;
+    ptr_f = x2 * x2 * x2 * xf;
+    rel = 7.5f * en + 80.0f * u;
+  } else {
+    const float lg = log2f(xf);
+    ptr_f = exp2f(p.inv_z_f * lg);
+    rel = 1.2f * p.inv_z_f * (en + 12.0f * u + 4.0f * u * fabsf(lg)) + 24.0f * u;
+  }
+  bool left = false, two = true, need = true;
+  if (num_f > 0.0f && en < 0.01f && rel < 0.05f && ptr_f > 1e-30f && ptr_f < 1e30f && mag < 1e18f) {
+    const float plo = ptr_f * (1.0f - rel), phi = ptr_f * (1.0f + rel);
+    const float ql = __fdividef(1.0f, fl.y), qr = __fdividef(1.0f, fr.y);
+    constexpr float r8 = 8.0f * u;
+    const float kf = p.kshock_f;
+    // brackets of s - 1's argument; 1 -/+ 8u covers p, 1/p and the products
+    const float sl_lo = sqrtf(1.0f + kf * fmaxf(plo * ql * (1.0f - r8) - 1.0f - r8, 0.0f));
+    const float sl_hi = sqrtf(1.0f + kf * fmaxf(phi * ql * (1.0f + r8) - 1.0f + r8, 0.0f));
+    const float sr_lo = sqrtf(1.0f + kf * fmaxf(plo * qr * (1.0f - r8) - 1.0f - r8, 0.0f));
+    const float sr_hi = sqrtf(1.0f + kf * fmaxf(phi * qr * (1.0f + r8) - 1.0f + r8, 0.0f));
+    const float el = 12.0f * u * (fl.x * sl_hi + fabsf(ulf)), er = 12.0f * u * (fr.x * sr_hi + fabsf(urf));
+    const bool L = fl.x * sl_lo - ulf - el > fr.x * sr_hi + urf + er;
+    const bool R = fr.x * sr_lo + urf - er > fl.x * sl_hi - ulf + el;
+    if (L || R) {
+      left = L;
+      two = false;
+      need = !(phi < (L ? fl.y : fr.y) * (1.0f - r8));
+    }
+  }
+  // the selected side (the right one first when both are evaluated)
+  const double as = left ? al : ar;
+  if (!need) {
+    const double us = __dmul_rn(left ? -vcl : vcr, ci);
+    return pos_part(us + as);
+  }
+  const double unl = __dmul_rn(vcl, ci), unr = __dmul_rn(vcr, ci);
+  double num = __fma_rn(-(0.5 * p.gm1), __dsub_rn(unr, unl), al + ar);
+  num = pos_part(num);
+  const double x = num / (azl + azr);
+  double ptr;
+  if (p.gamma75) {
+    const double x2 = x * x;
+    const double x4 = x2 * x2;
+    ptr = x4 * x2 * x;  // x^(2 gamma/(gamma-1)) = x^7
+  } else {
+    ptr = pow(x, p.inv_z);
+  }
+  const double ks = p.kshock;
+  const double ps = left ? pl : pr, ips = left ? ipl : ipr, us = left ? -unl : unr;
+  const double ss = gt_nonneg(ptr, ps) ? sqrt(1.0 + ks * (ptr - ps) * ips) : 1.0;
+  double lam = pos_part(us + as * ss);
+  if (two) {
+    const double so = gt_nonneg(ptr, pl) ? sqrt(1.0 + ks * (ptr - pl) * ipl) : 1.0;
+    lam = max_nonneg(lam, pos_part(-(unl - al * so)));
+  }
+  return lam;
 }
 
 // ---------------------------------------------------------------------------
@@ -572,8 +746,10 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
     // (every P_ij and increment is 0). The records start as NaN bit patterns,
     // which no admissible state matches.
     bool same = true;
+    double old[S];
+    load_rec_state<DIM>(Rr, old);
 #pragma unroll
-    for (int s = 0; s < S; ++s) same &= dbits(Rr[s]) == dbits(u[s]);
+    for (int s = 0; s < S; ++s) same &= dbits(old[s]) == dbits(u[s]);
     steady[i] = same ? (unsigned char)(was_rough ? 1 : 3) : (unsigned char)0;
     if (same) return;
   }
@@ -599,27 +775,33 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
     phi = eps * pow(rho, -p.gamma);
   }
   double eta = -rho * (log(phi) * p.inv_gm1);
+  double r[R::SIZE];
 #pragma unroll
-  for (int s = 0; s < S; ++s) Rr[s] = u[s];
+  for (int q = 0; q < R::SIZE; ++q) r[q] = 0.0;
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) Rr[R::V + k] = v[k];
-  Rr[R::P] = pr;
-  Rr[R::A] = a;
-  Rr[R::AZ] = az;
-  Rr[R::IP] = 1.0 / pr;
-  Rr[R::PHI] = phi;
-  Rr[R::ETA] = eta;
-  Rr[R::EPS] = eps;
-  Rr[R::H] = u[S - 1] + pr;
-  Rr[R::IRHO] = irho;
-  Rr[R::IEPS] = 1.0 / eps;
+  for (int s = 0; s < S; ++s) r[s] = u[s];
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) r[R::V + k] = v[k];
+  r[R::P] = pr;
+  r[R::A] = a;
+  r[R::AZ] = az;
+  r[R::IP] = 1.0 / pr;
+  r[R::PHI] = phi;
+  r[R::ETA] = eta;
+  r[R::H] = u[S - 1] + pr;
+  r[R::IRHO] = irho;
+  r[R::IEPS] = 1.0 / eps;
+  r[R::F32] = pack_f32(a, pr, az);
+#pragma unroll
+  for (int q = 0; q <= R::IEPS; q += 4) st4(Rr + q, r[q], r[q + 1], r[q + 2], r[q + 3]);
   if constexpr (!std::is_same<T, double>::value) {
     // the same record in the viscosity precision (mixed mode), with the flux
     T *Rv = vrec + (int64_t)i * R::VSIZE;
 #pragma unroll
-    for (int q = 0; q <= R::IEPS; ++q) Rv[q] = (T)Rr[q];
+    for (int q = 0; q <= R::IEPS; ++q)
+      if (q != R::F32) Rv[q] = (T)r[q];
     double f[S][DIM];
-    node_flux<DIM, double>(u + 1, v, pr, Rr[R::H], f);
+    node_flux<DIM, double>(u + 1, v, pr, r[R::H], f);
 #pragma unroll
     for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -629,255 +811,311 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
 
 // ---------------------------------------------------------------------------
 // k_visc: Algorithm 1 step 1 -- d_ij (j > i, mirrored through the transpose
-// index), the flux differences w_ij and the indicator alpha_i
+// index), the flux differences w_ij and a_ij of the indicator
 // ---------------------------------------------------------------------------
+// node i of an edge, as the row loop keeps it
+template <int DIM, typename T> struct ViscNode {
+  T v[DIM], mo[DIM], p, a, az, ip, eta, H;
+  T f[DIM + 2][DIM], q[DIM];  // FP32: the flux and the entropy flux
+  long long bits[DIM + 2];  // the FP64 state (the identical-state test compares FP64 bits in either precision)
+  float2 f32;               // FP64: the FP32 pair of the record
+  unsigned char steady;
+  // FP64: from the first 16 values of a record
+  __device__ __forceinline__ void from_record(const double *r) {
+    using R = Rec<DIM>;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+      v[k] = r[R::V + k];
+      mo[k] = r[1 + k];
+    }
+    p = r[R::P];
+    a = r[R::A];
+    az = r[R::AZ];
+    ip = r[R::IP];
+    eta = r[R::ETA];
+    H = r[R::H];
+    f32 = unpack_f32(r[R::F32]);
+  }
+};
+
+// the first 16 values of a node's FP64 record (everything k_visc reads)
+template <int DIM> __device__ __forceinline__ void load_rec(const Work &w, int i, double *r) {
+  static_assert(Rec<DIM>::H < 16 && Rec<DIM>::SIZE % 4 == 0, "record layout");
+  const double *R = w.rec + (int64_t)i * Rec<DIM>::SIZE;
+#pragma unroll
+  for (int q = 0; q < 16; q += 4) ld4(R + q, r[q], r[q + 1], r[q + 2], r[q + 3]);
+}
+
 template <int DIM, typename T>
-__global__ void __launch_bounds__(TPB_MAX) k_visc(MeshView m, Params p, Work w) {
+__device__ __forceinline__ ViscNode<DIM, T> visc_node(const Work &w, int i) {
   constexpr int S = DIM + 2;
   using R = Rec<DIM>;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.n || w.st->err) return;
-  const T *rec = (const T *)w.vrec;
-  const T *cij = (const T *)m.vcij;
-  const T *cn = (const T *)m.vcn;
-  const T *cinv = (const T *)m.vcinv;
-  constexpr bool packed = EdgeLayout<DIM, T>::packed;
-  constexpr int RS = vrec_stride<DIM, T>();
-  const T *Ri = rec + (int64_t)i * RS;
-  T vi[DIM], mi[DIM];
+  ViscNode<DIM, T> n;
+  if constexpr (sizeof(T) == 4) {
+    const T *Ri = (const T *)w.vrec + (int64_t)i * vrec_stride<DIM, T>();
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) {
-    vi[k] = Ri[R::V + k];
-    mi[k] = Ri[1 + k];
-  }
-  const T pi = Ri[R::P], ai = Ri[R::A], azi = Ri[R::AZ], ipi = Ri[R::IP], etai = Ri[R::ETA], Hi = Ri[R::H];
-  // FP64: w_ij from v.c_ij of both nodes (fewest FP64 operations). FP32: as
-  // differences of the two nodes' fluxes (rounded from FP64 by k_prep), then
-  // dotted with c_ij -- products taken per entry in FP32 (m_i (v_i.c_ij), or
-  // the flux formed in FP32) carry rounding errors that the difference of
-  // rounded fluxes does not: they left ~20x more of the limiter's l = 1
-  // checks failing on the Mach-3 cylinder and raised the error against FP64
-  constexpr bool flux_diff = sizeof(T) == 4;
-  T fi[DIM + 2][DIM], qi[DIM];
-  if constexpr (flux_diff) {
+    for (int k = 0; k < DIM; ++k) {
+      n.v[k] = Ri[R::V + k];
+      n.mo[k] = Ri[1 + k];
+    }
+    n.p = Ri[R::P];
+    n.a = Ri[R::A];
+    n.az = Ri[R::AZ];
+    n.ip = Ri[R::IP];
+    n.eta = Ri[R::ETA];
+    n.H = Ri[R::H];
 #pragma unroll
     for (int s = 0; s < S; ++s)
 #pragma unroll
-      for (int q = 0; q < DIM; ++q) fi[s][q] = Ri[R::F + s * DIM + q];
+      for (int q = 0; q < DIM; ++q) n.f[s][q] = Ri[R::F + s * DIM + q];
 #pragma unroll
-    for (int q = 0; q < DIM; ++q) qi[q] = vi[q] * etai;
+    for (int q = 0; q < DIM; ++q) n.q[q] = n.v[q] * n.eta;
+    double u[S];
+    load_rec_state<DIM>(w.rec + (int64_t)i * R::SIZE, u);
+#pragma unroll
+    for (int s = 0; s < S; ++s) n.bits[s] = dbits(u[s]);
+  } else {
+    double r[16];
+    load_rec<DIM>(w, i, r);
+    n.from_record(r);
+#pragma unroll
+    for (int s = 0; s < S; ++s) n.bits[s] = dbits(r[s]);
   }
-  const bool bi = m.isb[i] != 0;
-  // the FP64 state of node i as bit patterns (the identical-state test below
-  // compares FP64 bits in either precision)
-  long long ubi[S];
-  {
-    const double *Ri64 = w.rec + (int64_t)i * R::SIZE;
-#pragma unroll
-    for (int s = 0; s < S; ++s) ubi[s] = dbits(Ri64[s]);
+  n.steady = w.steady[i];
+  return n;
+}
+
+// the edge values of entry k = (i, j), j > i, and its mirror. BOTH: i and j
+// are boundary nodes (c_ji != -c_ij, Sec. 3.1: both directions evaluated).
+// FP64: w_ij from v.c_ij of both nodes (fewest FP64 operations). FP32: as
+// differences of the two nodes' fluxes (rounded from FP64 by k_prep), then
+// dotted with c_ij -- products taken per entry in FP32 (m_i (v_i.c_ij), or
+// the flux formed in FP32) carry rounding errors that the difference of
+// rounded fluxes does not: they left ~20x more of the limiter's l = 1
+// checks failing on the Mach-3 cylinder and raised the error against FP64
+template <int DIM, typename T, bool BOTH>
+__device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, const Work &w, const ViscNode<DIM, T> &n,
+                                          int i, int j, int64_t k) {
+  constexpr int S = DIM + 2;
+  using R = Rec<DIM>;
+  constexpr bool flux_diff = sizeof(T) == 4;
+  if (n.steady & 1) {
+    // both states unchanged since the previous k_visc, which stored this
+    // edge's values from the same bits; they were equal then (one of the
+    // two nodes had no differing neighbour), so they are now: nothing to
+    // store and no rough mark to set
+    const unsigned char stj = w.steady[j];
+    if ((stj & 1) && ((n.steady | stj) & 2)) return;
   }
-  const unsigned char sti = w.steady[i];
-  const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
-  for (int64_t k = k0; k < k1; ++k) {
-    const int j = m.col[k];
-    if (j <= i) continue;  // each unique edge once, from the row of min(i, j)
-    if (sti & 1) {
-      // both states unchanged since the previous k_visc, which stored this
-      // edge's values from the same bits; they were equal then (one of the
-      // two nodes had no differing neighbour), so they are now: nothing to
-      // store and no rough mark to set
-      const unsigned char stj = w.steady[j];
-      if ((stj & 1) && ((sti | stj) & 2)) continue;
+  const int32_t kt = m.tr[k];
+  T c[DIM], cn, ci, ct[DIM], cnt = T(0), cit = T(0);  // c_ij, and (BOTH) c_ji
+  load_geo<DIM, T>(m, k, c, cn, ci);
+  if constexpr (BOTH) load_geo<DIM, T>(m, kt, ct, cnt, cit);
+  double r[16];
+  bool same = true;
+  if constexpr (flux_diff) {
+    load_rec_state<DIM>(w.rec + (int64_t)j * R::SIZE, r);
+  } else {
+    load_rec<DIM>(w, j, r);
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s) same &= dbits(r[s]) == n.bits[s];
+  if (same) {
+    // U_j = U_i bit for bit: the flux and entropy-flux differences vanish,
+    // w_ij = a_ij = 0 exactly, and the two-rarefaction bound of Sec. 3.1
+    // reduces to lambda_max = |v.n_ij| + a (p_tr = p, both outer waves
+    // rarefactions), so d_ij = |v.c_ij| + a |c_ij| with no division, power
+    // or root. Any other edge marks both of its nodes rough.
+    T vc = T(0);
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) vc += n.v[q] * c[q];
+    T dij = abs_bits(vc) + n.a * cn;
+    if constexpr (BOTH) {  // the max over both directions
+      T vct = T(0);
+#pragma unroll
+      for (int q = 0; q < DIM; ++q) vct += n.v[q] * ct[q];
+      dij = max_nonneg(dij, abs_bits(vct) + n.a * cnt);
     }
-    const T *Rj = rec + (int64_t)j * RS;
-    const int32_t kt = m.tr[k];
-    {
-      // U_j = U_i bit for bit: the flux and entropy-flux differences vanish,
-      // w_ij = a_ij = 0 exactly, and the two-rarefaction bound of Sec. 3.1
-      // reduces to lambda_max = |v.n_ij| + a (p_tr = p, both outer waves
-      // rarefactions), so d_ij = |v.c_ij| + a |c_ij| with no division, power
-      // or root. Any other edge marks both of its nodes rough.
-      const double *Rj64 = w.rec + (int64_t)j * R::SIZE;
-      bool same = true;
-#pragma unroll
-      for (int s = 0; s < S; ++s) same &= dbits(Rj64[s]) == ubi[s];
-      if (same) {
-        T vc = T(0);
-#pragma unroll
-        for (int q = 0; q < DIM; ++q) vc += vi[q] * cij[(int64_t)q * m.nnz + k];
-        T dij = abs_bits(vc) + ai * cn[k];
-        if (bi && m.isb[j]) {  // c_ji != -c_ij: the max over both directions
-          T vct = T(0);
-#pragma unroll
-          for (int q = 0; q < DIM; ++q) vct += vi[q] * cij[(int64_t)q * m.nnz + kt];
-          dij = max_nonneg(dij, abs_bits(vct) + ai * cn[kt]);
-        }
-        store_zero_edge<DIM, T>(w, k, dij);
-        store_zero_edge<DIM, T>(w, kt, dij);
-        continue;
-      }
-      w.rough[i] = 1;
-      w.rough[j] = 1;
-    }
-    T vj[DIM], mj[DIM], c[DIM];
-    const T pj = Rj[R::P], etaj = Rj[R::ETA], Hj = Rj[R::H];
+    store_zero_edge<DIM, T>(w, k, dij);
+    store_zero_edge<DIM, T>(w, kt, dij);
+    return;
+  }
+  w.rough[i] = 1;
+  w.rough[j] = 1;
+  const T *Rj = (const T *)w.vrec + (int64_t)j * vrec_stride<DIM, T>();  // FP32 only
+  T vj[DIM], mj[DIM], pj, etaj, Hj, aj, azj, ipj;
+  float2 fj;
+  if constexpr (flux_diff) {
+    pj = Rj[R::P];
+    etaj = Rj[R::ETA];
+    Hj = Rj[R::H];
+    aj = Rj[R::A];
+    azj = Rj[R::AZ];
+    ipj = Rj[R::IP];
 #pragma unroll
     for (int q = 0; q < DIM; ++q) {
       vj[q] = Rj[R::V + q];
       mj[q] = Rj[1 + q];
-      c[q] = cij[(int64_t)q * m.nnz + k];
     }
-    // w_ij = (f(U_j) - f(U_i)) c_ij with f = (m, m v^T + p I, v (E + p));
-    // a_ij = (q_j - q_i) . c_ij with q = eta v
-    T vjc = T(0), vic = T(0);
+  } else {
+    ViscNode<DIM, T> nj;
+    nj.from_record(r);
+    pj = nj.p;
+    etaj = nj.eta;
+    Hj = nj.H;
+    aj = nj.a;
+    azj = nj.az;
+    ipj = nj.ip;
+    fj = nj.f32;
 #pragma unroll
     for (int q = 0; q < DIM; ++q) {
-      vjc += vj[q] * c[q];
-      vic += vi[q] * c[q];
+      vj[q] = nj.v[q];
+      mj[q] = nj.mo[q];
     }
-    const T dp = pj - pi;
-    T wv[S], a_ = T(0), dm[DIM];
+  }
+  // w_ij = (f(U_j) - f(U_i)) c_ij with f = (m, m v^T + p I, v (E + p));
+  // a_ij = (q_j - q_i) . c_ij with q = eta v
+  T vjc = T(0), vic = T(0);
+#pragma unroll
+  for (int q = 0; q < DIM; ++q) {
+    vjc += vj[q] * c[q];
+    vic += n.v[q] * c[q];
+  }
+  const T dp = pj - n.p;
+  T wv[S], a_ = T(0), dm[DIM];
+  if constexpr (flux_diff) {
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      T acc = T(0);
+#pragma unroll
+      for (int q = 0; q < DIM; ++q) acc += (Rj[R::F + s * DIM + q] - n.f[s][q]) * c[q];
+      wv[s] = acc;
+    }
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) a_ += __fsub_rn(__fmul_rn(vj[q], etaj), n.q[q]) * c[q];
+  } else {
+    // X_j (v_j.c) - X_i (v_i.c) as (X_j - X_i) (v_j.c) + X_i (v_j.c - v_i.c):
+    // exactly 0 when the two states are equal (a contracted X_j v_j.c -
+    // X_i v_i.c leaves the rounding error of one product), so that uniform
+    // regions keep P_ij = 0 and the limiter's cheapest exit
+    T w0 = T(0);
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) {
+      dm[q] = mj[q] - n.mo[q];
+      w0 += dm[q] * c[q];
+    }
+    const T dv = vjc - vic;
+    wv[0] = w0;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) wv[1 + a] = dm[a] * vjc + n.mo[a] * dv + dp * c[a];
+    wv[S - 1] = __fma_rn(Hj - n.H, vjc, __dmul_rn(n.H, dv));
+    a_ = __fma_rn(etaj - n.eta, vjc, __dmul_rn(n.eta, dv));
+  }
+  // the transposed entry: c_ji = -c_ij unless both nodes lie on the boundary
+  // (Sec. 3.1), so w_ji = w_ij and a_ji = a_ij; otherwise evaluate with c_ji
+  T wt[S], at = a_, vjct = T(0), vict = T(0);
+  if constexpr (!BOTH) {
+#pragma unroll
+    for (int s = 0; s < S; ++s) wt[s] = wv[s];
+  } else {
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) {
+      vjct += vj[q] * ct[q];
+      vict += n.v[q] * ct[q];
+    }
     if constexpr (flux_diff) {
+      at = T(0);
 #pragma unroll
       for (int s = 0; s < S; ++s) {
         T acc = T(0);
 #pragma unroll
-        for (int q = 0; q < DIM; ++q) acc += (Rj[R::F + s * DIM + q] - fi[s][q]) * c[q];
-        wv[s] = acc;
+        for (int q = 0; q < DIM; ++q) acc += (n.f[s][q] - Rj[R::F + s * DIM + q]) * ct[q];
+        wt[s] = acc;
       }
-      T qj[DIM];
 #pragma unroll
-      for (int q = 0; q < DIM; ++q) qj[q] = vj[q] * etaj;
-#pragma unroll
-      for (int q = 0; q < DIM; ++q) a_ += (qj[q] - qi[q]) * c[q];
+      for (int q = 0; q < DIM; ++q) at += __fsub_rn(n.q[q], __fmul_rn(vj[q], etaj)) * ct[q];
     } else {
-      // X_j (v_j.c) - X_i (v_i.c) as (X_j - X_i) (v_j.c) + X_i (v_j.c - v_i.c):
-      // exactly 0 when the two states are equal (a contracted X_j v_j.c -
-      // X_i v_i.c leaves the rounding error of one product), so that uniform
-      // regions keep P_ij = 0 and the limiter's cheapest exit
-      T w0 = T(0);
+      // (f_i - f_j) . c_ji = -[(f_j . c_ji) - (f_i . c_ji)], in the form above
+      T w0t = T(0);
+#pragma unroll
+      for (int q = 0; q < DIM; ++q) w0t += dm[q] * ct[q];
+      const T dvt = vjct - vict;
+      wt[0] = -w0t;
+#pragma unroll
+      for (int a = 0; a < DIM; ++a) wt[1 + a] = -(dm[a] * vjct + n.mo[a] * dvt + dp * ct[a]);
+      wt[S - 1] = -__fma_rn(Hj - n.H, vjct, __dmul_rn(n.H, dvt));
+      at = -__fma_rn(etaj - n.eta, vjct, __dmul_rn(n.eta, dvt));
+    }
+  }
+  // d_ij (Sec. 3.1), mirrored; normal velocities v . c_ij / |c_ij| (FP32:
+  // v . (c_ij / |c_ij|))
+  T dij;
+  if constexpr (flux_diff) {
+    T unl = T(0), unr = T(0);
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) {
+      unl += n.v[q] * (c[q] * ci);
+      unr += vj[q] * (c[q] * ci);
+    }
+    dij = lambda_max<T>(p, unl, n.p, n.a, n.az, n.ip, unr, pj, aj, azj, ipj) * cn;
+    if constexpr (BOTH) {
+      T unj = T(0), uni = T(0);
 #pragma unroll
       for (int q = 0; q < DIM; ++q) {
-        dm[q] = mj[q] - mi[q];
-        w0 += dm[q] * c[q];
+        T nq = ct[q] * cit;
+        unj += vj[q] * nq;
+        uni += n.v[q] * nq;
       }
-      const T dv = vjc - vic;
-      wv[0] = w0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) wv[1 + a] = dm[a] * vjc + mi[a] * dv + dp * c[a];
-      wv[S - 1] = (Hj - Hi) * vjc + Hi * dv;
-      a_ = (etaj - etai) * vjc + etai * dv;
-    }
-    const bool both = bi && m.isb[j];
-    // the transposed entry: c_ji = -c_ij unless both nodes lie on the boundary
-    // (Sec. 3.1), so w_ji = w_ij and a_ji = a_ij; otherwise evaluate with c_ji.
-    // Packed slots are stored whole once d_ij is known; otherwise each value
-    // is stored as soon as it is computed (fewer live registers).
-    // FP64 3D slots are two sectors: [w0..w3] stored at once, [w4, a, d, 0]
-    // once d_ij is known
-    constexpr bool two_sectors = packed && sizeof(T) == 8;
-    T wt[S], at = a_, vjct = T(0), vict = T(0);
-    if constexpr (!packed) {
-      T *wk = w_slot<DIM, T>(w, k);
-#pragma unroll
-      for (int s = 0; s < S; ++s) wk[s] = wv[s];
-      *a_ptr<DIM, T>(w, k) = a_;
-    } else if constexpr (two_sectors) {
-      store_sector((double *)w_slot<DIM, T>(w, k), wv[0], wv[1], wv[2], wv[3]);
-    }
-    if (!both) {
-#pragma unroll
-      for (int s = 0; s < S; ++s) wt[s] = wv[s];
-    } else {
-      T ct[DIM];
-#pragma unroll
-      for (int q = 0; q < DIM; ++q) ct[q] = cij[(int64_t)q * m.nnz + kt];
-#pragma unroll
-      for (int q = 0; q < DIM; ++q) {
-        vjct += vj[q] * ct[q];
-        vict += vi[q] * ct[q];
-      }
-      if constexpr (flux_diff) {
-        at = T(0);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          T acc = T(0);
-#pragma unroll
-          for (int q = 0; q < DIM; ++q) acc += (fi[s][q] - Rj[R::F + s * DIM + q]) * ct[q];
-          wt[s] = acc;
-        }
-#pragma unroll
-        for (int q = 0; q < DIM; ++q) at += (qi[q] - vj[q] * etaj) * ct[q];  // q_j as above
-      } else {
-        // (f_i - f_j) . c_ji = -[(f_j . c_ji) - (f_i . c_ji)], in the form above
-        T w0t = T(0);
-#pragma unroll
-        for (int q = 0; q < DIM; ++q) w0t += dm[q] * ct[q];
-        const T dvt = vjct - vict;
-        wt[0] = -w0t;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) wt[1 + a] = -(dm[a] * vjct + mi[a] * dvt + dp * ct[a]);
-        wt[S - 1] = -((Hj - Hi) * vjct + Hi * dvt);
-        at = -((etaj - etai) * vjct + etai * dvt);
-      }
-    }
-    if constexpr (!packed) {
-      T *wtk = w_slot<DIM, T>(w, kt);
-#pragma unroll
-      for (int s = 0; s < S; ++s) wtk[s] = wt[s];
-      *a_ptr<DIM, T>(w, kt) = at;
-    } else if constexpr (two_sectors) {
-      store_sector((double *)w_slot<DIM, T>(w, kt), wt[0], wt[1], wt[2], wt[3]);
-    }
-    // d_ij (Sec. 3.1), mirrored; normal velocities v . c_ij / |c_ij| (FP32:
-    // v . (c_ij / |c_ij|))
-    const T ci = cinv[k];
-    T unl = vic * ci, unr = vjc * ci;
-    if constexpr (flux_diff) {
-      unl = unr = T(0);
-#pragma unroll
-      for (int q = 0; q < DIM; ++q) {
-        unl += vi[q] * (c[q] * ci);
-        unr += vj[q] * (c[q] * ci);
-      }
-    }
-    T dij = lambda_max<T>(p, unl, pi, ai, azi, ipi, unr, pj, Rj[R::A], Rj[R::AZ], Rj[R::IP]) * cn[k];
-    if (both) {
-      const T cit = cinv[kt];
-      T unj = vjct * cit, uni = vict * cit;
-      if constexpr (flux_diff) {
-        unj = uni = T(0);
-#pragma unroll
-        for (int q = 0; q < DIM; ++q) {
-          T nq = cij[(int64_t)q * m.nnz + kt] * cit;
-          unj += vj[q] * nq;
-          uni += vi[q] * nq;
-        }
-      }
-      T dji = lambda_max<T>(p, unj, pj, Rj[R::A], Rj[R::AZ], Rj[R::IP], uni, pi, ai, azi, ipi) * cn[kt];
+      T dji = lambda_max<T>(p, unj, pj, aj, azj, ipj, uni, n.p, n.a, n.az, n.ip) * cnt;
       dij = max_nonneg(dij, dji);
     }
-    if constexpr (two_sectors) {
-      // values 4..7 of [w (S), a, d, 0...]
-      double hi[4] = {0.0, 0.0, 0.0, 0.0}, hit[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-      for (int s = 4; s < S; ++s) {
-        hi[s - 4] = wv[s];
-        hit[s - 4] = wt[s];
-      }
-      hi[S - 4] = a_;
-      hi[S - 3] = dij;
-      hit[S - 4] = at;
-      hit[S - 3] = dij;
-      store_sector((double *)w_slot<DIM, T>(w, k) + 4, hi[0], hi[1], hi[2], hi[3]);
-      store_sector((double *)w_slot<DIM, T>(w, kt) + 4, hit[0], hit[1], hit[2], hit[3]);
-    } else if constexpr (packed) {
-      store_slot<S>(w_slot<DIM, T>(w, k), wv, a_, dij);
-      store_slot<S>(w_slot<DIM, T>(w, kt), wt, at, dij);
-    } else {
-      *d_ptr<DIM, T>(w, k) = dij;
-      *d_ptr<DIM, T>(w, kt) = dij;
+  } else {
+    dij = lambda_max_sel(p, vic, vjc, ci, n.p, n.a, n.az, n.ip, n.f32, pj, aj, azj, ipj, fj) * cn;
+    if constexpr (BOTH) {
+      const T dji = lambda_max_sel(p, vjct, vict, cit, pj, aj, azj, ipj, fj, n.p, n.a, n.az, n.ip, n.f32) * cnt;
+      dij = max_nonneg(dij, dji);
     }
+  }
+  store_edge<DIM, T>(w, k, wv, a_, dij);
+  store_edge<DIM, T>(w, kt, wt, at, dij);
+}
+
+// Blocks [0, row_blocks): chunks of 32 rows, one row per lane, the entries of a
+// chunk dealt out to 2^lparts warps (entry q of a row to warp q mod 2^lparts),
+// so that on small meshes a row's edges run side by side: an FP64 instruction
+// occupies its warp for 63 cycles whatever else it could issue, and a few
+// thousand rows make too few warps with one thread per row. Every unique edge
+// is taken from the row of min(i, j); lanes of a warp work on the same entry
+// position, whose decisions agree between neighbouring rows. The remaining
+// blocks take the edges between two boundary nodes, one per thread, from a
+// list: in the row blocks a single such lane (a wall every few rows on small
+// meshes) would make its warp evaluate both directions (sweep of 256 small
+// cylinders: 238 -> 179 us with k_alpha).
+// Bound by FP64 issue: on a 998k-vertex cylinder, every edge general, 442 us
+// and 5.4M FP64 warp instructions (7.4M before lambda_max_sel) with the L1 at
+// 74 % of its throughput through 8-byte accesses, 358 us with 32-byte ones (FP64
+// pipe 80 % of the 84 % that it sustains); 493 us before both.
+template <int DIM, typename T>
+__global__ void __launch_bounds__(TPB_MAX) k_visc(MeshView m, Params p, Work w, unsigned row_blocks, int lparts) {
+  if (w.st->err) return;
+  if (blockIdx.x >= row_blocks) {
+    const int q = (blockIdx.x - row_blocks) * blockDim.x + threadIdx.x;
+    if (q >= m.n_bp) return;
+    const int i = m.bp_row[q], k = m.bp_pos[q];
+    const ViscNode<DIM, T> n = visc_node<DIM, T>(w, i);
+    visc_edge<DIM, T, true>(m, p, w, n, i, m.col[k], k);
+    return;
+  }
+  const unsigned warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int i = (warp >> lparts) * 32 + (threadIdx.x & 31);
+  if (i >= m.n) return;
+  const ViscNode<DIM, T> n = visc_node<DIM, T>(w, i);
+  const bool bi = m.isb[i] != 0;
+  const int64_t k1 = m.row_ptr[i + 1];
+  for (int64_t k = m.row_ptr[i] + (warp & ((1 << lparts) - 1)); k < k1; k += 1 << lparts) {
+    const int j = m.col[k];
+    if (j <= i || (bi && m.isb[j])) continue;
+    visc_edge<DIM, T, false>(m, p, w, n, i, j, k);
   }
 }
 
@@ -915,8 +1153,8 @@ __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w)
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   for (int64_t k = k0; k < k1; ++k) {
     if (m.col[k] == i) continue;
-    const T *wk = w_slot<DIM, T>(w, k);
-    const T a_ = *a_ptr<DIM, T>(w, k);
+    T wk[S], a_, d_;
+    load_edge<DIM, T>(w, k, wk, a_, d_);
     T b_ = T(0);
 #pragma unroll
     for (int s = 0; s < S; ++s) b_ += deta[s] * wk[s];
@@ -935,8 +1173,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
   using R = Rec<DIM>;
   const double *Ri = w.rec + (int64_t)i * R::SIZE;
   double ui[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) ui[s] = Ri[s];
+  load_rec_state<DIM>(Ri, ui);
   const double alphai = w.alpha[i];
 
   // U^L increment and the bounds in FP64; F^H in the viscosity precision T
@@ -963,9 +1200,11 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
       kd = k;
       continue;
     }
-    const double *Rj = w.rec + (int64_t)j * R::SIZE;
-    const T *wk = w_slot<DIM, T>(w, k);
-    const T dkT = *d_ptr<DIM, T>(w, k);
+    const double *Rj64 = w.rec + (int64_t)j * R::SIZE;
+    double Rj[S];
+    load_rec_state<DIM>(Rj64, Rj);
+    T wk[S], ak, dkT;
+    load_edge<DIM, T>(w, k, wk, ak, dkT);
     const double dk = (double)dkT;
     const T dH = T(alphai + w.alpha[j]) * dkT;  // w.alpha holds alpha / 2
     const double w0 = (double)wk[0];
@@ -991,7 +1230,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
       }
     }
     // Phi > 0: the integer order of the bit patterns is the numeric order
-    const long long pj = __double_as_longlong(Rj[R::PHI]), pm = __double_as_longlong(phimin);
+    const long long pj = __double_as_longlong(Rj64[R::PHI]), pm = __double_as_longlong(phimin);
     phimin = __longlong_as_double(pj < pm ? pj : pm);
     dsum += dk;
   }
@@ -1221,8 +1460,9 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
       if (longrow) w.la[k] = 1.0;
       continue;
     }
-    const double *Rj = w.rec + (int64_t)j * R::SIZE;
-    const double *Gj = Garr + (int64_t)j * SP;
+    double Rj[S], Gj[S];
+    load_rec_state<DIM>(w.rec + (int64_t)j * R::SIZE, Rj);
+    load_vec<DIM>(Garr + (int64_t)j * SP, Gj);
     const double dk = (double)*d_ptr<DIM, T>(w, k);
     const double dH = (alphai + w.alpha[j]) * dk;  // w.alpha holds alpha / 2
     const double cm = tc * m.betat[k], cd = coef * (dH - dk);
@@ -1230,8 +1470,8 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       P[s] = cm * (gi[s] - Gj[s]) + cd * (Rj[s] - ui[s]);
-      Pk[s] = P[s];
     }
+    store_vec<DIM>(Pk, P);
     if (P_trace) {
 #pragma unroll
       for (int s = 0; s < S; ++s) P_trace[k * SP + s] = P[s];
@@ -1318,9 +1558,7 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   const double lambda_i = m.lam[i];
   double u[S];
-  const double *Ui = Uin + (int64_t)i * SP;
-#pragma unroll
-  for (int s = 0; s < S; ++s) u[s] = Ui[s];
+  load_vec<DIM>(Uin + (int64_t)i * SP, u);
   const unsigned char *lone_in = w.lone + (int64_t)((slot - 1) & 1) * m.n;
   unsigned char *lone_out = w.lone + (int64_t)(slot & 1) * m.n;
   if (!w.rough2[i]) {  // every P_ij is 0 (see lim1_row): the state stays, every next search returns 1
@@ -1355,13 +1593,10 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
       const double r = w.rem[k];
       if (dbits(r) == 0) continue;  // nothing left of P_ij (rem stays 0)
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        P[s] = r * Pk[s];
-        Pk[s] = P[s];  // this pass's P_ij, for the remainder it leaves
-      }
+      for (int s = 0; s < S; ++s) P[s] = r * Pk[s];
+      store_vec<DIM>(Pk, P);  // this pass's P_ij, for the remainder it leaves
     } else {
-#pragma unroll
-      for (int s = 0; s < S; ++s) P[s] = Pk[s];
+      load_vec<DIM>(Pk, P);
     }
     // the update with l P; the remainder (1 - l) P is left as rem[k] (a
     // store of (1 - l) P here costs more than forming it where it is read,
@@ -1370,9 +1605,7 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     for (int s = 0; s < S; ++s) u[s] += lambda_i * l * P[s];
     w.rem[k] = 1.0 - l;
   }
-  double *Uo = Uout + (int64_t)i * SP;
-#pragma unroll
-  for (int s = 0; s < S; ++s) Uo[s] = u[s];
+  store_vec<DIM>(Uout + (int64_t)i * SP, u);
   const double *bi = w.bounds + (int64_t)i * 4;
   const double rmin = bi[0], rmax = bi[1], phimin = bi[2];
   const double phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
@@ -1716,9 +1949,7 @@ __device__ __forceinline__ void final_row(const MeshView &m, const Params &p, co
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   const double lambda_i = m.lam[i];
   double u[S];
-  const double *Ui = Uin + (int64_t)i * SP;
-#pragma unroll
-  for (int s = 0; s < S; ++s) u[s] = Ui[s];
+  load_vec<DIM>(Uin + (int64_t)i * SP, u);
   const unsigned char *lone = w.lone + (int64_t)((p.limiter_passes - 1) & 1) * m.n;  // of the last pass
   if (w.rough2[i] && p.limiter_passes >= 2) {
     // the remainder rem P that the last k_pass left: where rem = 0 (most
@@ -1873,7 +2104,14 @@ void launch_prep(const MeshView &m, const Params &p, const double *U, const Work
 }
 template <int DIM, typename T>
 void launch_visc(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {
-  k_visc<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
+  // warps a 32-row chunk, by the rows there are for the chip's 608 FP64 units:
+  // small meshes split the rows' chains (4k-vertex P1 vortex, k_visc + k_alpha
+  // 30.4 / 24.6 / 21.7 us with 1 / 2 / 4 warps; 62k cylinder 59.2 / 59.3 /
+  // 53.5), large ones read node i once (998k cylinder 552 / 565 / 642; between,
+  // 246k cylinder behind a shock 252 / 208 / 209, 375k in 3D 830 / 824 / 834)
+  const int lparts = m.n < 160 * 1024 ? 2 : m.n < 640 * 1024 ? 1 : 0;
+  const unsigned rows = nblocks((int64_t)nblocks(m.n, 32) << lparts, tpb / 32);
+  k_visc<DIM, T><<<rows + nblocks(m.n_bp, tpb), tpb, 0, s>>>(m, p, w, rows, lparts);
 }
 template <int DIM, typename T>
 void launch_alpha(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {

@@ -15,15 +15,13 @@ template <int DIM> struct Layout {
 };
 
 // Per-entry quantities of the viscosity kernel: w_ij (S values), a_ij, d_ij,
-// in precision T. FP64 2D: w_ij in a 4-value slot (one 32-byte sector), a_ij
-// and d_ij in arrays of their own. Otherwise (3D, and FP32 2D) one 8-value
-// slot [w_ij (S), a_ij, d_ij, 0...] per entry, so that the write of an edge
-// and its mirrored copy cover whole 32-byte sectors (partial slots and
-// separate a/d writes left partial sectors that the L2 completed from DRAM).
+// in precision T. FP64 2D: w_ij in a 4-value slot (one 32-byte sector) and
+// [a_ij, d_ij] in a pair of its own. Otherwise (3D, and FP32 2D) one 8-value
+// slot [w_ij (S), a_ij, d_ij, 0...] per entry. An edge and its mirrored copy
+// are written in whole sectors (or the pair in one access).
 template <int DIM, typename T> struct EdgeLayout {
   static constexpr bool packed = DIM == 3 || sizeof(T) == 4;
   static constexpr int SPW = packed ? 8 : 4;
-  static constexpr int A = DIM + 2;  // packed: slot index of a_ij
   static constexpr int D = DIM + 3;  // packed: slot index of d_ij
 };
 
@@ -39,7 +37,7 @@ template <int DIM> struct Rec {
   static constexpr int IP = 2 * DIM + 5;  // 1/p
   static constexpr int PHI = 2 * DIM + 6; // Phi = eps rho^-gamma
   static constexpr int ETA = 2 * DIM + 7; // eta = -rho s
-  static constexpr int EPS = 2 * DIM + 8; // internal energy eps
+  static constexpr int F32 = 2 * DIM + 8; // a and p as an FP32 pair (a = NaN: out of FP32's range), for lambda_max_sel
   static constexpr int H = 2 * DIM + 9;   // E + p
   static constexpr int IRHO = 2 * DIM + 10;  // 1/rho
   static constexpr int IEPS = 2 * DIM + 11;  // 1/eps
@@ -73,20 +71,17 @@ struct MeshView {
   const int64_t *row_ptr;
   const int32_t *col;
   const int32_t *tr;         // transpose position of every entry
-  const double *cij;         // [dim][nnz]
-  const double *cn;          // |c_ij|
-  const double *cinv;        // 1/|c_ij|
   const double *betat;       // m_ij / m_i (the consistent mass matrix is symmetric)
   const double *mi;
   const double *inv_mi;
   const double *relax;       // r_i (0 when the bounds are strict)
   const double *lam;         // lambda_i = 1 / (card I(i) - 1)
   const unsigned char *isb;  // 1 for boundary nodes
-  // arrays in the precision of the viscosity / flux part (double in FP64 mode,
-  // float in mixed mode): c_ij [dim][nnz], |c_ij|, 1/|c_ij|
-  const void *vcij;
-  const void *vcn;
-  const void *vcinv;
+  // in the precision of the viscosity / flux part (double in FP64 mode, float
+  // in mixed mode), four values an entry: 2D c_x, c_y, |c_ij|, 1/|c_ij|;
+  // 3D c_x, c_y, c_z, |c_ij|, with 1/|c_ij| in geo_inv (2D: not used)
+  const void *geo;
+  const void *geo_inv;
   const int32_t *bnd_index;  // per node: index into the boundary arrays, -1 inside
   const int32_t *bnd_node;   // [n_bnd] node of every boundary entry
   int n_nonreflecting;       // boundary nodes of the two non-reflecting kinds
@@ -94,6 +89,10 @@ struct MeshView {
   const double *bnd_normal;  // [dim][n_bnd]
   const double *bnd_state;   // [S][n_bnd]
   int n_bnd;
+  // the unique edges between two boundary nodes: row i and entry k = (i, j), j > i
+  int n_bp;
+  const int32_t *bp_row;
+  const int32_t *bp_pos;
   // independent instances (block-diagonal CSR): rows [inst_row_off[k], inst_row_off[k+1])
   int ninst;
   const int32_t *inst;          // instance of every row
@@ -108,6 +107,7 @@ struct Params {
   double inv_z;              // 2 gamma/(gamma-1)
   double kshock;             // (gamma+1)/(2 gamma)
   double inv_gm1;            // 1/(gamma - 1)
+  float gm1_f, inv_z_f, kshock_f;  // gamma - 1, inv_z and kshock rounded to FP32 (lambda_max_sel)
   int limiter_passes;        // 1 + the passes of k_pass (k_final reads rem when >= 2)
 };
 
@@ -132,7 +132,6 @@ struct Work {
   // gather of the transposed limiter for an entry between two such rows
   unsigned char *lone;    // [2][n]
   double *w;       // [nnz][SP]  (f(U_j) - f(U_i)) c_ij
-  double *d;       // [nnz]      d^L_ij (diagonal: d_ii)
   double *inc;     // [n][SP]    sum_{j != i} d_ij (U_j - U_i) - w_ij
   double *FH;      // [n][SP]    F^H_i / m_i
   double *bounds;  // [n][4]     rho_min, rho_max, Phi_min
@@ -159,8 +158,7 @@ struct Work {
   // float arrays in mixed mode)
   void *vrec;      // [n][Rec::SIZE] node record in that precision
   void *vw;        // [nnz][EdgeLayout::SPW] w_ij (and, packed, a_ij and d_ij)
-  void *vd;        // [nnz]      d_ij (not packed)
-  void *va;        // [nnz]      (q(U_j) - q(U_i)) . c_ij of the indicator (not packed)
+  void *vad;       // [nnz][2]   a_ij = (q(U_j) - q(U_i)) . c_ij of the indicator and d^L_ij (diagonal: d_ii; not packed)
   void *vFH;       // [n][SP]    F^H_i / m_i
   double *G64;     // [n][SP]    F^H_i / m_i in FP64 (mixed mode: the FP32 value widened once per node,
                    //            so that k_lim1 converts nothing per entry; FP64 mode: alias of FH)
@@ -186,7 +184,8 @@ constexpr int LSQ_SLOTS = 8;  // limiter passes per stage, at most
 
 // Launchers (all asynchronous on 'stream'). T is the precision of the
 // viscosity / high-order-flux part: double (FP64 mode) or float (mixed mode).
-// 'tpb' is the block size (threads = rows per block): 64, 128 or 256.
+// 'tpb' is the block size: 64, 128 or 256 threads, a thread per row (k_visc: a
+// lane per row, the row's entries dealt out to one, two or four warps).
 constexpr int TPB_MAX = 256;
 template <int DIM, typename T>
 void launch_prep(const MeshView &m, const Params &p, const double *U, const Work &w, int tpb, cudaStream_t s);
