@@ -42,6 +42,7 @@ struct eh_ctx {
          *trace_P = nullptr;
   DevStatus *st = nullptr;
   DevStatus *st_host = nullptr;  // pinned
+  unsigned long long *mesh_err = nullptr;  // error key of the mesh checks
   // host bookkeeping
   int64_t steps = 0;
   double last_dt = 0.0;
@@ -610,7 +611,9 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
     }
     c->own_stream = true;
   }
-  if (cudaMalloc(&c->st, sizeof(DevStatus)) != cudaSuccess ||
+  // (the mesh checks' error key sits behind the status)
+  static_assert(sizeof(DevStatus) % 8 == 0, "status alignment");
+  if (cudaMalloc(&c->st, sizeof(DevStatus) + sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost(&c->st_host, sizeof(DevStatus)) != cudaSuccess) {
     if (c->st) cudaFree(c->st);
     if (c->own_stream) cudaStreamDestroy(c->stream);
@@ -618,6 +621,7 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
     return EH_ERR_OOM;
   }
   cudaMemset(c->st, 0, sizeof(DevStatus));
+  c->mesh_err = (unsigned long long *)(c->st + 1);
   if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) c->nsm = 0;
   if (cfg->dim == 3) {
     // 3D: eh_autotune on a 6.0M-vertex extruded cylinder (after 100 steps
@@ -684,140 +688,139 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   free_mesh(c);
   const int dim = c->cfg.dim, S = S_of(c);
-  // ---- validation (host) ----
+  // ---- checks on the host: what the device's checks index by ----
   if (row_ptr[0] != 0 || row_ptr[n] != nnz) return fail(c, EH_ERR_BAD_MESH, "row_ptr must start at 0 and end at nnz");
-  for (int i = 0; i < n; ++i) {
+  for (int i = 0; i < n; ++i)
     if (row_ptr[i + 1] - row_ptr[i] < 2) return fail(c, EH_ERR_BAD_MESH, "row %d has fewer than 2 entries", i);
-    bool diag = false;
-    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-      if (col[k] < 0 || col[k] >= n) return fail(c, EH_ERR_BAD_MESH, "column out of range in row %d", i);
-      if (k > row_ptr[i] && col[k] <= col[k - 1]) return fail(c, EH_ERR_BAD_MESH, "row %d not sorted/unique", i);
-      if (col[k] == i) diag = true;
-    }
-    if (!diag) return fail(c, EH_ERR_BAD_MESH, "row %d has no diagonal entry", i);
-    if (!(mi[i] > 0.0)) return fail(c, EH_ERR_BAD_MESH, "m_%d <= 0", i);
-  }
-  std::vector<int32_t> tr(nnz);
-  for (int i = 0; i < n; ++i) {
-    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-      const int j = col[k];
-      const int32_t *b = col + row_ptr[j], *e = col + row_ptr[j + 1];
-      const int32_t *f = std::lower_bound(b, e, i);
-      if (f == e || *f != i) return fail(c, EH_ERR_BAD_MESH, "pattern not symmetric at (%d,%d)", i, j);
-      tr[k] = (int32_t)(row_ptr[j] + (f - b));
-    }
-  }
-  // c_ij, |c_ij|, 1/|c_ij| per entry in the viscosity precision (MeshView::geo)
-  std::vector<double> betat(nnz), geo64, ginv64;
-  std::vector<float> geo32, ginv32;
-  if (mixed(c)) geo32.resize(4 * (size_t)nnz); else geo64.resize(4 * (size_t)nnz);
-  if (dim == 3) {
-    if (mixed(c)) ginv32.resize(nnz); else ginv64.resize(nnz);
-  }
-  for (int i = 0; i < n; ++i) {
-    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
-      double s2 = 0.0;
-      for (int d = 0; d < dim; ++d) s2 += cij[(int64_t)d * nnz + k] * cij[(int64_t)d * nnz + k];
-      const double cn = std::sqrt(s2), cinv = cn > 0.0 ? 1.0 / cn : 0.0;
-      if (col[k] != i && !(cn > 0.0)) return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry");
-      double g[5];
-      for (int d = 0; d < dim; ++d) g[d] = cij[(int64_t)d * nnz + k];
-      g[dim] = cn;
-      g[dim + 1] = cinv;
-      for (int q = 0; q < 4; ++q) {
-        if (mixed(c)) geo32[4 * k + q] = (float)g[q]; else geo64[4 * k + q] = g[q];
-      }
-      if (dim == 3) {
-        if (mixed(c)) ginv32[k] = (float)cinv; else ginv64[k] = cinv;
-      }
-      // the consistent mass matrix is symmetric (m_ij = int phi_i phi_j);
-      // k_lim1 relies on it, with the mean of the two entries
-      const double a = mij[k], b = mij[tr[k]];
-      if (std::fabs(a - b) > 1e-12 * std::max(std::fabs(a), std::fabs(b)))
-        return fail(c, EH_ERR_BAD_MESH, "consistent mass not symmetric at (%d,%d)", i, col[k]);
-      betat[k] = 0.5 * (a + b) / mi[i];
-    }
-  }
-  std::vector<double> inv_mi(n), relax(n, 0.0), lam(n);
-  double area = 0.0;
-  for (int i = 0; i < n; ++i) area += mi[i];
-  for (int i = 0; i < n; ++i) {
-    inv_mi[i] = 1.0 / mi[i];
-    lam[i] = 1.0 / (double)(row_ptr[i + 1] - row_ptr[i] - 1);
-    if (c->cfg.bound_relaxation) relax[i] = std::pow(mi[i] / area, 1.5 / dim);
-  }
   std::vector<unsigned char> isb(n, 0);
-  std::vector<int32_t> bidx(n, -1);
+  int nonreflecting = 0;
   for (int b = 0; b < n_bnd; ++b) {
     const int i = bnd_node[b];
-    if (i < 0 || i >= n || bidx[i] >= 0) return fail(c, EH_ERR_BAD_MESH, "boundary node %d invalid or repeated", i);
+    if (i < 0 || i >= n || isb[i]) return fail(c, EH_ERR_BAD_MESH, "boundary node %d invalid or repeated", i);
     if (bnd_kind[b] < EH_BC_SLIP || bnd_kind[b] > EH_BC_GODUNOV)
       return fail(c, EH_ERR_BAD_MESH, "boundary kind %d invalid", bnd_kind[b]);
     if (bnd_kind[b] != EH_BC_SLIP && bnd_kind[b] != EH_BC_DO_NOTHING && !bnd_state)
       return fail(c, EH_ERR_BAD_MESH, "boundary kind %d needs a Dirichlet state", bnd_kind[b]);
+    if (bnd_kind[b] == EH_BC_CHARACTERISTIC || bnd_kind[b] == EH_BC_GODUNOV) ++nonreflecting;
     isb[i] = 1;
-    bidx[i] = b;
   }
-  std::vector<int32_t> bprow, bppos;  // edges between two boundary nodes, from the smaller one's row
+  // edges between two boundary nodes, from the smaller one's row (columns are
+  // not checked yet; a mesh with a bad one is rejected below)
+  std::vector<int32_t> bprow, bppos;
   for (int i = 0; i < n; ++i)
     if (isb[i])
       for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k)
-        if (col[k] > i && isb[col[k]]) {
+        if (col[k] > i && col[k] < n && isb[col[k]]) {
           bprow.push_back(i);
           bppos.push_back((int32_t)k);
         }
-  // ---- device arrays ----
+  std::vector<double> relax;
+  if (c->cfg.bound_relaxation) {
+    relax.resize(n);
+    double area = 0.0;
+    for (int i = 0; i < n; ++i) area += mi[i];
+    for (int i = 0; i < n; ++i) relax[i] = std::pow(mi[i] / area, 1.5 / dim);
+  }
+  // ---- device arrays; the remaining checks run on the device ----
   eh_status st;
-  if ((st = alloc_static(c, n, nnz, n_bnd, (int64_t)bprow.size())) != EH_OK) {
+  if ((st = alloc_static(c, n, nnz, n_bnd, (int64_t)bprow.size())) != EH_OK ||
+      (st = alloc_work(c, n, nnz)) != EH_OK) {
     free_mesh(c);
     return st;
   }
+  // the caller's c_ij and m_ij, needed until the static arrays are made from
+  // them: in work arrays where there are some
+  static_assert(Layout<2>::SP >= 2 && Layout<3>::SP >= 3, "c_ij fits P");
+  double *cij_d = c->wk.P, *mij_d = c->wk.rem;
+  void *tmp = nullptr;
+  if (c->static_only) {
+    if (cudaMalloc(&tmp, sizeof(double) * (size_t)(dim + 1) * nnz) != cudaSuccess) {
+      cudaGetLastError();
+      free_mesh(c);
+      return fail(c, EH_ERR_OOM, "cudaMalloc of %zu bytes", sizeof(double) * (size_t)(dim + 1) * nnz);
+    }
+    cij_d = (double *)tmp;
+    mij_d = cij_d + (size_t)dim * nnz;
+  }
   MeshView &m = c->mv;
-  auto up = [&](const void *dst, const void *src, size_t bytes) -> cudaError_t {
-    if (bytes == 0) return cudaSuccess;
-    return cudaMemcpy(const_cast<void *>(dst), src, bytes, cudaMemcpyHostToDevice);
-  };
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = up(m.row_ptr, row_ptr, sizeof(int64_t) * (n + 1));
-  if (e == cudaSuccess) e = up(m.col, col, sizeof(int32_t) * nnz);
-  if (e == cudaSuccess) e = up(m.tr, tr.data(), sizeof(int32_t) * nnz);
-  if (e == cudaSuccess) {
-    const size_t v = mixed(c) ? sizeof(float) : sizeof(double);
-    e = up(m.geo, mixed(c) ? (const void *)geo32.data() : (const void *)geo64.data(), 4 * v * nnz);
-    if (e == cudaSuccess && dim == 3)
-      e = up(m.geo_inv, mixed(c) ? (const void *)ginv32.data() : (const void *)ginv64.data(), v * nnz);
-  }
-  if (e == cudaSuccess) e = up(m.betat, betat.data(), sizeof(double) * nnz);
-  if (e == cudaSuccess) e = up(m.mi, mi, sizeof(double) * n);
-  if (e == cudaSuccess) e = up(m.inv_mi, inv_mi.data(), sizeof(double) * n);
-  if (e == cudaSuccess) e = up(m.relax, relax.data(), sizeof(double) * n);
-  if (e == cudaSuccess) e = up(m.lam, lam.data(), sizeof(double) * n);
-  if (e == cudaSuccess) e = up(m.isb, isb.data(), n);
-  if (e == cudaSuccess) e = up(m.bnd_index, bidx.data(), sizeof(int32_t) * n);
-  if (e == cudaSuccess) e = up(m.bnd_node, bnd_node, sizeof(int32_t) * n_bnd);
-  if (e == cudaSuccess) e = up(m.bnd_kind, bnd_kind, sizeof(int32_t) * n_bnd);
-  if (e == cudaSuccess) e = up(m.bnd_normal, bnd_normal, sizeof(double) * dim * n_bnd);
-  if (e == cudaSuccess && bnd_state) e = up(m.bnd_state, bnd_state, sizeof(double) * S * n_bnd);
-  if (e == cudaSuccess) e = up(m.bp_row, bprow.data(), sizeof(int32_t) * bprow.size());
-  if (e == cudaSuccess) e = up(m.bp_pos, bppos.data(), sizeof(int32_t) * bppos.size());
-  if (e != cudaSuccess) {
-    free_mesh(c);
-    return fail(c, EH_ERR_CUDA, "mesh upload: %s", cudaGetErrorString(e));
-  }
   m.n = n;
   m.nnz = nnz;
   m.n_bnd = n_bnd;
   m.n_bp = (int)bprow.size();
-  m.n_nonreflecting = 0;
-  for (int b = 0; b < n_bnd; ++b)
-    if (bnd_kind[b] == EH_BC_CHARACTERISTIC || bnd_kind[b] == EH_BC_GODUNOV) ++m.n_nonreflecting;
+  m.n_nonreflecting = nonreflecting;
+  cudaStream_t s = c->stream;
+  cudaError_t e = cudaSuccess;
+  auto up = [&](const void *dst, const void *src, size_t bytes) {
+    if (e == cudaSuccess && bytes > 0)
+      e = cudaMemcpyAsync(const_cast<void *>(dst), src, bytes, cudaMemcpyHostToDevice, s);
+  };
+  auto fill = [&](const void *dst, int value, size_t bytes) {
+    if (e == cudaSuccess && bytes > 0) e = cudaMemsetAsync(const_cast<void *>(dst), value, bytes, s);
+  };
+  unsigned long long key = ~0ull;
+  unsigned long long *err = c->mesh_err;
+  fill(err, 0xFF, sizeof(key));
+  fill(m.bnd_index, 0xFF, sizeof(int32_t) * n);
+  fill(m.isb, 0, n);
+  fill(m.relax, 0, sizeof(double) * n);
+  up(m.row_ptr, row_ptr, sizeof(int64_t) * (n + 1));
+  up(m.col, col, sizeof(int32_t) * nnz);
+  up(m.mi, mi, sizeof(double) * n);
+  if (e == cudaSuccess) {
+    launch_mesh_rows(m, const_cast<double *>(m.inv_mi), const_cast<double *>(m.lam), err, s);
+    launch_mesh_transpose(m, const_cast<int32_t *>(m.tr), err, s);
+    e = cudaGetLastError();
+  }
+  up(cij_d, cij, sizeof(double) * dim * nnz);
+  up(mij_d, mij, sizeof(double) * nnz);
+  if (e == cudaSuccess) {
+    double *betat = const_cast<double *>(m.betat);
+    void *geo = const_cast<void *>(m.geo), *ginv = const_cast<void *>(m.geo_inv);
+    if (dim == 2) {
+      if (mixed(c)) launch_mesh_entries<2, float>(m, cij_d, mij_d, (float *)geo, (float *)ginv, betat, err, s);
+      else launch_mesh_entries<2, double>(m, cij_d, mij_d, (double *)geo, (double *)ginv, betat, err, s);
+    } else {
+      if (mixed(c)) launch_mesh_entries<3, float>(m, cij_d, mij_d, (float *)geo, (float *)ginv, betat, err, s);
+      else launch_mesh_entries<3, double>(m, cij_d, mij_d, (double *)geo, (double *)ginv, betat, err, s);
+    }
+    e = cudaGetLastError();
+  }
+  up(m.bnd_node, bnd_node, sizeof(int32_t) * n_bnd);
+  up(m.bnd_kind, bnd_kind, sizeof(int32_t) * n_bnd);
+  up(m.bnd_normal, bnd_normal, sizeof(double) * dim * n_bnd);
+  if (bnd_state) up(m.bnd_state, bnd_state, sizeof(double) * S * n_bnd);
+  if (!relax.empty()) up(m.relax, relax.data(), sizeof(double) * n);
+  up(m.bp_row, bprow.data(), sizeof(int32_t) * bprow.size());
+  up(m.bp_pos, bppos.data(), sizeof(int32_t) * bppos.size());
+  if (e == cudaSuccess) {
+    launch_mesh_boundary(m, const_cast<int32_t *>(m.bnd_index), const_cast<unsigned char *>(m.isb), s);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&key, err, sizeof(key), cudaMemcpyDeviceToHost, s);
+  const cudaError_t es = cudaStreamSynchronize(s);  // also before the temporary and the host vectors go
+  if (e == cudaSuccess) e = es;
+  if (tmp) cudaFree(tmp);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    free_mesh(c);
+    return fail(c, EH_ERR_CUDA, "mesh upload: %s", cudaGetErrorString(e));
+  }
+  if (key != ~0ull) {
+    free_mesh(c);
+    const int row = (int)((key >> 16) & 0xFFFFFFFFu);
+    switch (key & 0xFFFF) {
+      case MESH_ERR_COL: return fail(c, EH_ERR_BAD_MESH, "column out of range in row %d", row);
+      case MESH_ERR_ORDER: return fail(c, EH_ERR_BAD_MESH, "row %d not sorted/unique", row);
+      case MESH_ERR_DIAG: return fail(c, EH_ERR_BAD_MESH, "row %d has no diagonal entry", row);
+      case MESH_ERR_MASS: return fail(c, EH_ERR_BAD_MESH, "m_%d <= 0", row);
+      case MESH_ERR_PATTERN: return fail(c, EH_ERR_BAD_MESH, "pattern not symmetric in row %d", row);
+      case MESH_ERR_CIJ: return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry of row %d", row);
+      default: return fail(c, EH_ERR_BAD_MESH, "consistent mass not symmetric in row %d", row);
+    }
+  }
   c->n = n;
   c->nnz = nnz;
   c->n_bnd = n_bnd;
-  if ((st = alloc_work(c, n, nnz)) != EH_OK) {
-    free_mesh(c);
-    return st;
-  }
   const int64_t one[2] = {0, (int64_t)n};
   if ((st = setup_instances(c, 1, one, nullptr)) != EH_OK) {
     free_mesh(c);

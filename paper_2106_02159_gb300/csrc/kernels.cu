@@ -2225,6 +2225,112 @@ template <int DIM> void launch_count_not_admissible(int n, const double *U, DevS
   k_count_not_admissible<DIM><<<nblocks(n, 256), 256, 0, s>>>(n, U, st);
 }
 
+// ---------------------------------------------------------------------------
+// the mesh's checks and static arrays (eh_upload_mesh), one thread per row; on
+// the host, one pass each over the entries for the checks, the transpose (a
+// binary search an entry) and the norms took most of an upload (998k vertices,
+// 9.0M entries: 104 ms; here 8.5 ms, bound by the copies of the caller's arrays)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void mesh_error(unsigned long long *err, int phase, int row, int code) {
+  atomicMin(err, (unsigned long long)phase << 56 | (unsigned long long)(unsigned)row << 16 | (unsigned)code);
+}
+__device__ __forceinline__ bool mesh_failed(const unsigned long long *err) { return *err != ~0ull; }
+
+__global__ void k_mesh_rows(MeshView m, double *inv_mi, double *lam, unsigned long long *err) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m.n) return;
+  const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
+  bool diag = false;
+  int prev = -1, code = 0;
+  for (int64_t k = k0; k < k1 && !code; ++k) {
+    const int c = m.col[k];
+    if (c < 0 || c >= m.n) code = MESH_ERR_COL;
+    else if (k > k0 && c <= prev) code = MESH_ERR_ORDER;
+    if (c == i) diag = true;
+    prev = c;
+  }
+  if (!code && !diag) code = MESH_ERR_DIAG;
+  if (!code && !(m.mi[i] > 0.0)) code = MESH_ERR_MASS;
+  if (code) mesh_error(err, 0, i, code);
+  inv_mi[i] = 1.0 / m.mi[i];
+  lam[i] = 1.0 / (double)(k1 - k0 - 1);
+}
+
+__global__ void k_mesh_transpose(MeshView m, int32_t *tr, unsigned long long *err) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m.n || mesh_failed(err)) return;
+  for (int64_t k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
+    const int j = m.col[k];
+    int64_t lo = m.row_ptr[j], hi = m.row_ptr[j + 1];
+    const int64_t end = hi;
+    while (lo < hi) {  // the first entry of row j that is >= i
+      const int64_t mid = lo + (hi - lo) / 2;
+      if (m.col[mid] < i) lo = mid + 1; else hi = mid;
+    }
+    if (lo == end || m.col[lo] != i) {
+      mesh_error(err, 1, i, MESH_ERR_PATTERN);
+      return;
+    }
+    tr[k] = (int32_t)lo;
+  }
+}
+
+template <int DIM, typename T>
+__global__ void k_mesh_entries(MeshView m, const double *cij, const double *mij, T *geo, T *geo_inv, double *betat,
+                               unsigned long long *err) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= m.n) return;
+  // (an error of this phase leaves the other rows running: the smallest key counts)
+  if ((*(volatile unsigned long long *)err >> 56) < 2) return;
+  for (int64_t k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
+    double c[DIM], s2 = 0.0;
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) {
+      c[q] = cij[(int64_t)q * m.nnz + k];
+      s2 = __fma_rn(c[q], c[q], s2);
+    }
+    const double cn = sqrt(s2), ci = cn > 0.0 ? 1.0 / cn : 0.0;
+    if (m.col[k] != i && !(cn > 0.0)) {
+      mesh_error(err, 2, i, MESH_ERR_CIJ);
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) geo[4 * k + q] = (T)c[q];
+    geo[4 * k + DIM] = (T)cn;
+    if constexpr (DIM == 2) geo[4 * k + 3] = (T)ci; else geo_inv[k] = (T)ci;
+    // the consistent mass matrix is symmetric (m_ij = int phi_i phi_j);
+    // k_lim1 relies on it, with the mean of the two entries
+    const double a = mij[k], b = mij[m.tr[k]];
+    if (fabs(a - b) > 1e-12 * fmax(fabs(a), fabs(b))) {
+      mesh_error(err, 2, i, MESH_ERR_MIJ);
+      return;
+    }
+    betat[k] = 0.5 * (a + b) / m.mi[i];
+  }
+}
+
+__global__ void k_mesh_boundary(MeshView m, int32_t *bnd_index, unsigned char *isb) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= m.n_bnd) return;
+  bnd_index[m.bnd_node[b]] = b;
+  isb[m.bnd_node[b]] = 1;
+}
+
+void launch_mesh_rows(const MeshView &m, double *inv_mi, double *lam, unsigned long long *err, cudaStream_t s) {
+  k_mesh_rows<<<nblocks(m.n, 128), 128, 0, s>>>(m, inv_mi, lam, err);
+}
+void launch_mesh_transpose(const MeshView &m, int32_t *tr, unsigned long long *err, cudaStream_t s) {
+  k_mesh_transpose<<<nblocks(m.n, 128), 128, 0, s>>>(m, tr, err);
+}
+template <int DIM, typename T>
+void launch_mesh_entries(const MeshView &m, const double *cij, const double *mij, T *geo, T *geo_inv, double *betat,
+                         unsigned long long *err, cudaStream_t s) {
+  k_mesh_entries<DIM, T><<<nblocks(m.n, 128), 128, 0, s>>>(m, cij, mij, geo, geo_inv, betat, err);
+}
+void launch_mesh_boundary(const MeshView &m, int32_t *bnd_index, unsigned char *isb, cudaStream_t s) {
+  if (m.n_bnd > 0) k_mesh_boundary<<<nblocks(m.n_bnd, 256), 256, 0, s>>>(m, bnd_index, isb);
+}
+
 // dst[i] = src[i] + add (nonneg_only: only where src[i] >= 0; -1 entries
 // stay): the index arrays of one instance placed into a block-diagonal union
 template <typename I> __global__ void k_offset_copy(I *dst, const I *src, int64_t count, I add, int nonneg_only) {
@@ -2243,6 +2349,8 @@ template void launch_offset_copy<int32_t>(int32_t *, const int32_t *, int64_t, i
 template void launch_offset_copy<int64_t>(int64_t *, const int64_t *, int64_t, int64_t, bool, cudaStream_t);
 
 #define EH_INSTANTIATE_T(DIM, T)                                                                                     \
+  template void launch_mesh_entries<DIM, T>(const MeshView &, const double *, const double *, T *, T *, double *,      \
+                                            unsigned long long *, cudaStream_t);                                     \
   template void launch_prep<DIM, T>(const MeshView &, const Params &, const double *, const Work &, int, cudaStream_t); \
   template void launch_visc<DIM, T>(const MeshView &, const Params &, const Work &, int, cudaStream_t);               \
   template void launch_alpha<DIM, T>(const MeshView &, const Params &, const Work &, int, cudaStream_t);              \

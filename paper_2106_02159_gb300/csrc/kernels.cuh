@@ -229,6 +229,24 @@ constexpr int STAT_BLOCKS = 304;
 template <int DIM>
 void launch_state_stats(int n, const double *U, const double *mi, double *part, double *out, cudaStream_t s);
 
+// Mesh checks and static arrays of eh_upload_mesh, from the caller's arrays
+// copied to the device. *err (all-ones before) receives the smallest error
+// key found, row-major: phase << 56 | row << 16 | code (MESH_ERR_*); a kernel
+// whose predecessor found an error does nothing, so no index is used before it
+// is checked (row_ptr itself is checked by the caller).
+enum { MESH_ERR_COL = 1, MESH_ERR_ORDER = 2, MESH_ERR_DIAG = 3, MESH_ERR_MASS = 4, MESH_ERR_PATTERN = 5,
+       MESH_ERR_CIJ = 6, MESH_ERR_MIJ = 7 };
+// sorted unique columns in range, a diagonal, m_i > 0; 1/m_i and lambda_i
+void launch_mesh_rows(const MeshView &m, double *inv_mi, double *lam, unsigned long long *err, cudaStream_t s);
+// the transpose index
+void launch_mesh_transpose(const MeshView &m, int32_t *tr, unsigned long long *err, cudaStream_t s);
+// geo (and geo_inv) from c_ij [dim][nnz], m_ij/m_i from the symmetric m_ij
+template <int DIM, typename T>
+void launch_mesh_entries(const MeshView &m, const double *cij, const double *mij, T *geo, T *geo_inv, double *betat,
+                         unsigned long long *err, cudaStream_t s);
+// bnd_index (-1 before) and isb (0 before) of the boundary nodes
+void launch_mesh_boundary(const MeshView &m, int32_t *bnd_index, unsigned char *isb, cudaStream_t s);
+
 // dst[i] = src[i] + add over count entries (nonneg_only: negative entries
 // copied unchanged); int32_t and int64_t
 template <typename I>
