@@ -655,6 +655,7 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
   p.inv_z = 1.0 / p.z;
   p.kshock = (cfg->gamma + 1.0) / (2.0 * cfg->gamma);
   p.inv_gm1 = 1.0 / (cfg->gamma - 1.0);
+  p.gamma_f = (float)p.gamma;
   p.gm1_f = (float)p.gm1;
   p.inv_z_f = (float)p.inv_z;
   p.kshock_f = (float)p.kshock;

@@ -69,6 +69,18 @@ __device__ __forceinline__ double abs_bits(double x) {
 }
 __device__ __forceinline__ float abs_bits(float x) { return fabsf(x); }
 
+// x rounded towards zero to FP32 on the integer units (relative error 2^-23;
+// 0 below 2^-126, +-inf from 2^127 on and for NaN): an FP64 -> FP32 conversion
+// instruction takes part of an FP64 issue slot, this takes none
+__device__ __forceinline__ float trunc_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = (hi >> 20) & 0x7ffu, sg = hi & 0x80000000u;
+  unsigned r = ((__funnelshift_l(lo, hi, 3) - (384u << 23)) & 0x7fffffffu) | sg;
+  if (e < 897u) r = sg;
+  if (e > 1149u) r = sg | 0x7f800000u;
+  return __uint_as_float(r);
+}
+
 // 256-bit accesses (sm_100 on): a lane's 32-byte sector in one instruction.
 // Lanes of a row kernel read sectors of different lines (rows are 64 to 288
 // bytes apart), so L1 serves one lane's line at a time whatever the width:
@@ -267,18 +279,6 @@ __device__ __forceinline__ T lambda_max(const Params &p, T unl, T pl, T al, T az
   T lam1 = unl - al * sl;
   T lam3 = unr + ar * sr;
   return max_nonneg(pos_part(-lam1), pos_part(lam3));
-}
-
-// x rounded towards zero to FP32 on the integer units (relative error 2^-23;
-// 0 below 2^-126, +-inf from 2^127 on and for NaN): an FP64 -> FP32 conversion
-// instruction takes part of an FP64 issue slot, this takes none
-__device__ __forceinline__ float trunc_f32(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned e = (hi >> 20) & 0x7ffu, sg = hi & 0x80000000u;
-  unsigned r = ((__funnelshift_l(lo, hi, 3) - (384u << 23)) & 0x7fffffffu) | sg;
-  if (e < 897u) r = sg;
-  if (e > 1149u) r = sg | 0x7f800000u;
-  return __uint_as_float(r);
 }
 
 // a and p of a node as an FP32 pair in one FP64 slot of its record (Rec::F32),
@@ -557,54 +557,127 @@ __device__ double line_search_iterate(const Params &p, const double *ub, const d
   return lL;
 }
 
-// FP32 pre-decision of the entropy test at l = 1 (gamma = 7/5): with
-// u = ub + P, does (rho E - |m|^2/2)^5 >= Phi_min^5 rho^12 hold, for the FP64
-// inputs, in exact arithmetic? The FP32 evaluation carries error bounds built
-// from the inputs' magnitudes (every conversion and operation rounds by at most
-// 2^-24 relative): +1 = holds with a margin that covers them, -1 = fails with
-// such a margin, 0 = too close to call (or outside the range where the FP32
-// powers can neither overflow nor underflow). Every error term is
-// over-estimated by a third or more (3 units for a chain that rounds twice, 8
-// and 16 for chains of 3 and 6 roundings, B scaled by 1.01), so a decided
-// outcome holds with a relative margin of at least ~1e-7 -- far beyond the
-// FP64 test's own rounding (~1e-15): it is the outcome the FP64 test reaches,
-// and the FP64 test runs only where this returns 0.
+// ---------------------------------------------------------------------------
+// Pre-decision of the entropy test at l = 1: with u = ub + P, does
+// rho E - |m|^2/2 >= Phi_min rho^(gamma+1) hold (gamma = 7/5: fifth powers of
+// both sides), for the FP64 inputs, in exact arithmetic? +1: it holds, -1: it
+// fails, each with a margin far beyond the FP64 test's own rounding (~1e-15),
+// so that it is the outcome the FP64 test reaches; 0: too close to call, or
+// outside the range of the FP32 powers. Two levels, both on the FP32 units (76
+// instructions for one FP64 issue slot), where the FP64 test takes 17 slots
+// and a warp with one open lane pays for all:
+//  - FP32 with error bounds built from the inputs' magnitudes (relative margin
+//    ~1e-5 at Mach 3);
+//  - gamma = 7/5: pairs of FP32 values (48 bits; margin ~1e-12), which leave
+//    the FP64 test to states that agree to their last bits.
+// ---------------------------------------------------------------------------
 struct RowF32 {
-  float u[5];   // ub rounded to FP32
-  float phi5;   // Phi_min^5 rounded to FP32 (0 when out of range)
+  float u[5];  // ub truncated to FP32
+  float phi;   // Phi_min^5 (gamma = 7/5) or Phi_min, truncated; 0: no pre-decision for the row
 };
-// The row's FP32 data of the pre-decision. Rows whose density bounds are
-// within 1e-6 of each other (near-uniform neighbourhoods) skip it: there psi(1)
-// sits within the FP32 error of 0 almost always (on the Mach-3 cylinder most
-// such rows differ from their neighbours by a few ulps, and psi(1) is within
-// 1e-13 of 0), and a warp with one undecided lane pays for both tests.
+// The row's FP32 data. Rows whose density bounds, or whose smallest and largest
+// Phi over the stencil, agree to 2^17 ulps (3e-11) skip the pre-decision: their
+// states differ from their neighbours' by rounding (on the Mach-3 cylinder most
+// such rows by a few ulps, psi(1) within 1e-13 of 0), or the flow is isentropic
+// there and psi(1) is rounding (a vortex in a uniform stream).
 template <int DIM>
-__device__ __forceinline__ RowF32 row_f32(const double *ub, double rmin, double rmax, double phimin5) {
+__device__ __forceinline__ RowF32 row_f32(const Params &p, const double *ub, double rmin, double rmax, double phimin,
+                                          double phimax, double phimin5) {
   RowF32 r;
 #pragma unroll
   for (int s = 0; s < DIM + 2; ++s) r.u[s] = 0.0f;
-  r.phi5 = 0.0f;
-  // 2^-40 <= Phi_min^5 <= 2^40 (else no pre-decision)
-  if (!(gt_pos(rmax - rmin, 1e-6 * rmax) && gt_pos(phimin5, 9.094947017729282e-13) &&
-        lt_pos(phimin5, 1.099511627776e12)))
+  r.phi = 0.0f;
+  // 2^-40 <= Phi_min^5 <= 2^40 (gamma != 7/5: Phi_min itself)
+  const double ph = p.gamma75 ? phimin5 : phimin;
+  if (!(dbits(rmax) - dbits(rmin) > 1 << 17 && dbits(phimax) - dbits(phimin) > 1 << 17 &&
+        gt_pos(ph, 9.094947017729282e-13) && lt_pos(ph, 1.099511627776e12)))
     return r;
 #pragma unroll
-  for (int s = 0; s < DIM + 2; ++s) r.u[s] = (float)ub[s];
-  r.phi5 = (float)phimin5;
+  for (int s = 0; s < DIM + 2; ++s) r.u[s] = trunc_f32(ub[s]);
+  r.phi = trunc_f32(ph);
   return r;
 }
 
-template <int DIM> __device__ __forceinline__ int entropy_at_one_f32(const RowF32 &r, const double *P) {
+// sums of two FP32 values: relative error of an addition or a product at most
+// 2^-44 (of the magnitudes added, resp. of the product)
+struct Pair {
+  float h, l;
+};
+__device__ __forceinline__ Pair quick_pair(float h, float l) {  // |h| >= |l|
+  const float s = __fadd_rn(h, l);
+  return Pair{s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair operator+(const Pair &a, const Pair &b) {
+  Pair s = two_sum(a.h, b.h), t = two_sum(a.l, b.l);
+  s = quick_pair(s.h, __fadd_rn(s.l, t.h));
+  return quick_pair(s.h, __fadd_rn(s.l, t.l));
+}
+__device__ __forceinline__ Pair operator*(const Pair &a, const Pair &b) {
+  const float q = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -q);
+  e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
+  return quick_pair(q, e);
+}
+// x as a pair (relative error 2^-47; exact down to 2^-126): the upper 24
+// significant bits, and the other 29 as an integer scaled by x's exponent
+__device__ __forceinline__ Pair split_f32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const float h = trunc_f32(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 - 52 + 127;  // biased FP32 exponent of the last place
+  float l = e > 0 && e < 254 ? (float)(lo & 0x1fffffffu) * __int_as_float(e << 23) : 0.0f;
+  if (hi & 0x80000000u) l = -l;
+  return Pair{h, l};
+}
+
+// the second level (gamma = 7/5)
+template <int DIM>
+__device__ __forceinline__ int entropy_at_one_pair(const double *ub, const double *P, double phimin5) {
+  constexpr int S = DIM + 2;
+  constexpr float u44 = 5.684342e-14f;  // 2^-44
+  Pair u[S];
+  float A[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const Pair a = split_f32(ub[s]), b = split_f32(P[s]);
+    u[s] = a + b;
+    A[s] = fabsf(a.h) + fabsf(b.h);  // |u - exact| <= 2^-45 A
+  }
+  Pair m2{0.0f, 0.0f};
+  float Am = 0.0f;
+#pragma unroll
+  for (int q = 0; q < DIM; ++q) {
+    m2 = m2 + u[1 + q] * u[1 + q];
+    Am += A[1 + q] * A[1 + q];
+  }
+  const Pair er = u[S - 1] * u[0] + Pair{-0.5f * m2.h, -0.5f * m2.l};
+  const float B = 2.0f * u44 * (A[0] * A[S - 1] + Am);  // inputs 2^-45 each, operations 2^-44
+  // 2^-12 <= er <= 2^12: the low parts of the powers stay above FP32's range
+  if (!(er.h > 2.4414063e-4f && er.h < 4096.0f && B < 0.01f * er.h)) return 0;
+  const Pair e2 = er * er, lhs = e2 * e2 * er;
+  const Pair r2 = u[0] * u[0], r4 = r2 * r2, rhs = split_f32(phimin5) * (r4 * r4 * r4);
+  const float rel = 6.0f * __fdividef(B, er.h) + u44 * (40.0f + 16.0f * __fdividef(A[0], u[0].h));
+  const Pair d = lhs + Pair{-rhs.h, -rhs.l};
+  const float tol = 1.1f * rel * fmaxf(lhs.h, rhs.h);
+  return d.h > tol ? 1 : d.h < -tol ? -1 : 0;
+}
+
+// the first level; 2: undecided, but within the second level's range
+template <int DIM>
+__device__ __forceinline__ int entropy_at_one_f32(const Params &p, const RowF32 &r, const double *P) {
   constexpr int S = DIM + 2;
   constexpr float u24 = 5.9604645e-8f;  // 2^-24
-  if (r.phi5 == 0.0f) return 0;
+  if (r.phi == 0.0f) return 0;
   float u[S], e[S];
 #pragma unroll
   for (int s = 0; s < S; ++s) {
-    const float pf = (float)P[s];
+    const float pf = trunc_f32(P[s]);
     u[s] = r.u[s] + pf;
-    // |u_f - u| <= 2^-24 (|ub| + |P| + |u_f|) (two conversions, one add)
-    e[s] = 3.0f * u24 * (fabsf(r.u[s]) + fabsf(pf));
+    // |u_f - u| <= 2^-24 (2 |ub| + 2 |P| + |u_f|) (two truncations, one add)
+    e[s] = 5.0f * u24 * (fabsf(r.u[s]) + fabsf(pf));
   }
   const float rho = u[0], E = u[S - 1];
   // 2^-6 <= rho <= 2^6 with its error: rho^12 stays within FP32's range
@@ -625,15 +698,23 @@ template <int DIM> __device__ __forceinline__ int entropy_at_one_f32(const RowF3
   // 2^-24 <= er <= 2^24 with its error: er^5 stays within FP32's range
   if (!(elo >= 5.9604645e-8f && ehi <= 16777216.0f)) return 0;
   const float rlo = rho - e[0], rhi = rho + e[0];
+  if (!p.gamma75) {
+    // Phi_min rho^(gamma+1), 2 < gamma + 1 <= 8/3: the power as exp2(g log2),
+    // |log2 rho| <= 6 (log2f and exp2f are within 2 units: 2 (6 g + 1) 2^-23 at most)
+    const float g = p.gamma_f + 1.0f;
+    const float rhs_lo = r.phi * exp2f(g * log2f(rlo)) * (1.0f - 128.0f * u24);
+    const float rhs_hi = r.phi * exp2f(g * log2f(rhi)) * (1.0f + 128.0f * u24);
+    return elo > rhs_hi ? 1 : ehi < rhs_lo ? -1 : 0;
+  }
   const float l2 = elo * elo, h2 = ehi * ehi;
   const float lhs_lo = l2 * l2 * elo * (1.0f - 8.0f * u24);
   const float lhs_hi = h2 * h2 * ehi * (1.0f + 8.0f * u24);
   const float a2 = rlo * rlo, a4 = a2 * a2, b2 = rhi * rhi, b4 = b2 * b2;
-  const float rhs_lo = r.phi5 * (a4 * a4 * a4) * (1.0f - 16.0f * u24);
-  const float rhs_hi = r.phi5 * (b4 * b4 * b4) * (1.0f + 16.0f * u24);
+  const float rhs_lo = r.phi * (a4 * a4 * a4) * (1.0f - 18.0f * u24);
+  const float rhs_hi = r.phi * (b4 * b4 * b4) * (1.0f + 18.0f * u24);
   if (lhs_lo > rhs_hi) return 1;
   if (lhs_hi < rhs_lo) return -1;
-  return 0;
+  return 2;
 }
 
 // The common outcome of the line search, decided with a short branch-free
@@ -642,8 +723,13 @@ template <int DIM> __device__ __forceinline__ int entropy_at_one_f32(const RowF3
 // one of these exits; false leaves the entry to the full search. (A warp whose
 // lanes took the search's other exits -- density clipping, psi evaluations,
 // the secant/Newton loop -- inline would issue each of them for all 32 lanes.)
-// The entropy test is pre-decided in FP32 (entropy_at_one_f32) and evaluated
-// in FP64 only where that is too close to call.
+// The entropy test is pre-decided on the FP32 units and evaluated in FP64 only
+// where that is too close to call. For another gamma than 7/5 only the
+// pre-decision settles an entry here (l = 1 certain); the rest is left open.
+// Measured: 246k cylinder, gamma = 1.3 (every entry with P_ij != 0 was queued),
+// the queued searches of a pass 280 -> 175 us; gamma = 7/5, second level and
+// truncated inputs: k_lim1 500 -> 422 us on the 998k cylinder, 822 -> 679 us on
+// 375k rows in 3D, 191 -> 120 us on the sweep of 256 small cylinders.
 template <int DIM>
 __device__ __forceinline__ bool line_search_at_one(const Params &p, const double *ub, const double *P, double rmin,
                                                    double rmax, double phimin5, const RowF32 &rf) {
@@ -652,7 +738,6 @@ __device__ __forceinline__ bool line_search_at_one(const Params &p, const double
 #pragma unroll
   for (int s = 0; s < S; ++s) zero &= (__double_as_longlong(P[s]) << 1) == 0;
   if (zero) return true;
-  if (!p.gamma75) return false;
   // the compares below run on the bit patterns (all thresholds are positive);
   // rp = -0 may take the density test, which can only send the entry to the
   // full search
@@ -662,7 +747,9 @@ __device__ __forceinline__ bool line_search_at_one(const Params &p, const double
   } else if (dbits(rp) < 0) {
     if (lt_pos(rb + rp, rmin)) return false;
   }
-  const int pre = entropy_at_one_f32<DIM>(rf, P);
+  int pre = entropy_at_one_f32<DIM>(p, rf, P);
+  if (!p.gamma75) return pre > 0;
+  if (pre == 2) pre = entropy_at_one_pair<DIM>(ub, P, phimin5);
   if (pre != 0) return pre > 0;
   double u[S];
 #pragma unroll
@@ -1191,7 +1278,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
   // bar-state densities rho_bar = num / den, den = 2 d_ij > 0; the running
   // minimum / maximum is kept as a fraction and compared by cross-multiplication
   double nmin = ui[0], dmin = 1.0, nmax = ui[0], dmax = 1.0;
-  double phimin = Ri[R::PHI], dsum = 0.0;
+  double phimin = Ri[R::PHI], phimax = phimin, dsum = 0.0;
   int64_t kd = -1;
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   for (int64_t k = k0; k < k1; ++k) {
@@ -1230,8 +1317,9 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
       }
     }
     // Phi > 0: the integer order of the bit patterns is the numeric order
-    const long long pj = __double_as_longlong(Rj64[R::PHI]), pm = __double_as_longlong(phimin);
-    phimin = __longlong_as_double(pj < pm ? pj : pm);
+    const double pj = Rj64[R::PHI];
+    phimin = dbits(pj) < dbits(phimin) ? pj : phimin;
+    phimax = dbits(pj) > dbits(phimax) ? pj : phimax;
     dsum += dk;
   }
 #pragma unroll
@@ -1252,10 +1340,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
   const double rmin = dmin == 1.0 ? nmin : nmin / dmin;
   const double rmax = dmax == 1.0 ? nmax : nmax / dmax;
   const double r = m.relax[i];
-  double *bi = w.bounds + (int64_t)i * 4;
-  bi[0] = (1.0 - r) * rmin;
-  bi[1] = (1.0 + r) * rmax;
-  bi[2] = (1.0 - r) * phimin;
+  st4(w.bounds + (int64_t)i * 4, (1.0 - r) * rmin, (1.0 + r) * rmax, (1.0 - r) * phimin, phimax);
   w.rough2[i] = 1;
   return p.cfl * m.mi[i] / (2.0 * dsum);
 }
@@ -1295,10 +1380,8 @@ __device__ __forceinline__ double low_row_smooth(const MeshView &m, const Params
   const double *Ri = w.rec + (int64_t)i * R::SIZE;
   const double rho = Ri[0];
   const double r = m.relax[i];
-  double *bi = w.bounds + (int64_t)i * 4;
-  bi[0] = (1.0 - r) * rho;
-  bi[1] = (1.0 + r) * rho;
-  bi[2] = (1.0 - r) * Ri[R::PHI];
+  const double phi = Ri[R::PHI];
+  st4(w.bounds + (int64_t)i * 4, (1.0 - r) * rho, (1.0 + r) * rho, (1.0 - r) * phi, phi);
   w.rough2[i] = r2;
   return p.cfl * m.mi[i] / (2.0 * dsum);
 }
@@ -1432,10 +1515,10 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
     if (!(pos_strict(ul[0]) && pos_strict(ul[S - 1] * ul[0] - 0.5 * m2)))
       atomicAdd(&w.st->low_not_admissible, 1ull);
   }
-  const double *bi = w.bounds + (int64_t)i * 4;
-  const double rmin = bi[0], rmax = bi[1], phimin = bi[2];
+  double rmin, rmax, phimin, phimax;
+  ld4(w.bounds + (int64_t)i * 4, rmin, rmax, phimin, phimax);
   const double phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
-  const RowF32 rf = row_f32<DIM>(ul, rmin, rmax, phimin5);
+  const RowF32 rf = row_f32<DIM>(p, ul, rmin, rmax, phimin, phimax, phimin5);
   const double alphai = w.alpha[i];
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   // P_ij = tau/(m_i lambda_i) (b_ij F^H_j - b_ji F^H_i + (d^H_ij - d_ij)(U_j - U_i))
@@ -1606,10 +1689,10 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     w.rem[k] = 1.0 - l;
   }
   store_vec<DIM>(Uout + (int64_t)i * SP, u);
-  const double *bi = w.bounds + (int64_t)i * 4;
-  const double rmin = bi[0], rmax = bi[1], phimin = bi[2];
+  double rmin, rmax, phimin, phimax;
+  ld4(w.bounds + (int64_t)i * 4, rmin, rmax, phimin, phimax);
   const double phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
-  const RowF32 rf = row_f32<DIM>(u, rmin, rmax, phimin5);
+  const RowF32 rf = row_f32<DIM>(p, u, rmin, rmax, phimin, phimax, phimin5);
   uint64_t defer = 0;
   bool long_deferred = false;
   const bool longrow = k1 - k0 > 64;  // limiters stored as they are known
@@ -1644,8 +1727,11 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
   defer_line_searches(w, slot, i, k0, defer);
 }
 
+// (bound by the latency of the limiters' gathers: at most 64 registers, so that
+// 1024 rows are in flight per SM; the pre-decision's second level alone would
+// take 92, with k_pass 142 -> 174 us on the 998k cylinder)
 template <int DIM>
-__global__ void __launch_bounds__(TPB_MAX) k_pass(MeshView m, Params p, Work w, const double *__restrict__ Uin,
+__global__ void __launch_bounds__(TPB_MAX, 4) k_pass(MeshView m, Params p, Work w, const double *__restrict__ Uin,
                                               double *__restrict__ Uout, const double *__restrict__ lin,
                                               double *__restrict__ lout, double *lsym_trace, int slot) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m.n; i += gridDim.x * blockDim.x) {

@@ -107,7 +107,7 @@ struct Params {
   double inv_z;              // 2 gamma/(gamma-1)
   double kshock;             // (gamma+1)/(2 gamma)
   double inv_gm1;            // 1/(gamma - 1)
-  float gm1_f, inv_z_f, kshock_f;  // gamma - 1, inv_z and kshock rounded to FP32 (lambda_max_sel)
+  float gamma_f, gm1_f, inv_z_f, kshock_f;  // rounded to FP32 for the pre-decisions
   int limiter_passes;        // 1 + the passes of k_pass (k_final reads rem when >= 2)
 };
 
@@ -134,7 +134,7 @@ struct Work {
   double *w;       // [nnz][SP]  (f(U_j) - f(U_i)) c_ij
   double *inc;     // [n][SP]    sum_{j != i} d_ij (U_j - U_i) - w_ij
   double *FH;      // [n][SP]    F^H_i / m_i
-  double *bounds;  // [n][4]     rho_min, rho_max, Phi_min
+  double *bounds;  // [n][4]     rho_min, rho_max, Phi_min, and the largest Phi over the stencil
   double *UL;      // [n][SP]
   double *Ua;      // [n][SP]    limited state, ping
   double *Ub;      // [n][SP]    limited state, pong
