@@ -656,6 +656,8 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
   p.kshock = (cfg->gamma + 1.0) / (2.0 * cfg->gamma);
   p.inv_gm1 = 1.0 / (cfg->gamma - 1.0);
   p.gamma_f = (float)p.gamma;
+  p.cfl_f = (float)p.cfl;
+  p.relaxed = cfg->bound_relaxation ? 1 : 0;
   p.gm1_f = (float)p.gm1;
   p.inv_z_f = (float)p.inv_z;
   p.kshock_f = (float)p.kshock;
@@ -951,6 +953,11 @@ eh_status eh_run(eh_ctx *c, int32_t nsteps, double dt) {
   return EH_OK;
 }
 
+static void set_cfl(eh_ctx *c, double cfl) {
+  c->prm.cfl = cfl;
+  c->prm.cfl_f = (float)cfl;
+}
+
 eh_status eh_step_adaptive(eh_ctx *c, double cfl_max, double *dt_used, double *cfl_used, int32_t *restarts) {
   eh_status st = require_ready(c);
   if (st) return st;
@@ -967,7 +974,7 @@ eh_status eh_step_adaptive(eh_ctx *c, double cfl_max, double *dt_used, double *c
   double cfl = cfl_max;
   int32_t r = 0;
   for (;;) {
-    c->prm.cfl = cfl;
+    set_cfl(c, cfl);
     CUDA_TRY(c, cudaMemsetAsync(&c->st->err, 0, sizeof(int), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(&c->st->low_not_admissible, 0, sizeof(unsigned long long), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(&c->st->not_admissible, 0, sizeof(unsigned long long), c->stream));
@@ -978,7 +985,7 @@ eh_status eh_step_adaptive(eh_ctx *c, double cfl_max, double *dt_used, double *c
     const int e = c->st_host->err;
     const bool failed = e == EH_ERR_NOT_ADMISSIBLE || c->st_host->low_not_admissible > 0;
     if (e && !failed) {
-      c->prm.cfl = c->cfg.cfl;
+      set_cfl(c, c->cfg.cfl);
       return check_device_error(c);
     }
     if (!failed) break;
@@ -989,13 +996,13 @@ eh_status eh_step_adaptive(eh_ctx *c, double cfl_max, double *dt_used, double *c
     CUDA_TRY(c, cudaMemsetAsync(&c->st->err, 0, sizeof(int), c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     if (cfl <= 1.0) {  // cannot happen for an admissible state: U^L is then invariant-domain preserving
-      c->prm.cfl = c->cfg.cfl;
+      set_cfl(c, c->cfg.cfl);
       return fail(c, EH_ERR_NOT_ADMISSIBLE, "no admissible step down to c_cfl = %g", cfl);
     }
     cfl *= 0.5;
     ++r;
   }
-  c->prm.cfl = c->cfg.cfl;
+  set_cfl(c, c->cfg.cfl);
   c->steps += 1;
   c->last_stage_traced = false;
   if (dt_used) *dt_used = c->st_host->tau;

@@ -1251,10 +1251,73 @@ __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w)
   w.alpha[i] = D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;  // alpha_i / 2 (exact): d^H_ij = (a_i/2 + a_j/2) d_ij
 }
 
+// The running minimum and maximum of a row's bar-state densities rho_bar = num /
+// den, den = 2 d_ij > 0, kept as fractions. Against both, a new fraction is
+// first compared in FP32 (8 units of 2^-24 a quotient; margin 2e-6, 32 units):
+// most lie clearly between, or clearly outside; only near ties are compared as
+// the FP64 cross products decide (4 FP64 instructions an entry otherwise).
+struct DensityBounds {
+  double nmin, dmin, nmax, dmax;
+  float fmin, fmax;  // the fractions in FP32
+  __device__ __forceinline__ explicit DensityBounds(double rho)
+      : nmin(rho), dmin(1.0), nmax(rho), dmax(1.0), fmin(trunc_f32(rho)), fmax(fmin) {}
+  __device__ __forceinline__ void add(double num, double dk) {  // dk = d_ij > 0
+    const float nf = trunc_f32(num), df = 2.0f * trunc_f32(dk);
+    const float q = __fdividef(nf, df);
+    constexpr float lo = 1.0f - 2e-6f, hi = 1.0f + 2e-6f;
+    const bool fine = nf > 1e-30f && nf < 1e30f && df > 1e-30f && df < 1e30f && fmin > 1e-30f && fmax < 1e30f;
+    if (fine && q > fmin * hi && q < fmax * lo) return;
+    const double den = 2.0 * dk;
+    if (fine && q < fmin * lo) {
+      nmin = num;
+      dmin = den;
+      fmin = q;
+    } else if (fine && q > fmax * hi) {
+      nmax = num;
+      dmax = den;
+      fmax = q;
+    } else {
+      if (order_key(num * dmin) < order_key(nmin * den)) {
+        nmin = num;
+        dmin = den;
+        fmin = q;
+      }
+      if (order_key(num * dmax) > order_key(nmax * den)) {
+        nmax = num;
+        dmax = den;
+        fmax = q;
+      }
+    }
+  }
+  __device__ __forceinline__ double rho_min() const { return dmin == 1.0 ? nmin : nmin / dmin; }
+  __device__ __forceinline__ double rho_max() const { return dmax == 1.0 ? nmax : nmax / dmax; }
+};
+
+// c_cfl m_i / (2 sum_j d_ij), or +inf where FP32 shows it to be above the
+// instance's minimum so far (which only ever falls): the division is then left out
+__device__ __forceinline__ double row_cfl_bound(const Params &p, double m, double dsum, unsigned long long so_far) {
+  const float est = __fdividef(0.5f * p.cfl_f * trunc_f32(m), trunc_f32(dsum));
+  if (est > trunc_f32(__longlong_as_double((long long)so_far)) * (1.0f + 4e-6f) && est < 1e30f) return INFINITY;
+  return p.cfl * m / (2.0 * dsum);
+}
+
+// the local bounds, relaxed by (1 -/+ r_i) where the context asks for it
+__device__ __forceinline__ void store_bounds(const MeshView &m, const Params &p, const Work &w, int i, double rmin,
+                                             double rmax, double phimin, double phimax) {
+  if (p.relaxed) {
+    const double r = m.relax[i];
+    rmin = (1.0 - r) * rmin;
+    rmax = (1.0 + r) * rmax;
+    phimin = (1.0 - r) * phimin;
+  }
+  st4(w.bounds + (int64_t)i * 4, rmin, rmax, phimin, phimax);
+}
+
 // Algorithm 1 steps 2-3 for one row; returns the row's CFL bound
-// c_cfl m_i / (2 sum_{j != i} d_ij)
+// c_cfl m_i / (2 sum_{j != i} d_ij), or +inf (row_cfl_bound)
 template <int DIM, typename T>
-__device__ __forceinline__ double low_row(const MeshView &m, const Params &p, const Work &w, int i) {
+__device__ __forceinline__ double low_row(const MeshView &m, const Params &p, const Work &w, int i,
+                                          unsigned long long so_far) {
   constexpr int S = DIM + 2;
   constexpr int SP = Layout<DIM>::SP;
   using R = Rec<DIM>;
@@ -1275,9 +1338,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
     wsum[s] = T(0);
     fh[s] = T(0);
   }
-  // bar-state densities rho_bar = num / den, den = 2 d_ij > 0; the running
-  // minimum / maximum is kept as a fraction and compared by cross-multiplication
-  double nmin = ui[0], dmin = 1.0, nmax = ui[0], dmax = 1.0;
+  DensityBounds rb(ui[0]);
   double phimin = Ri[R::PHI], phimax = phimin, dsum = 0.0;
   int64_t kd = -1;
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
@@ -1302,20 +1363,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
       fh[s] += dH * (T)du;
       wsum[s] += wk[s];
     }
-    if (dbits(dk) > 0) {  // dk >= 0
-      const double num = dk * (ui[0] + Rj[0]) - w0;
-      const double den = 2.0 * dk;
-      const long long knew_min = order_key(num * dmin), kmin = order_key(nmin * den);
-      const long long knew_max = order_key(num * dmax), kmax = order_key(nmax * den);
-      if (knew_min < kmin) {
-        nmin = num;
-        dmin = den;
-      }
-      if (knew_max > kmax) {
-        nmax = num;
-        dmax = den;
-      }
-    }
+    if (dbits(dk) > 0) rb.add(dk * (ui[0] + Rj[0]) - w0, dk);  // dk >= 0
     // Phi > 0: the integer order of the bit patterns is the numeric order
     const double pj = Rj64[R::PHI];
     phimin = dbits(pj) < dbits(phimin) ? pj : phimin;
@@ -1337,12 +1385,9 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
     fhi[s] = fh[s] * imi;
     if constexpr (sizeof(T) == 4) w.G64[(int64_t)i * SP + s] = (double)fhi[s];
   }
-  const double rmin = dmin == 1.0 ? nmin : nmin / dmin;
-  const double rmax = dmax == 1.0 ? nmax : nmax / dmax;
-  const double r = m.relax[i];
-  st4(w.bounds + (int64_t)i * 4, (1.0 - r) * rmin, (1.0 + r) * rmax, (1.0 - r) * phimin, phimax);
+  store_bounds(m, p, w, i, rb.rho_min(), rb.rho_max(), phimin, phimax);
   w.rough2[i] = 1;
-  return p.cfl * m.mi[i] / (2.0 * dsum);
+  return row_cfl_bound(p, m.mi[i], dsum, so_far);
 }
 
 // The same for a row whose neighbours all carry U_i bit for bit (rough[i] =
@@ -1351,7 +1396,8 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
 // the values the general row gives, bit for bit. Only sum_j d_ij remains
 // (same order). rough2[i] records whether a neighbour is rough.
 template <int DIM, typename T>
-__device__ __forceinline__ double low_row_smooth(const MeshView &m, const Params &p, const Work &w, int i) {
+__device__ __forceinline__ double low_row_smooth(const MeshView &m, const Params &p, const Work &w, int i,
+                                                 unsigned long long so_far) {
   constexpr int S = DIM + 2;
   constexpr int SP = Layout<DIM>::SP;
   using R = Rec<DIM>;
@@ -1379,43 +1425,51 @@ __device__ __forceinline__ double low_row_smooth(const MeshView &m, const Params
   }
   const double *Ri = w.rec + (int64_t)i * R::SIZE;
   const double rho = Ri[0];
-  const double r = m.relax[i];
   const double phi = Ri[R::PHI];
-  st4(w.bounds + (int64_t)i * 4, (1.0 - r) * rho, (1.0 + r) * rho, (1.0 - r) * phi, phi);
+  store_bounds(m, p, w, i, rho, rho, phi, phi);
   w.rough2[i] = r2;
-  return p.cfl * m.mi[i] / (2.0 * dsum);
+  return row_cfl_bound(p, m.mi[i], dsum, so_far);
 }
 
 // ---------------------------------------------------------------------------
 // k_low: Algorithm 1 steps 2-3 -- d_ii, CFL bound, low-order increment, local
 // bounds and high-order fluxes
 // ---------------------------------------------------------------------------
+// the smallest of a warp's bit patterns
+__device__ __forceinline__ unsigned long long warp_min_bits(unsigned long long b) {
+  const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32));
+  const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0xffffffffu);
+  return (unsigned long long)hi << 32 | lo;
+}
+
+// Folds the rows' CFL bounds into their instances' minima (exact and order
+// independent: the bit patterns of positive doubles order like their values,
+// and NaN patterns like values above every bound). A warp whose rows lie in one
+// instance reduces first; an atomic is issued only below the minimum so far.
+__device__ __forceinline__ void fold_bound(const Work &w, double bound, int inst, unsigned long long so_far) {
+  const unsigned long long b = (unsigned long long)dbits(bound), inf = 0x7FF0000000000000ull;
+  if (__reduce_min_sync(0xffffffffu, (unsigned)inst) == __reduce_max_sync(0xffffffffu, (unsigned)inst)) {
+    const unsigned long long m = warp_min_bits(b);
+    if ((threadIdx.x & 31) == 0 && m < inf && m < so_far) atomicMin(&w.bound_bits[inst], m);
+  } else if (b < inf && b < so_far) {
+    atomicMin(&w.bound_bits[inst], b);
+  }
+}
+
+// Bound by FP64 issue. Of the 32.6 FP64 instructions an entry that a row took
+// (998k cylinder: 8.1M warp instructions, 486 us), the sums need 21; the bar
+// states' cross products, the relaxation of strict bounds, most rows' division
+// for the CFL bound and the minima's FP64 compares are gone: 26.7 (397 us).
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_low(MeshView m, Params p, Work w) {
-  __shared__ double smin[TPB_MAX / 32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double bound = INFINITY;
-  if (i < m.n && !w.st->err) bound = w.rough[i] ? low_row<DIM, T>(m, p, w, i) : low_row_smooth<DIM, T>(m, p, w, i);
-  // per-instance minimum of the CFL bound (exact and order independent: the
-  // bit patterns of positive doubles order like their values). A block whose
-  // rows lie in one instance reduces first and issues one atomic.
-  const int first = blockIdx.x * blockDim.x;
-  const int last = min(first + (int)blockDim.x, m.n) - 1;
-  const int k_first = m.inst ? m.inst[first] : 0;
-  const int k_last = m.inst ? m.inst[last] : 0;
-  if (k_first == k_last) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) bound = fmin(bound, __shfl_xor_sync(0xffffffffu, bound, off));
-    if ((threadIdx.x & 31) == 0) smin[threadIdx.x >> 5] = bound;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double b = smin[0];
-      for (int q = 1; q < (int)(blockDim.x >> 5); ++q) b = fmin(b, smin[q]);
-      if (b < INFINITY) atomicMin(&w.bound_bits[k_first], (unsigned long long)__double_as_longlong(b));
-    }
-  } else if (i < m.n && bound < INFINITY) {
-    atomicMin(&w.bound_bits[m.inst[i]], (unsigned long long)__double_as_longlong(bound));
-  }
+  const int inst = m.inst ? m.inst[min(i, m.n - 1)] : 0;
+  const unsigned long long so_far = __ldcg(&w.bound_bits[inst]);
+  if (i < m.n && !w.st->err)
+    bound = w.rough[i] ? low_row<DIM, T>(m, p, w, i, so_far) : low_row_smooth<DIM, T>(m, p, w, i, so_far);
+  __syncwarp();
+  fold_bound(w, bound, inst, so_far);
 }
 
 // ---------------------------------------------------------------------------

@@ -107,7 +107,8 @@ struct Params {
   double inv_z;              // 2 gamma/(gamma-1)
   double kshock;             // (gamma+1)/(2 gamma)
   double inv_gm1;            // 1/(gamma - 1)
-  float gamma_f, gm1_f, inv_z_f, kshock_f;  // rounded to FP32 for the pre-decisions
+  float gamma_f, gm1_f, inv_z_f, kshock_f, cfl_f;  // rounded to FP32 for the pre-decisions
+  int relaxed;               // the local bounds are relaxed (MeshView::relax)
   int limiter_passes;        // 1 + the passes of k_pass (k_final reads rem when >= 2)
 };
 
