@@ -463,10 +463,12 @@ struct LsBracket {
   bool done;
 };
 
-// phimin5 = phimin^5 (used by the gamma = 7/5 fast check only).
+// the exits without psi: P = 0, the density limit l, (gamma = 7/5) the entropy
+// bound met there; otherwise done = false and l is set. phimin5 = phimin^5 (used
+// by the gamma = 7/5 fast check only).
 template <int DIM>
-__device__ LsBracket line_search_start(const Params &p, const double *ub, const double *P, double rmin, double rmax,
-                                       double phimin, double phimin5) {
+__device__ __forceinline__ LsBracket line_search_bracket(const Params &p, const double *ub, const double *P, double rmin,
+                                                         double rmax, double phimin5) {
   constexpr int S = DIM + 2;
   LsBracket b{1.0, 0.0, 0.0, 0.0, true};
   // P = 0 (every edge whose previous limiter was 1, uniform flow): every l gives
@@ -504,12 +506,24 @@ __device__ LsBracket line_search_start(const Params &p, const double *ub, const 
         if (lt_pos(rhs, 1e300) && dbits(lhs) >= dbits(rhs)) return b;
       }
     }
+  }
+  b.done = false;
+  return b;
+}
+
+template <int DIM>
+__device__ LsBracket line_search_start(const Params &p, const double *ub, const double *P, double rmin, double rmax,
+                                       double phimin, double phimin5) {
+  LsBracket b = line_search_bracket<DIM>(p, ub, P, rmin, rmax, phimin5);
+  if (b.done) return b;
+  b.done = true;
+  if (p.gamma75) {
     double r0;
-    b.pr = psi_g75<DIM>(ub, P, l, phimin, &b.rR);
+    b.pr = psi_g75<DIM>(ub, P, b.l, phimin, &b.rR);
     if (!neg_strict(b.pr)) return b;
     b.pl = psi_g75<DIM>(ub, P, 0.0, phimin, &r0);
   } else {
-    b.pr = psi<DIM>(p, ub, P, l, phimin);
+    b.pr = psi<DIM>(p, ub, P, b.l, phimin);
     if (!neg_strict(b.pr)) return b;
     b.pl = psi<DIM>(p, ub, P, 0.0, phimin);
   }
@@ -555,6 +569,75 @@ __device__ double line_search_iterate(const Params &p, const double *ub, const d
     }
   }
   return lL;
+}
+
+// The line search by pairs of neighbouring lanes that hold the same search, with
+// line_search_start's and line_search_iterate's values bit for bit: psi(l) and
+// psi(0), the secant's and Newton's divisions, and psi at their two points are
+// evaluated side by side (74 instead of 122 FP64 instructions an iteration, at
+// 63 cycles each). For queues that leave the chip idle; a full one is faster
+// with a search per lane. gamma = 7/5 (with another gamma the powers are most of
+// the time). All lanes of a warp call both.
+template <int DIM>
+__device__ __forceinline__ LsBracket line_search_start_pair(const Params &p, const double *ub, const double *P,
+                                                            double rmin, double rmax, double phimin, double phimin5) {
+  constexpr unsigned all = 0xffffffffu;
+  const bool odd = threadIdx.x & 1;
+  LsBracket b = line_search_bracket<DIM>(p, ub, P, rmin, rmax, phimin5);
+  double r;
+  const double mine = psi_g75<DIM>(ub, P, odd ? 0.0 : b.l, phimin, &r);
+  const double other = __shfl_xor_sync(all, mine, 1), r_other = __shfl_xor_sync(all, r, 1);
+  b.pr = odd ? other : mine;
+  b.pl = odd ? mine : other;
+  b.rR = odd ? r_other : r;
+  if (!b.done && !neg_strict(b.pr)) b.done = true;
+  if (!b.done && !pos_strict(b.pl)) {
+    b.l = 0.0;
+    b.done = true;
+  }
+  return b;
+}
+
+template <int DIM>
+__device__ __forceinline__ double line_search_iterate_pair(const double *ub, const double *P, double phimin,
+                                                           const LsBracket &b) {
+  constexpr unsigned all = 0xffffffffu;
+  const bool odd = threadIdx.x & 1;
+  bool done = b.done;
+  double lL = 0.0, lR = b.l, pl = b.pl, pr = b.pr, rR = b.rR, result = b.l;
+  for (int it = 0; it < LINE_SEARCH_ITERATIONS; ++it) {
+    if (__all_sync(all, done)) break;
+    const double dr = dpsi_g75<DIM>(ub, P, lR, rR, phimin);
+    // (a finished search divides 1 by 1: a zero would take the division's slow path)
+    const double q = (done ? 1.0 : odd ? pr : pl * (lR - lL)) / (done ? 1.0 : odd ? dr : pl - pr);
+    const double mine = odd ? (neg_strict(dr) ? lR - q : lR) : lL + q;
+    const double other = __shfl_xor_sync(all, mine, 1);
+    const double ls = odd ? other : mine;
+    double ln = odd ? mine : other;
+    if (order_key(ln) < order_key(ls)) ln = ls;
+    double r_mine;
+    const double p_mine = psi_g75<DIM>(ub, P, odd ? ln : ls, phimin, &r_mine);
+    const double p_other = __shfl_xor_sync(all, p_mine, 1), r_other = __shfl_xor_sync(all, r_mine, 1);
+    const double ps = odd ? p_other : p_mine, pn = odd ? p_mine : p_other, rn = odd ? r_mine : r_other;
+    const double lL0 = lL, lR0 = lR;
+    if (!neg_strict(ps)) {
+      lL = ls;
+      pl = ps;
+    }
+    if (neg_strict(pn)) {
+      lR = ln;
+      pr = pn;
+      rR = rn;
+    } else {
+      lL = ln;
+      pl = pn;
+    }
+    if (!done) result = lL;
+    // the same bracket again: every further iteration gives it again (psi at a
+    // point is a function of the point)
+    if (dbits(lL) == dbits(lL0) && dbits(lR) == dbits(lR0)) done = true;
+  }
+  return result;
 }
 
 // ---------------------------------------------------------------------------
@@ -1209,46 +1292,109 @@ __global__ void __launch_bounds__(TPB_MAX) k_visc(MeshView m, Params p, Work w, 
 // ---------------------------------------------------------------------------
 // k_alpha: the indicator alpha_i (Sec. 3.2) from the row's w_ij and a_ij
 // ---------------------------------------------------------------------------
+// eta'(U_i) from node i's record
+template <int DIM, typename T> __device__ __forceinline__ void entropy_gradient(const Params &p, const T *Ri, T *deta) {
+  using R = Rec<DIM>;
+  // eta' = (-s - rho/(gamma-1) (|v|^2/(2 eps) - gamma/rho), g1 v, -g1), g1 = rho/((gamma-1) eps)
+  const T igm1 = T(p.inv_gm1);
+  const T rho = Ri[0], irho = Ri[R::IRHO], ieps = Ri[R::IEPS];
+  T s_i = -Ri[R::ETA] * irho;
+  T g1 = rho * igm1 * ieps;
+  T v2 = T(0);
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) v2 += Ri[R::V + k] * Ri[R::V + k];
+  deta[0] = -s_i - rho * igm1 * (T(0.5) * v2 * ieps - T(p.gamma) * irho);
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) deta[1 + k] = g1 * Ri[R::V + k];
+  deta[DIM + 1] = -g1;
+}
+// entry k's terms of N_i and D_i
+template <int DIM, typename T>
+__device__ __forceinline__ void indicator_terms(const Work &w, int64_t k, const T *deta, T &n, T &d) {
+  constexpr int S = DIM + 2;
+  T wk[S], a_, d_;
+  load_edge<DIM, T>(w, k, wk, a_, d_);
+  T b_ = T(0);
+#pragma unroll
+  for (int s = 0; s < S; ++s) b_ += deta[s] * wk[s];
+  n = a_ - b_;
+  d = abs_bits(a_) + abs_bits(b_);
+}
+// alpha_i / 2 (exact): d^H_ij = (a_i/2 + a_j/2) d_ij
+template <typename T> __device__ __forceinline__ double half_alpha(T N, T D) {
+  return D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;
+}
+
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w) {
   constexpr int S = DIM + 2;
-  using R = Rec<DIM>;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.n || w.st->err) return;
   if (!w.rough[i]) {  // every w_ij and a_ij of the row is 0: N_i = D_i = 0
     w.alpha[i] = 0.0;
     return;
   }
-  const T *Ri = (const T *)w.vrec + (int64_t)i * vrec_stride<DIM, T>();
-  // eta'(U_i)
   T deta[S];
-  {
-    // eta' = (-s - rho/(gamma-1) (|v|^2/(2 eps) - gamma/rho), g1 v, -g1), g1 = rho/((gamma-1) eps)
-    const T igm1 = T(p.inv_gm1);
-    const T rho = Ri[0], irho = Ri[R::IRHO], ieps = Ri[R::IEPS];
-    T s_i = -Ri[R::ETA] * irho;
-    T g1 = rho * igm1 * ieps;
-    T v2 = T(0);
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) v2 += Ri[R::V + k] * Ri[R::V + k];
-    deta[0] = -s_i - rho * igm1 * (T(0.5) * v2 * ieps - T(p.gamma) * irho);
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) deta[1 + k] = g1 * Ri[R::V + k];
-    deta[S - 1] = -g1;
-  }
+  entropy_gradient<DIM, T>(p, (const T *)w.vrec + (int64_t)i * vrec_stride<DIM, T>(), deta);
   T N = T(0), D = T(0);
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
   for (int64_t k = k0; k < k1; ++k) {
     if (m.col[k] == i) continue;
-    T wk[S], a_, d_;
-    load_edge<DIM, T>(w, k, wk, a_, d_);
-    T b_ = T(0);
-#pragma unroll
-    for (int s = 0; s < S; ++s) b_ += deta[s] * wk[s];
-    N += a_ - b_;
-    D += abs_bits(a_) + abs_bits(b_);
+    T n, d;
+    indicator_terms<DIM, T>(w, k, deta, n, d);
+    N += n;
+    D += d;
   }
-  w.alpha[i] = D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;  // alpha_i / 2 (exact): d^H_ij = (a_i/2 + a_j/2) d_ij
+  w.alpha[i] = half_alpha(N, D);
+}
+
+// ---------------------------------------------------------------------------
+// Small meshes. One thread per row leaves most of the chip's 608 FP64 units
+// without a warp below ~20k rows, and an FP64 instruction holds its warp for 63
+// cycles: a row's serial chain (9 entries of 8 to 27 of them) is what a kernel
+// then takes. The *_split kernels give a chunk of 32 rows (a lane each) to a
+// block of several warps: the entries are dealt out (entry q to warp q mod
+// PARTS) where they are independent, the components of a sum where the order of
+// its terms matters (every sum keeps its row's column order, so the results
+// are the row kernels' bit for bit). The instruction count grows by what the
+// warps repeat, so large meshes keep one thread per row (SPLIT_ROWS).
+// ---------------------------------------------------------------------------
+constexpr int PARTS = 4;
+
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * PARTS) k_alpha_split(MeshView m, Params p, Work w) {
+  constexpr int S = DIM + 2;
+  __shared__ T sn[2][PARTS][32], sd[2][PARTS][32], sD[32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  const bool in = i < m.n && !w.st->err;
+  const bool act = in && w.rough[i];
+  T deta[S];
+  int64_t k0 = 0, k1 = 0;
+  if (act) {
+    entropy_gradient<DIM, T>(p, (const T *)w.vrec + (int64_t)i * vrec_stride<DIM, T>(), deta);
+    k0 = m.row_ptr[i];
+    k1 = m.row_ptr[i + 1];
+  }
+  // rounds of PARTS entries: every warp its entry's terms, then warp 0 adds the
+  // round's N terms and warp 1 its D terms in column order (an absent or
+  // diagonal entry adds 0, exactly)
+  T sum = T(0);
+  for (int r = 0;; ++r) {
+    const int64_t k = k0 + r * PARTS + part;
+    T n = T(0), d = T(0);
+    if (k < k1 && m.col[k] != i) indicator_terms<DIM, T>(w, k, deta, n, d);
+    sn[r & 1][part][lane] = n;
+    sd[r & 1][part][lane] = d;
+    const int more = __syncthreads_or(k0 + (r + 1) * PARTS < k1);
+    if (part < 2) {
+#pragma unroll
+      for (int q = 0; q < PARTS; ++q) sum += part == 0 ? sn[r & 1][q][lane] : sd[r & 1][q][lane];
+    }
+    if (!more) break;  // (the next round writes the other half of the buffers)
+  }
+  if (part == 1) sD[lane] = sum;
+  __syncthreads();
+  if (part == 0 && in) w.alpha[i] = act ? half_alpha(sum, sD[lane]) : 0.0;
 }
 
 // The running minimum and maximum of a row's bar-state densities rho_bar = num /
@@ -1472,6 +1618,74 @@ __global__ void __launch_bounds__(TPB_MAX) k_low(MeshView m, Params p, Work w) {
   fold_bound(w, bound, inst, so_far);
 }
 
+// The split form: warp s < S the sums of component s, warp S the bar-state and
+// Phi bounds, sum_j d_ij and the CFL bound.
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * (DIM + 3)) k_low_split(MeshView m, Params p, Work w) {
+  constexpr int S = DIM + 2, SP = Layout<DIM>::SP;
+  using R = Rec<DIM>;
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  const bool in = i < m.n && !w.st->err;
+  const bool rough = in && w.rough[i];
+  const int64_t k0 = in ? m.row_ptr[i] : 0, k1 = in ? m.row_ptr[i + 1] : 0;
+  if (part < S) {
+    if (!rough) return;  // (warp S writes a smooth row's zeros)
+    const int c = part;
+    const double ui = w.rec[(int64_t)i * R::SIZE + c], alphai = w.alpha[i];
+    double inc = 0.0;
+    T wsum = T(0), fh = T(0);
+    for (int64_t k = k0; k < k1; ++k) {
+      const int j = m.col[k];
+      if (j == i) continue;
+      const T dkT = *d_ptr<DIM, T>(w, k);
+      const T dH = T(alphai + w.alpha[j]) * dkT;
+      const double du = w.rec[(int64_t)j * R::SIZE + c] - ui;
+      inc += (double)dkT * du;
+      fh += dH * (T)du;
+      wsum += w_slot<DIM, T>(w, k)[c];
+    }
+    inc -= (double)wsum;
+    fh -= wsum;
+    const T g = fh * T(m.inv_mi[i]);
+    w.inc[(int64_t)i * SP + c] = inc;
+    ((T *)w.vFH)[(int64_t)i * SP + c] = g;
+    if constexpr (sizeof(T) == 4) w.G64[(int64_t)i * SP + c] = (double)g;
+    return;
+  }
+  const int inst = m.inst ? m.inst[min(i, m.n - 1)] : 0;
+  const unsigned long long so_far = __ldcg(&w.bound_bits[inst]);
+  double bound = INFINITY;
+  if (rough) {
+    const double *Ri = w.rec + (int64_t)i * R::SIZE;
+    const double rho = Ri[0];
+    DensityBounds rb(rho);
+    double phimin = Ri[R::PHI], phimax = phimin, dsum = 0.0;
+    int64_t kd = -1;
+    for (int64_t k = k0; k < k1; ++k) {
+      const int j = m.col[k];
+      if (j == i) {
+        kd = k;
+        continue;
+      }
+      const double *Rj = w.rec + (int64_t)j * R::SIZE;
+      const double dk = (double)*d_ptr<DIM, T>(w, k);
+      if (dbits(dk) > 0) rb.add(dk * (rho + Rj[0]) - (double)w_slot<DIM, T>(w, k)[0], dk);
+      const double pj = Rj[R::PHI];
+      phimin = dbits(pj) < dbits(phimin) ? pj : phimin;
+      phimax = dbits(pj) > dbits(phimax) ? pj : phimax;
+      dsum += dk;
+    }
+    *d_ptr<DIM, T>(w, kd) = (T)(-dsum);
+    store_bounds(m, p, w, i, rb.rho_min(), rb.rho_max(), phimin, phimax);
+    w.rough2[i] = 1;
+    bound = row_cfl_bound(p, m.mi[i], dsum, so_far);
+  } else if (in) {
+    bound = low_row_smooth<DIM, T>(m, p, w, i, so_far);
+  }
+  __syncwarp();
+  fold_bound(w, bound, inst, so_far);
+}
+
 // ---------------------------------------------------------------------------
 // k_tau: each instance's CFL bound (the minimum gathered by k_low); fixes the
 // instance's tau at the first stage (Sec. 3.1) and resets the minimum
@@ -1519,8 +1733,12 @@ __global__ void __launch_bounds__(256) k_tau(MeshView m, Work w, int stage, doub
 // ---------------------------------------------------------------------------
 // k_lim1: Algorithm 1 step 4 -- U^L, P_ij and the first line search
 // ---------------------------------------------------------------------------
-template <int DIM, typename T>
-__device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, const Work &w, double *P_trace, int i) {
+// U^L and the entries q = part, part + STEP, ... of row i; returns the mask of
+// entries left to the queued searches (of the first 64 of a row; later ones are
+// queued at once and set long_deferred)
+template <int DIM, typename T, int STEP>
+__device__ __forceinline__ uint64_t lim1_entries(const MeshView &m, const Params &p, const Work &w, double *P_trace,
+                                                 int i, int part, bool &long_deferred) {
   constexpr int S = DIM + 2;
   constexpr int SP = Layout<DIM>::SP;
   using R = Rec<DIM>;
@@ -1528,19 +1746,18 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
     // row and neighbours without a differing neighbour state: the increment
     // is 0 (U^L = U_i) and every P_ij = (tc m_ij/m_i)(0 - 0) + (.)(U_j - U_i)
     // is 0, so every search returns 1 (reading R5b) -- as the general row
-    const double *Ri = w.rec + (int64_t)i * R::SIZE;
-    double *ULi = w.UL + (int64_t)i * SP;
+    if (part == 0) {
+      double u[S];
+      load_rec_state<DIM>(w.rec + (int64_t)i * R::SIZE, u);
+      store_vec<DIM>(w.UL + (int64_t)i * SP, u);
+      if (P_trace) {
+        for (int64_t k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
 #pragma unroll
-    for (int s = 0; s < S; ++s) ULi[s] = Ri[s];
-    const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
-    if (P_trace) {
-      for (int64_t k = k0; k < k1; ++k) {
-#pragma unroll
-        for (int s = 0; s < S; ++s) P_trace[k * SP + s] = 0.0;
+          for (int s = 0; s < S; ++s) P_trace[k * SP + s] = 0.0;
+        }
       }
     }
-    w.lone[i] = 1;  // every limiter is 1; la is not written (readers check lone first)
-    return;
+    return 0;  // every limiter is 1; la is not written (readers check lone first)
   }
   const double tau = w.tau_inst[m.inst ? m.inst[i] : 0];
   const double *Ri = w.rec + (int64_t)i * R::SIZE;
@@ -1556,10 +1773,8 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
     ul[s] = ui[s] + tm * inci[s];
     gi[s] = Gi[s];
   }
-  double *ULi = w.UL + (int64_t)i * SP;
-#pragma unroll
-  for (int s = 0; s < S; ++s) ULi[s] = ul[s];
-  {
+  if (part == 0) {
+    store_vec<DIM>(w.UL + (int64_t)i * SP, ul);
     // U^L admissible: rho > 0 and rho E - |M|^2/2 > 0 (no division); with
     // c_cfl <= 1 it always is (invariant-domain property), above 1 the
     // adaptive step restarts on it
@@ -1582,9 +1797,8 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
   const double tc = tau * (double)(k1 - k0 - 1);
   const double coef = tc * m.inv_mi[i];
   uint64_t defer = 0;  // entries whose line search goes to k_ls_deferred
-  bool long_deferred = false;
   const bool longrow = k1 - k0 > 64;  // limiters stored as they are known
-  for (int64_t k = k0; k < k1; ++k) {
+  for (int64_t k = k0 + part; k < k1; k += STEP) {
     const int j = m.col[k];
     double *Pk = w.P + k * SP;
     if (j == i) {
@@ -1622,14 +1836,21 @@ __device__ __forceinline__ void lim1_row(const MeshView &m, const Params &p, con
       long_deferred = true;
     }
   }
-  const bool lone = defer == 0 && !long_deferred;
-  w.lone[i] = lone ? 1 : 0;
-  // a row with a queued search stores its other limiters (1); a row without
-  // one stores none (every limiter of it is 1, and its lone flag says so)
-  if (!lone && !longrow)
-    for (int64_t k = k0; k < k1; ++k)
-      if (!((defer >> (k - k0)) & 1ull)) w.la[k] = 1.0;
-  defer_line_searches(w, 0, i, k0, defer);
+  return defer;
+}
+
+// the row's all-ones flag, the limiters it stores and its queued searches: a row
+// with a queued search stores its other limiters (1); a row without one stores
+// none (every limiter of it is 1, and its lone flag says so)
+template <int STEP>
+__device__ __forceinline__ void lim_finish(const MeshView &m, const Work &w, unsigned char *lone_out, double *lout,
+                                           int slot, int i, int part, uint64_t defer, bool lone) {
+  const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
+  if (part == 0) lone_out[i] = lone ? 1 : 0;
+  if (!lone && k1 - k0 <= 64)
+    for (int64_t k = k0 + part; k < k1; k += STEP)
+      if (!((defer >> (k - k0)) & 1ull)) lout[k] = 1.0;
+  defer_line_searches(w, slot, i, k0, defer);
 }
 
 // rows i, i + grid size, ... (the grid may be capped to limit the rows in
@@ -1638,9 +1859,28 @@ template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_lim1(MeshView m, Params p, Work w, double *P_trace) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m.n; i += gridDim.x * blockDim.x) {
     if (w.st->err) return;
-    lim1_row<DIM, T>(m, p, w, P_trace, i);
+    bool long_deferred = false;
+    const uint64_t defer = lim1_entries<DIM, T, 1>(m, p, w, P_trace, i, 0, long_deferred);
+    lim_finish<1>(m, w, w.lone, w.la, 0, i, 0, defer, defer == 0 && !long_deferred);
   }
 }
+
+// the split form: the entries dealt out to PARTS warps
+template <int DIM, typename T>
+__global__ void __launch_bounds__(32 * PARTS) k_lim1_split(MeshView m, Params p, Work w, double *P_trace) {
+  __shared__ int queued[32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  if (part == 0) queued[lane] = 0;
+  __syncthreads();
+  const bool in = i < m.n && !w.st->err;
+  bool long_deferred = false;
+  uint64_t defer = 0;
+  if (in) defer = lim1_entries<DIM, T, PARTS>(m, p, w, P_trace, i, part, long_deferred);
+  if (defer != 0 || long_deferred) queued[lane] = 1;
+  __syncthreads();
+  if (in) lim_finish<PARTS>(m, w, w.lone, w.la, 0, i, part, defer, queued[lane] == 0);
+}
+
 
 // min of two limiters in [0, 1]: non-negative doubles order like their bit
 // patterns, so an integer min (no FP64 instruction) gives the same value
@@ -1686,6 +1926,47 @@ __device__ __forceinline__ void sym_limiters(const MeshView &m, const double *__
 // ---------------------------------------------------------------------------
 // k_pass: symmetrise the limiter, update, shrink P and search again
 // ---------------------------------------------------------------------------
+// the next search from the updated state u on the entries q = part, part + STEP,
+// ... of row i (as lim1_entries)
+template <int DIM, int STEP>
+__device__ __forceinline__ uint64_t pass_search(const MeshView &m, const Params &p, const Work &w, const double *u,
+                                                double *__restrict__ lout, int slot, int i, int part,
+                                                bool &long_deferred) {
+  constexpr int S = DIM + 2;
+  constexpr int SP = Layout<DIM>::SP;
+  const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
+  double rmin, rmax, phimin, phimax;
+  ld4(w.bounds + (int64_t)i * 4, rmin, rmax, phimin, phimax);
+  const double phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
+  const RowF32 rf = row_f32<DIM>(p, u, rmin, rmax, phimin, phimax, phimin5);
+  uint64_t defer = 0;
+  const bool longrow = k1 - k0 > 64;  // limiters stored as they are known
+  for (int64_t k = k0 + part; k < k1; k += STEP) {
+    if (m.col[k] == i) {
+      if (longrow) lout[k] = 1.0;
+      continue;
+    }
+    const double r = w.rem[k];
+    if (dbits(r) == 0) {  // the remainder is 0: every l gives the same state, the largest is 1
+      if (longrow) lout[k] = 1.0;
+      continue;
+    }
+    const double *Pk = w.P + k * SP;
+    double P[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) P[s] = r * Pk[s];
+    if (line_search_at_one<DIM>(p, u, P, rmin, rmax, phimin5, rf)) {
+      if (longrow) lout[k] = 1.0;
+    } else if (k - k0 < 64) {
+      defer |= 1ull << (k - k0);
+    } else {
+      defer_line_searches(w, slot, i, k, 1ull);
+      long_deferred = true;
+    }
+  }
+  return defer;
+}
+
 template <int DIM>
 __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, const Work &w, const double *__restrict__ Uin,
                                          double *__restrict__ Uout, const double *__restrict__ lin,
@@ -1743,42 +2024,9 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     w.rem[k] = 1.0 - l;
   }
   store_vec<DIM>(Uout + (int64_t)i * SP, u);
-  double rmin, rmax, phimin, phimax;
-  ld4(w.bounds + (int64_t)i * 4, rmin, rmax, phimin, phimax);
-  const double phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
-  const RowF32 rf = row_f32<DIM>(p, u, rmin, rmax, phimin, phimax, phimin5);
-  uint64_t defer = 0;
   bool long_deferred = false;
-  const bool longrow = k1 - k0 > 64;  // limiters stored as they are known
-  for (int64_t k = k0; k < k1; ++k) {
-    if (m.col[k] == i) {
-      if (longrow) lout[k] = 1.0;
-      continue;
-    }
-    const double r = w.rem[k];
-    if (dbits(r) == 0) {  // the remainder is 0: every l gives the same state, the largest is 1
-      if (longrow) lout[k] = 1.0;
-      continue;
-    }
-    const double *Pk = w.P + k * SP;
-    double P[S];
-#pragma unroll
-    for (int s = 0; s < S; ++s) P[s] = r * Pk[s];
-    if (line_search_at_one<DIM>(p, u, P, rmin, rmax, phimin5, rf)) {
-      if (longrow) lout[k] = 1.0;
-    } else if (k - k0 < 64) {
-      defer |= 1ull << (k - k0);
-    } else {
-      defer_line_searches(w, slot, i, k, 1ull);
-      long_deferred = true;
-    }
-  }
-  const bool lone = defer == 0 && !long_deferred;
-  lone_out[i] = lone ? 1 : 0;
-  if (!lone && !longrow)  // as in k_lim1: only a row with a queued search stores its limiters
-    for (int64_t k = k0; k < k1; ++k)
-      if (!((defer >> (k - k0)) & 1ull)) lout[k] = 1.0;
-  defer_line_searches(w, slot, i, k0, defer);
+  const uint64_t defer = pass_search<DIM, 1>(m, p, w, u, lout, slot, i, 0, long_deferred);
+  lim_finish<1>(m, w, lone_out, lout, slot, i, 0, defer, defer == 0 && !long_deferred);
 }
 
 // (bound by the latency of the limiters' gathers: at most 64 registers, so that
@@ -1792,6 +2040,68 @@ __global__ void __launch_bounds__(TPB_MAX, 4) k_pass(MeshView m, Params p, Work 
     if (w.st->err) return;
     pass_row<DIM>(m, p, w, Uin, Uout, lin, lout, lsym_trace, slot, i);
   }
+}
+
+// The split form, of the first pass after k_lim1 only (a later pass also
+// rewrites P in place): warp s adds up component s of the update (3D: warp 0
+// also the fifth), the last warp stores the remainder factors, then the
+// entries of the next search are dealt out.
+template <int DIM>
+__global__ void __launch_bounds__(32 * PARTS) k_pass_split(MeshView m, Params p, Work w, const double *__restrict__ Uin,
+                                                           double *__restrict__ Uout, const double *__restrict__ lin,
+                                                           double *__restrict__ lout, double *lsym_trace) {
+  constexpr int S = DIM + 2;
+  constexpr int SP = Layout<DIM>::SP;
+  __shared__ double su[S][32];
+  __shared__ int queued[32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  if (part == 0) queued[lane] = 0;
+  const bool in = i < m.n && !w.st->err;
+  const unsigned char *lone_in = w.lone;
+  unsigned char *lone_out = w.lone + (int64_t)m.n;
+  const bool rough = in && w.rough2[i];
+  const int64_t k0 = in ? m.row_ptr[i] : 0, k1 = in ? m.row_ptr[i + 1] : 0;
+  if (in) {
+    const bool one_i = lone_in[i] != 0;
+    const double lambda_i = m.lam[i];
+    double u = Uin[(int64_t)i * SP + part], u4 = 0.0;
+    if constexpr (S > PARTS) u4 = Uin[(int64_t)i * SP + PARTS];
+    if (rough || (lsym_trace && part == PARTS - 1)) {
+      for (int64_t k = k0; k < k1; ++k) {
+        const int j = m.col[k];
+        if (j == i) {
+          if (lsym_trace && part == PARTS - 1) lsym_trace[k] = 1.0;
+          continue;
+        }
+        const double l = lmin(one_i ? 1.0 : lin[k], lone_in[j] ? 1.0 : lin[m.tr[k]]);
+        if (part == PARTS - 1) {
+          if (lsym_trace) lsym_trace[k] = l;
+          if (rough) w.rem[k] = 1.0 - l;
+        }
+        if (!rough) continue;
+        const double *Pk = w.P + k * SP;
+        u += lambda_i * l * Pk[part];
+        if constexpr (S > PARTS) {
+          if (part == 0) u4 += lambda_i * l * Pk[PARTS];
+        }
+      }
+    }
+    su[part][lane] = u;
+    if constexpr (S > PARTS) {
+      if (part == 0) su[PARTS][lane] = u4;
+    }
+  }
+  __syncthreads();
+  double u[S];
+#pragma unroll
+  for (int c = 0; c < S; ++c) u[c] = su[c][lane];
+  if (in && part == 0) store_vec<DIM>(Uout + (int64_t)i * SP, u);
+  bool long_deferred = false;
+  uint64_t defer = 0;
+  if (rough) defer = pass_search<DIM, PARTS>(m, p, w, u, lout, 1, i, part, long_deferred);
+  if (defer != 0 || long_deferred) queued[lane] = 1;
+  __syncthreads();
+  if (in) lim_finish<PARTS>(m, w, lone_out, lout, 1, i, part, defer, queued[lane] == 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1811,25 +2121,60 @@ __device__ __forceinline__ bool queue_iteration(const Work &w, int slot, const L
   return true;
 }
 
+// queues of at most this many searches are run by lane pairs: two lanes for each
+// still leave every FP64 unit at most one warp (608 units, 32 lanes)
+constexpr unsigned LS_PAIRS = 608 * 32 / 2;
+
+// the start state and direction of search (i, k) of pass 'slot'
+template <int DIM>
+__device__ __forceinline__ void ls_load(const Work &w, const double *__restrict__ ub, int slot, int i, int k, double *u,
+                                        double *P) {
+  constexpr int S = DIM + 2;
+  constexpr int SP = Layout<DIM>::SP;
+  const double r = slot > 0 ? w.rem[k] : 1.0;  // a later pass: the remainder rem P
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    u[s] = ub[(int64_t)i * SP + s];
+    P[s] = slot > 0 ? r * w.P[(int64_t)k * SP + s] : w.P[(int64_t)k * SP + s];
+  }
+}
+// the lane pair's place in a queue run by pairs: one warp (16 searches) a block,
+// and so an SM, before a second one anywhere
+__device__ __forceinline__ unsigned pair_warp() { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
 template <int DIM>
 __global__ void __launch_bounds__(256) k_ls_deferred(MeshView m, Params p, Work w, const double *__restrict__ ub,
                                                      int slot, double *__restrict__ lout) {
   constexpr int S = DIM + 2;
-  constexpr int SP = Layout<DIM>::SP;
   if (w.st->err) return;
   const unsigned cnt = min(w.lsq_count[slot], w.lsq_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&w.st->line_searches_deferred, (unsigned long long)cnt);
+  if (cnt == 0) return;
+  if (p.gamma75 && cnt <= LS_PAIRS) {
+    // few searches: to their end here, by lane pairs, one warp (16 searches) a
+    // block and SM before a second one anywhere
+    const unsigned first = pair_warp() * 16, q = first + ((threadIdx.x & 31) >> 1);
+    if (first >= cnt) return;
+    const int2 it = w.lsq[min(q, cnt - 1)];
+    const double *bi = w.bounds + (int64_t)it.x * 4;
+    const double phimin = bi[2], phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
+    double u[S], P[S];
+    ls_load<DIM>(w, ub, slot, it.x, it.y, u, P);
+    LsBracket b = line_search_start_pair<DIM>(p, u, P, bi[0], bi[1], phimin, phimin5);
+    if (q >= cnt) b.done = true;
+    const unsigned open = __ballot_sync(0xffffffffu, !b.done);
+    if (open && (threadIdx.x & 31) == 0)
+      atomicAdd(&w.st->line_searches_iterated, (unsigned long long)(__popc(open) / 2));
+    const double l = line_search_iterate_pair<DIM>(u, P, phimin, b);
+    if (q < cnt && !(threadIdx.x & 1)) lout[it.y] = l;
+    return;
+  }
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < cnt; q += gridDim.x * blockDim.x) {
     const int2 it = w.lsq[q];
     const double *bi = w.bounds + (int64_t)it.x * 4;
     const double phimin = bi[2], phimin2 = phimin * phimin, phimin5 = phimin2 * phimin2 * phimin;
     double u[S], P[S];
-    const double r = slot > 0 ? w.rem[it.y] : 1.0;  // a later pass: the remainder rem P
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      u[s] = ub[(int64_t)it.x * SP + s];
-      P[s] = slot > 0 ? r * w.P[(int64_t)it.y * SP + s] : w.P[(int64_t)it.y * SP + s];
-    }
+    ls_load<DIM>(w, ub, slot, it.x, it.y, u, P);
     const LsBracket b = line_search_start<DIM>(p, u, P, bi[0], bi[1], phimin, phimin5);
     if (b.done)
       lout[it.y] = b.l;
@@ -1842,20 +2187,26 @@ template <int DIM>
 __global__ void __launch_bounds__(256) k_ls_iterate(MeshView m, Params p, Work w, const double *__restrict__ ub,
                                                     int slot, double *__restrict__ lout) {
   constexpr int S = DIM + 2;
-  constexpr int SP = Layout<DIM>::SP;
   if (w.st->err) return;
   const unsigned cnt = min(w.lsq2_count[slot], w.lsq2_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&w.st->line_searches_iterated, (unsigned long long)cnt);
+  if (cnt == 0) return;
+  if (p.gamma75 && cnt <= LS_PAIRS) {
+    const unsigned first = pair_warp() * 16, q = first + ((threadIdx.x & 31) >> 1);
+    if (first >= cnt) return;
+    const LsItem it = w.lsq2[min(q, cnt - 1)];
+    double u[S], P[S];
+    ls_load<DIM>(w, ub, slot, it.i, it.k, u, P);
+    const double l = line_search_iterate_pair<DIM>(u, P, w.bounds[(int64_t)it.i * 4 + 2],
+                                                   LsBracket{it.l, it.pl, it.pr, it.rR, q >= cnt});
+    if (q < cnt && !(threadIdx.x & 1)) lout[it.k] = l;
+    return;
+  }
   for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < cnt; q += gridDim.x * blockDim.x) {
     const LsItem it = w.lsq2[q];
     const double phimin = w.bounds[(int64_t)it.i * 4 + 2];
     double u[S], P[S];
-    const double r = slot > 0 ? w.rem[it.k] : 1.0;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      u[s] = ub[(int64_t)it.i * SP + s];
-      P[s] = slot > 0 ? r * w.P[(int64_t)it.k * SP + s] : w.P[(int64_t)it.k * SP + s];
-    }
+    ls_load<DIM>(w, ub, slot, it.i, it.k, u, P);
     const LsBracket b{it.l, it.pl, it.pr, it.rR, false};
     lout[it.k] = line_search_iterate<DIM>(p, u, P, phimin, b);
   }
@@ -2178,7 +2529,7 @@ __global__ void __launch_bounds__(TPB_MAX) k_final(MeshView m, Params p, Work w,
 // the non-reflecting boundary nodes of a stage: post-processing (Sec. 4.2),
 // SSP combination and admissibility, as k_final does for the other nodes
 template <int DIM>
-__global__ void __launch_bounds__(256) k_final_nonreflecting(MeshView m, Params p, Work w, const double *U0,
+__global__ void __launch_bounds__(32) k_final_nonreflecting(MeshView m, Params p, Work w, const double *U0,
                                                              double coef, double *out) {
   constexpr int S = DIM + 2;
   constexpr int SP = Layout<DIM>::SP;
@@ -2238,6 +2589,14 @@ template <int DIM> __global__ void k_count_not_admissible(int n, const double *U
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+// rows below which the split forms run. Microseconds a launch, row form ->
+// split form: 4k-vertex vortex k_visc + k_alpha 22.3 -> 17.8, k_low 19.0 -> 13.6,
+// k_lim1 18.8 -> 12.1, k_pass 13.5 -> 12.7; 6.6k vortex in a box with queued
+// searches 25.6 -> 23.1, 21.4 -> 17.4, 38.5 -> 20.7, 32.0 -> 20.5; 62k cylinder
+// 53.5 -> 56.1, 38.3 -> 46.6, 55.0 -> 49.9, 41.2 -> 40.3; 196k rows: all slower.
+// (The launch shape of eh_set_launch_shape applies to the row forms.)
+constexpr int SPLIT_SUMS = 32 * 1024;     // k_alpha, k_low: the warps repeat loads and half of the products
+constexpr int SPLIT_ENTRIES = 64 * 1024;  // k_lim1, k_pass: the entries are independent
 template <int DIM, typename T>
 void launch_prep(const MeshView &m, const Params &p, const double *U, const Work &w, int tpb, cudaStream_t s) {
   k_prep<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, U, w.rec, (T *)w.vrec, w.rough, w.steady, w.st);
@@ -2255,11 +2614,17 @@ void launch_visc(const MeshView &m, const Params &p, const Work &w, int tpb, cud
 }
 template <int DIM, typename T>
 void launch_alpha(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {
-  k_alpha<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
+  if (m.n < SPLIT_SUMS)
+    k_alpha_split<DIM, T><<<nblocks(m.n, 32), 32 * PARTS, 0, s>>>(m, p, w);
+  else
+    k_alpha<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
 }
 template <int DIM, typename T>
 void launch_low(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {
-  k_low<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
+  if (m.n < SPLIT_SUMS)
+    k_low_split<DIM, T><<<nblocks(m.n, 32), 32 * (DIM + 3), 0, s>>>(m, p, w);
+  else
+    k_low<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
 }
 void launch_tau(const MeshView &m, const Work &w, int stage, double dt_given, double cfl, bool advance_time,
                 cudaStream_t s) {
@@ -2274,12 +2639,18 @@ inline unsigned capped_grid(int64_t n, int tpb, int max_blocks) {
 template <int DIM, typename T>
 void launch_lim1(const MeshView &m, const Params &p, const Work &w, double *P_trace, int tpb, int max_blocks,
                  cudaStream_t s) {
-  k_lim1<DIM, T><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, P_trace);
+  if (m.n < SPLIT_ENTRIES)
+    k_lim1_split<DIM, T><<<nblocks(m.n, 32), 32 * PARTS, 0, s>>>(m, p, w, P_trace);
+  else
+    k_lim1<DIM, T><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, P_trace);
 }
 template <int DIM>
 void launch_pass(const MeshView &m, const Params &p, const Work &w, const double *Uin, double *Uout, const double *lin,
                  double *lout, double *lsym_trace, int slot, int tpb, int max_blocks, cudaStream_t s) {
-  k_pass<DIM><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, Uin, Uout, lin, lout, lsym_trace, slot);
+  if (slot == 1 && m.n < SPLIT_ENTRIES)
+    k_pass_split<DIM><<<nblocks(m.n, 32), 32 * PARTS, 0, s>>>(m, p, w, Uin, Uout, lin, lout, lsym_trace);
+  else
+    k_pass<DIM><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, Uin, Uout, lin, lout, lsym_trace, slot);
 }
 template <int DIM>
 void launch_ls_deferred(const MeshView &m, const Params &p, const Work &w, const double *ub, int slot, double *lout,
@@ -2296,7 +2667,10 @@ void launch_final(const MeshView &m, const Params &p, const Work &w, const doubl
   k_final<DIM><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, Uin, lin, U0, coef, out, Upre_trace,
                                                                  lsym_trace);
   if (m.n_nonreflecting > 0)
-    k_final_nonreflecting<DIM><<<nblocks(m.n_bnd, 256), 256, 0, s>>>(m, p, w, U0, coef, out);
+    // a warp a block: the few hundred nodes of a boundary run chains of ~400 FP64
+    // instructions (three powers); eight warps on one SM share its FP64 rate
+    // (80 x 80 box: 49 -> 35 us with k_final)
+    k_final_nonreflecting<DIM><<<nblocks(m.n_bnd, 32), 32, 0, s>>>(m, p, w, U0, coef, out);
 }
 template <int DIM> void launch_apply_bc(const MeshView &m, const Params &p, double *U, cudaStream_t s) {
   k_apply_bc<DIM><<<nblocks(m.n, 256), 256, 0, s>>>(m, p, U);
