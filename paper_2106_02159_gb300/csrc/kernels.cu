@@ -281,6 +281,30 @@ __device__ __forceinline__ T lambda_max(const Params &p, T unl, T pl, T al, T az
   return max_nonneg(pos_part(-lam1), pos_part(lam3));
 }
 
+// a - b on the integer units where a and b have the same sign and exponent (their
+// bit patterns' difference is then the exact result's significand: nothing is
+// rounded), an FP64 subtraction otherwise: the same value always. For the
+// differences of neighbouring densities, streamwise momenta and energies, which
+// rarely cross a power of two: ~26 integer instructions run beside the FP64
+// pipe instead of one of its 19-cycle slots (k_low 397 -> 386 us, k_lim1 419 ->
+// 391 us on the 998k cylinder; 609 -> 485 and 679 -> 634 us in 3D).
+__device__ __forceinline__ double sub_near(double a, double b) {
+  const int ah = __double2hiint(a), bh = __double2hiint(b);
+  const unsigned e = ((unsigned)ah >> 20) & 0x7ffu;
+  if ((unsigned)(ah ^ bh) >> 20 != 0 || e - 65u >= 0x7ffu - 65u) {
+    double r;  // (volatile: kept inside the branch, not evaluated ahead of it)
+    asm volatile("sub.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
+    return r;
+  }
+  const long long d = dbits(a) - dbits(b);
+  const long long sg = d >> 63;
+  const unsigned long long m = (unsigned long long)((d ^ sg) - sg);
+  const int sh = __clzll((long long)m) - 11;
+  const unsigned long long r = ((unsigned long long)(e - 1 - sh) << 52) + (m << sh);
+  const unsigned long long sign = ((unsigned long long)sg ^ (unsigned long long)dbits(a)) & 0x8000000000000000ull;
+  return m == 0 ? 0.0 : __longlong_as_double((long long)(r | sign));
+}
+
 // a and p of a node as an FP32 pair in one FP64 slot of its record (Rec::F32),
 // for lambda_max_sel; a = NaN when a, p or a p^-z could leave FP32's range
 __device__ __forceinline__ double pack_f32(double a, double pr, double az) {
@@ -619,7 +643,6 @@ __device__ __forceinline__ double line_search_iterate_pair(const double *ub, con
     const double p_mine = psi_g75<DIM>(ub, P, odd ? ln : ls, phimin, &r_mine);
     const double p_other = __shfl_xor_sync(all, p_mine, 1), r_other = __shfl_xor_sync(all, r_mine, 1);
     const double ps = odd ? p_other : p_mine, pn = odd ? p_mine : p_other, rn = odd ? r_mine : r_other;
-    const double lL0 = lL, lR0 = lR;
     if (!neg_strict(ps)) {
       lL = ls;
       pl = ps;
@@ -633,9 +656,6 @@ __device__ __forceinline__ double line_search_iterate_pair(const double *ub, con
       pl = pn;
     }
     if (!done) result = lL;
-    // the same bracket again: every further iteration gives it again (psi at a
-    // point is a function of the point)
-    if (dbits(lL) == dbits(lL0) && dbits(lR) == dbits(lR0)) done = true;
   }
   return result;
 }
@@ -1504,7 +1524,7 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
     const double w0 = (double)wk[0];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const double du = Rj[s] - ui[s];
+      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : Rj[s] - ui[s];
       inc[s] += dk * du;  // sum_j d_ij (U_j - U_i); the sum of w_ij is subtracted once
       fh[s] += dH * (T)du;
       wsum[s] += wk[s];
@@ -1820,7 +1840,8 @@ __device__ __forceinline__ uint64_t lim1_entries(const MeshView &m, const Params
     double P[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      P[s] = cm * (gi[s] - Gj[s]) + cd * (Rj[s] - ui[s]);
+      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : Rj[s] - ui[s];
+      P[s] = __fma_rn(cm, gi[s] - Gj[s], __dmul_rn(cd, du));
     }
     store_vec<DIM>(Pk, P);
     if (P_trace) {
