@@ -279,7 +279,7 @@ eh_status eh_profile_read(eh_ctx *ctx, int kernel, double *total_ms, int64_t *la
  * the current device; the call does not synchronise. Returns EH_ERR_CUDA,
  * without launching, if a CUDA error from earlier work is pending (it is left
  * in place for the caller to read), and EH_ERR_CUDA if a launch fails.
- * Scratch: a file-scope device array of EH_CFL_NOALLOC_MAX_ROWS / 128 + 1
+ * Scratch: a file-scope device array of EH_CFL_NOALLOC_MAX_ROWS / 128 + 2
  * doubles (512 KiB) that every GPU loading the library keeps until the process ends;
  * n above EH_CFL_NOALLOC_MAX_ROWS returns EH_ERR_INVALID_ARG before any work.
  * The first call in each CUDA context of a device looks the array's device

@@ -24,10 +24,10 @@ constexpr int kThreads = 128;
 constexpr int kMaxBlocks = EH_CFL_NOALLOC_MAX_ROWS / kThreads;
 constexpr int kMaxDevices = 64;
 
-// The scratch: one 8-byte slot per block of kThreads rows (512 KiB; first the
-// block's FP32 bracket of its smallest bound, then its exact minimum) and one
-// more for the smallest upper end over all blocks.
-static __device__ __align__(256) double g_cfl_block_min[kMaxBlocks + 1];
+// The scratch: one 8-byte slot per block of kThreads rows (512 KiB; the lower end
+// of the block's FP32 bracket) and two more: the smallest upper end over all
+// blocks, and the order key of the smallest exact bound.
+static __device__ __align__(256) double g_cfl_block_min[kMaxBlocks + 2];
 
 // Device address of g_cfl_block_min, looked up once per device and context:
 // the address belongs to the module loaded into one CUDA context, so the cache
@@ -57,6 +57,19 @@ template <int DIM> __device__ inline Node<DIM> load_state(const double *U, int n
   return w;
 }
 
+// x^(-1/7): Newton's method on r^-7 = x, r <- r (8 - x r^7) / 7, from an FP32 seed
+// (gamma = 7/5: p^-z with a tenth of pow's FP64 instructions; the same accuracy)
+__device__ inline double inverse_root7(double x) {
+  if (!(x > 1e-30 && x < 1e30)) return pow(x, -1.0 / 7.0);
+  double r = (double)exp2f((-1.0f / 7.0f) * log2f((float)x));
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double r2 = r * r, r7 = r2 * r2 * r2 * r;
+    r = r * (8.0 - x * r7) * (1.0 / 7.0);
+  }
+  return r;
+}
+
 template <int DIM> __device__ inline void derive(Node<DIM> &w, double gamma) {
   double m2 = 0.0;
 #pragma unroll
@@ -64,7 +77,7 @@ template <int DIM> __device__ inline void derive(Node<DIM> &w, double gamma) {
   double eps = w.E - m2 / (2.0 * w.rho);
   w.p = (gamma - 1.0) * eps;
   w.a = sqrt(gamma * w.p / w.rho);
-  w.az = w.a * pow(w.p, -(gamma - 1.0) / (2.0 * gamma));
+  w.az = w.a * (gamma == 1.4 ? inverse_root7(w.p) : pow(w.p, -(gamma - 1.0) / (2.0 * gamma)));
   w.ip = 1.0 / w.p;
 }
 
@@ -81,7 +94,8 @@ template <int DIM> __device__ inline double normal_velocity(const Node<DIM> &w, 
 template <int DIM>
 __device__ inline double wave_bound(const Node<DIM> &l, double ul, const Node<DIM> &r, double ur, double gamma) {
   double num = fmax(l.a + r.a - 0.5 * (gamma - 1.0) * (ur - ul), 0.0);
-  double ptr = pow(num / (l.az + r.az), 2.0 * gamma / (gamma - 1.0));
+  const double x = num / (l.az + r.az), x2 = x * x, x4 = x2 * x2;
+  double ptr = gamma == 1.4 ? x4 * x2 * x : pow(x, 2.0 * gamma / (gamma - 1.0));
   double k = (gamma + 1.0) / (2.0 * gamma);
   double sl = ptr > l.p ? sqrt(1.0 + k * (ptr - l.p) * l.ip) : 1.0;
   double sr = ptr > r.p ? sqrt(1.0 + k * (ptr - r.p) * r.ip) : 1.0;
@@ -161,10 +175,18 @@ __device__ inline double graph_viscosity(const Arrays &g, int i, int j, int64_t 
   return d;
 }
 
-// min(a, b) that keeps a NaN: a row whose state is not admissible (rho <= 0 or
-// internal energy <= 0) gives a NaN bound, which must reach dt_out instead of
-// being dropped by the reduction
-__device__ __forceinline__ double nan_min(double a, double b) { return (a < b || a != a) ? a : b; }
+// An integer key with the order of the doubles, a NaN below everything: a row
+// whose state is not admissible (rho <= 0 or internal energy <= 0) gives a NaN
+// bound, which must reach dt_out instead of being dropped by the reduction.
+__device__ __forceinline__ long long bound_key(double x) {
+  if (x != x) return (long long)0x8000000000000000ull;
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFLL);
+}
+__device__ __forceinline__ double key_bound(long long k) {
+  if (k == (long long)0x8000000000000000ull) return NAN;
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFLL));
+}
 
 // the row's own state must be admissible: otherwise the wave speeds are
 // undefined and the step is NaN
@@ -211,15 +233,15 @@ template <int DIM> __device__ inline double row_bound_warp(const Arrays &g, int 
 // ---------------------------------------------------------------------------
 // The FP32 bracket of a row's bound. Only the smallest bound is wanted, and
 // FP64 issues at 1/76 of the FP32 rate on this part: every row's bound is
-// bracketed in FP32 interval arithmetic, and only rows whose lower end does
-// not exceed the smallest upper end are evaluated in FP64 (998k-vertex Q1
-// cylinder, perturbed flow: 6757 -> 275 us for the step, the same bits; before,
-// every entry took 3 powers, 2 roots and 6 divisions in FP64, twice per edge;
-// what remains is the gather of the neighbours' states). The brackets below
-// carry every rounding (u = 2^-23 per conversion or operation is twice what
-// either does; log2f and exp2f are within 2 units); a row with anything out
-// of FP32's range, or not clearly admissible, gets (-inf, inf) and is
-// evaluated in FP64.
+// bracketed in FP32, and only rows whose lower end does not exceed the smallest
+// upper end are evaluated in FP64. 998k-vertex Q1 cylinder, perturbed flow:
+// 6757 us with every entry in FP64 (3 powers, 2 roots and 6 divisions an entry),
+// 275 us with FP32 interval arithmetic (both ends of every quantity, 520
+// instructions an entry), 179 us with a value and an error bound for each: bound by
+// instruction issue in k_cfl_bracket. The bounds carry every rounding (u = 2^-23
+// per conversion or operation is twice what either does; log2f and exp2f are
+// within 2 units); a row with anything out of FP32's range, or not clearly
+// admissible, gets (-inf, inf) and is evaluated in FP64.
 // ---------------------------------------------------------------------------
 struct Bracket {
   float lo, hi;
@@ -240,17 +262,21 @@ __device__ __forceinline__ float trunc_f32(double x) {
   return __uint_as_float(r);
 }
 
-// a node in FP32: velocity, its 1-norm, p, a and a p^-z, and a bound on the
-// relative error of those three (velocity: 5 u)
-template <int DIM> struct NodeF {
-  float v[DIM], V, p, a, az, err;
-  bool ok;
+struct Gas {
+  float gamma, gm1, g, z, iz, k;  // gamma, gamma-1, (gamma-1)/2, z, 1/z, (gamma+1)/(2 gamma)
+  int gamma75;
 };
 
-template <int DIM> __device__ inline NodeF<DIM> node_f32(const Arrays &g, float gamma, float z, int i) {
-  NodeF<DIM> w;
+// a node in FP32: velocity, its 1-norm, p, 1/p, a and a p^-z, and a bound on the
+// relative error of those four (velocity: 5 u)
+template <int DIM> struct NodeF {
+  float v[DIM], V, p, ip, a, az, err;
+};
+
+// false: out of range, or not clearly admissible
+template <int DIM> __device__ inline bool node_f32(const Arrays &g, const Gas &G, int i, NodeF<DIM> &w) {
   const float rho = trunc_f32(g.U[i]), E = trunc_f32(g.U[(int64_t)(DIM + 1) * g.n + i]);
-  const float ir = 1.0f / rho;
+  const float ir = __fdividef(1.0f, rho);
   float m2 = 0.0f;
   w.V = 0.0f;
 #pragma unroll
@@ -261,66 +287,75 @@ template <int DIM> __device__ inline NodeF<DIM> node_f32(const Arrays &g, float 
     w.V += fabsf(w.v[q]);
   }
   const float ke = 0.5f * m2 * ir, eps = E - ke;
-  const float ee = 10.0f * kU * (E + ke) / eps;  // relative error of eps
-  w.p = (gamma - 1.0f) * eps;
-  w.a = sqrtf(gamma * w.p * ir);
-  const float lp = log2f(w.p);
-  w.az = w.a * exp2f(-z * lp);
-  w.err = ee + 16.0f * kU + 4.0f * kU * z * fabsf(lp);
-  w.ok = rho > 1e-30f && eps > 1e-30f && ee < 0.01f && w.err < 0.02f && E < 1e30f && w.p > 1e-30f && w.a < 1e18f &&
-         w.V < 1e18f && w.az > 1e-30f && w.az < 1e30f;
-  return w;
+  const float ee = __fdividef(10.0f * kU * (E + ke), eps);  // relative error of eps
+  w.p = G.gm1 * eps;
+  w.ip = __fdividef(1.0f, w.p);
+  w.a = sqrtf(G.gamma * w.p * ir);
+  const float lp = __log2f(w.p);  // absolute error 2^-21.5 in [0.5, 2], else 3 ulps: within 4 u (1 + |lp|)
+  w.az = w.a * exp2f(-G.z * lp);
+  w.err = ee + 20.0f * kU + 6.0f * kU * G.z * (1.0f + fabsf(lp));
+  return rho > 1e-30f && rho < 1e30f && eps > 1e-30f && ee < 0.01f && w.err < 0.02f && E < 1e30f && w.p > 1e-30f &&
+         w.a > 1e-18f && w.a < 1e18f && w.V < 1e18f && w.az > 1e-30f && w.az < 1e30f;
 }
 
-struct Gas {
-  float gamma, g, z, iz, k;  // gamma, (gamma-1)/2, z, 1/z, (gamma+1)/(2 gamma)
-};
-
-// bracket of lambda_max |c| from l to r along c; false: out of range
+// lambda_max |c| from l to r along c, as a value and a bound on its absolute
+// error; false: out of range. An error of the numerator of p_tr is carried to
+// x = num / den, to p_tr (iz times) and to s = sqrt(1 + k (p_tr/p - 1)_+): with
+// s >= 1 and s^2 >= k p_tr/p + (1 - k), an error e of p_tr/p changes s by at most
+// 0.5 k (p_tr/p) e / s <= 0.5 s e / (1 - ...) <= s e (taken twice over).
 template <int DIM>
-__device__ inline bool wave_f32(const Gas &G, const NodeF<DIM> &l, const NodeF<DIM> &r, const float *c, float sgn,
-                                float *dlo, float *dhi) {
-  float s2 = 0.0f, ul = 0.0f, ur = 0.0f;
-#pragma unroll
-  for (int q = 0; q < DIM; ++q) s2 += c[q] * c[q];
-  const float cn = sqrtf(s2), ci = sgn / cn;
+__device__ inline bool wave_f32(const Gas &G, const NodeF<DIM> &l, const NodeF<DIM> &r, const float *c, float *d,
+                                float *err) {
+  float s2 = 0.0f, vl = 0.0f, vr = 0.0f;
 #pragma unroll
   for (int q = 0; q < DIM; ++q) {
-    ul += l.v[q] * (c[q] * ci);
-    ur += r.v[q] * (c[q] * ci);
+    s2 += c[q] * c[q];
+    vl += l.v[q] * c[q];
+    vr += r.v[q] * c[q];
   }
-  const float du_l = 12.0f * kU * l.V, du_r = 12.0f * kU * r.V;  // absolute errors of ul, ur
+  const float ci = rsqrtf(s2), cn = s2 * ci, ul = vl * ci, ur = vr * ci;
   const float num = l.a + r.a - G.g * (ur - ul);
-  const float en = l.err * l.a + r.err * r.a + 10.0f * kU * (l.a + r.a + l.V + r.V);
-  const float iden = 1.0f / (l.az + r.az), ed = l.err + r.err + 8.0f * kU;
-  const float xlo = fmaxf(num - en, 0.0f) * iden * (1.0f - ed), xhi = fmaxf(num + en, 0.0f) * iden * (1.0f + ed);
-  const float Llo = log2f(xlo), Lhi = log2f(xhi);
-  const float elo = G.iz * (3.0f * kU * fabsf(Llo) + 2.0f * kU) + 8.0f * kU;
-  const float ehi = G.iz * (3.0f * kU * fabsf(Lhi) + 2.0f * kU) + 8.0f * kU;
-  const float plo = xlo > 0.0f ? exp2f(G.iz * Llo) * (1.0f - fminf(elo, 1.0f)) : 0.0f;
-  const float phi = xhi > 0.0f ? exp2f(G.iz * Lhi) * (1.0f + ehi) : 0.0f;
-  const float fl = l.err + 4.0f * kU, fr = r.err + 4.0f * kU;
-  const float ipl = 1.0f / l.p, ipr = 1.0f / r.p;
-  // s = sqrt(1 + k (p_tr / p - 1)_+), a s, and the two outer speeds
-  const float sll = sqrtf(1.0f + G.k * fmaxf(plo * ipl * (1.0f - fl) - 1.0f - 4.0f * kU, 0.0f));
-  const float slh = sqrtf(1.0f + G.k * fmaxf(phi * ipl * (1.0f + fl) - 1.0f + 4.0f * kU, 0.0f));
-  const float srl = sqrtf(1.0f + G.k * fmaxf(plo * ipr * (1.0f - fr) - 1.0f - 4.0f * kU, 0.0f));
-  const float srh = sqrtf(1.0f + G.k * fmaxf(phi * ipr * (1.0f + fr) - 1.0f + 4.0f * kU, 0.0f));
-  const float el = l.err + 12.0f * kU, er = r.err + 12.0f * kU;
-  const float alo = l.a * sll * (1.0f - el), ahi = l.a * slh * (1.0f + el);
-  const float blo = r.a * srl * (1.0f - er), bhi = r.a * srh * (1.0f + er);
-  const float lo = fmaxf(fmaxf(alo - ul - du_l - 4.0f * kU * alo, blo + ur - du_r - 4.0f * kU * blo), 0.0f);
-  const float hi = fmaxf(fmaxf(ahi - ul + du_l + 4.0f * kU * ahi, bhi + ur + du_r + 4.0f * kU * bhi), 0.0f);
-  *dlo = lo * cn * (1.0f - 8.0f * kU);
-  *dhi = hi * cn * (1.0f + 8.0f * kU);
-  return s2 > 1e-30f && s2 < 1e30f && phi < 1e30f && ehi < 0.1f && hi < 1e18f;
+  const float en = l.err * l.a + r.err * r.a + 10.0f * kU * (l.a + r.a + l.V + r.V);  // absolute
+  const float ed = l.err + r.err + 8.0f * kU;
+  float ptr = 0.0f, ep = 0.0f;  // p_tr and its relative error
+  bool ok = s2 > 1e-30f && s2 < 1e30f;
+  if (num > -en) {
+    const float x = __fdividef(fmaxf(num, en), l.az + r.az);
+    const float ex = __fdividef(en, fmaxf(num, en)) + ed + 4.0f * kU;
+    if (G.gamma75) {
+      const float x2 = x * x;
+      ptr = x2 * x2 * x2 * x;
+      ep = 7.0f * ex + 8.0f * kU;
+    } else {
+      const float lx = log2f(x);
+      ptr = exp2f(G.iz * lx);
+      ep = G.iz * (ex + 3.0f * kU * fabsf(lx) + 2.0f * kU) + 8.0f * kU;
+    }
+    // (a numerator within its error of 0: p_tr <= p on both sides only if the
+    // upper end is; the bound below then covers it or the row is undecided)
+    ep *= 1.1f;
+    ok = ok && ep < 0.05f && ptr < 1e30f;
+  }
+  const float ql = ptr * l.ip, qr = ptr * r.ip;
+  const float fl = ep + l.err + 4.0f * kU, fr = ep + r.err + 4.0f * kU;
+  const float sl = sqrtf(1.0f + G.k * fmaxf(ql - 1.0f, 0.0f)), sr = sqrtf(1.0f + G.k * fmaxf(qr - 1.0f, 0.0f));
+  // q (1 +- f) below 1 leaves s = 1 exactly
+  const float dl = ql * (1.0f + 2.0f * fl) > 1.0f ? fl : 0.0f, dr = qr * (1.0f + 2.0f * fr) > 1.0f ? fr : 0.0f;
+  const float wl = l.a * sl, wr = r.a * sr;
+  const float L = wl - ul, R = wr + ur;
+  const float eL = wl * (2.0f * dl + l.err + 16.0f * kU) + 16.0f * kU * l.V;
+  const float eR = wr * (2.0f * dr + r.err + 16.0f * kU) + 16.0f * kU * r.V;
+  const float lam = fmaxf(fmaxf(L, R), 0.0f);
+  *d = lam * cn;
+  *err = (fmaxf(eL, eR) + 8.0f * kU * lam) * cn * 1.01f;
+  return ok && lam < 1e18f;
 }
 
 template <int DIM> __device__ inline Bracket row_bracket(const Arrays &g, const Gas &G, int i) {
   const Bracket unknown{-INFINITY, INFINITY};
-  const NodeF<DIM> own = node_f32<DIM>(g, G.gamma, G.z, i);
-  bool ok = own.ok;
-  float slo = 0.0f, shi = 0.0f;
+  NodeF<DIM> own, w;
+  bool ok = node_f32<DIM>(g, G, i, own);
+  float sum = 0.0f, err = 0.0f;
   const int64_t k0 = g.row_ptr[i], k1 = g.row_ptr[i + 1];
   const bool bi = g.isb && g.isb[i];
   for (int64_t k = k0; k < k1; ++k) {
@@ -328,38 +363,39 @@ template <int DIM> __device__ inline Bracket row_bracket(const Arrays &g, const 
     if (j == i) continue;
     const bool both = bi && g.isb[j];
     const bool up = j > i;
-    const NodeF<DIM> w = node_f32<DIM>(g, G.gamma, G.z, j);
+    ok &= node_f32<DIM>(g, G, j, w);
     int64_t kt = k;
     if (!up || both) kt = transposed(g.row_ptr, g.col, i, j, k - k0);
     if (kt < 0) continue;
-    float c[DIM], lo, hi;
+    float c[DIM], d, e;
     // from min(i, j) to max(i, j) with the entry of row min(i, j); a pair of
     // boundary nodes also the other way round
 #pragma unroll
     for (int q = 0; q < DIM; ++q) c[q] = trunc_f32(g.cij[(int64_t)q * g.nnz + (up ? k : kt)]);
-    // (along +c from the left state; seen from node i of a lower entry the
-    // two sides swap)
-    ok &= w.ok && wave_f32<DIM>(G, up ? own : w, up ? w : own, c, 1.0f, &lo, &hi);
+    if (up) ok &= wave_f32<DIM>(G, own, w, c, &d, &e);
+    else ok &= wave_f32<DIM>(G, w, own, c, &d, &e);
     if (both) {
-      float lo2, hi2;
+      float d2, e2;
 #pragma unroll
       for (int q = 0; q < DIM; ++q) c[q] = trunc_f32(g.cij[(int64_t)q * g.nnz + (up ? kt : k)]);
-      ok &= wave_f32<DIM>(G, up ? w : own, up ? own : w, c, 1.0f, &lo2, &hi2);
-      lo = fmaxf(lo, lo2);
-      hi = fmaxf(hi, hi2);
+      if (up) ok &= wave_f32<DIM>(G, w, own, c, &d2, &e2);
+      else ok &= wave_f32<DIM>(G, own, w, c, &d2, &e2);
+      d = fmaxf(d, d2);
+      e = fmaxf(e, e2);
     }
-    slo += lo;
-    shi += hi;
+    sum += d;
+    err += e;
   }
   const float m = trunc_f32(g.mi[i]), e = ((float)(k1 - k0) + 16.0f) * kU;
-  if (!ok || !(m > 1e-30f && m < 1e30f && slo > 1e-30f && shi < 1e30f && e < 0.1f)) return unknown;
+  if (!ok || !(m > 1e-30f && m < 1e30f && sum > 1e-30f && sum < 1e30f && e < 0.1f && err < 0.5f * sum)) return unknown;
   const float t = 0.5f * (float)g.cfl * m;
-  const float lo = t / shi * (1.0f - e), hi = t / slo * (1.0f + e);
+  const float lo = t / (sum + err) * (1.0f - e), hi = t / (sum - err) * (1.0f + e);
   if (!(lo > 1e-30f && hi < 1e30f)) return unknown;
   return Bracket{lo, hi};
 }
 
-// the block's smallest lower and upper ends
+// the block's smallest lower end; the smallest upper end of all (positive
+// floats order like their bit patterns; the caller fills the slot with 0x7f)
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_cfl_bracket(Arrays g, Gas G, double *slots) {
   __shared__ float slo[kThreads / 32], shi[kThreads / 32];
@@ -382,91 +418,59 @@ __global__ void __launch_bounds__(kThreads) k_cfl_bracket(Arrays g, Gas G, doubl
       b.lo = fminf(b.lo, slo[q]);
       b.hi = fminf(b.hi, shi[q]);
     }
-    reinterpret_cast<float2 *>(slots)[blockIdx.x] = make_float2(b.lo, b.hi);
+    *reinterpret_cast<float *>(slots + blockIdx.x) = b.lo;
+    unsigned *limit = reinterpret_cast<unsigned *>(slots + kMaxBlocks);
+    if (b.hi < INFINITY && __float_as_uint(b.hi) < *(volatile unsigned *)limit) atomicMin(limit, __float_as_uint(b.hi));
+    if (blockIdx.x == 0) *reinterpret_cast<long long *>(slots + kMaxBlocks + 1) = bound_key(INFINITY);
   }
 }
 
-// the smallest upper end over all blocks, into the last slot
-__global__ void __launch_bounds__(1024) k_cfl_upper(double *slots, int nb) {
-  __shared__ float sm[32];
-  float b = INFINITY;
-  const float2 *s = reinterpret_cast<const float2 *>(slots);
-  for (int q = threadIdx.x; q < nb; q += blockDim.x) b = fminf(b, s[q].y);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) b = fminf(b, __shfl_xor_sync(0xffffffffu, b, off));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = b;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) b = fminf(b, sm[q]);
-    *reinterpret_cast<float *>(slots + kMaxBlocks) = b;
-  }
-}
-
-// the exact minimum over the block's rows that can hold the smallest bound (a
-// NaN for a row that is not admissible); +inf for a block without one. Few
-// such rows: a warp each, an entry per lane (a thread would run the serial
-// chain of a whole row, 9 entries of ~400 FP64 instructions at 63 cycles each);
-// many: a thread each, which leaves no lane idle.
+// the exact bounds of the block's rows that can be the smallest. Few such rows:
+// a warp each, an entry per lane (a thread would run the serial chain of a whole
+// row, 9 entries of ~100 to 400 FP64 instructions at 63 cycles each); many: a
+// thread each, which leaves no lane idle.
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_cfl_exact(Arrays g, Gas G, double *slots) {
-  __shared__ double smin[kThreads / 32];
   __shared__ int list[kThreads], count;
   const float limit = *reinterpret_cast<const float *>(slots + kMaxBlocks);
-  const float block_lo = reinterpret_cast<const float2 *>(slots)[blockIdx.x].x;
-  __syncthreads();  // the slot is read by every thread before it is rewritten
-  if (block_lo > limit) {
-    if (threadIdx.x == 0) slots[blockIdx.x] = INFINITY;
-    return;
-  }
+  if (*reinterpret_cast<const float *>(slots + blockIdx.x) > limit) return;
   if (threadIdx.x == 0) count = 0;
   __syncthreads();
   const int i = blockIdx.x * kThreads + threadIdx.x;
   if (i < g.n && row_bracket<DIM>(g, G, i).lo <= limit) list[atomicAdd(&count, 1)] = i;
   __syncthreads();
   const int rows = count;
-  double bound = INFINITY;
+  long long key = bound_key(INFINITY);
   if (rows <= kThreads / 8) {
-    for (int q = threadIdx.x >> 5; q < rows; q += kThreads / 32) bound = nan_min(bound, row_bound_warp<DIM>(g, list[q]));
+    for (int q = threadIdx.x >> 5; q < rows; q += kThreads / 32) {
+      const long long b = bound_key(row_bound_warp<DIM>(g, list[q]));
+      key = b < key ? b : key;
+    }
   } else if ((int)threadIdx.x < rows) {
-    bound = row_bound<DIM>(g, list[threadIdx.x]);
+    key = bound_key(row_bound<DIM>(g, list[threadIdx.x]));
   }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) bound = nan_min(bound, __shfl_xor_sync(0xffffffffu, bound, off));
-  if ((threadIdx.x & 31) == 0) smin[threadIdx.x >> 5] = bound;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = smin[0];
-#pragma unroll
-    for (int q = 1; q < kThreads / 32; ++q) b = nan_min(b, smin[q]);
-    slots[blockIdx.x] = b;
+  for (int off = 16; off > 0; off >>= 1) {
+    const long long o = __shfl_xor_sync(0xffffffffu, key, off);
+    key = o < key ? o : key;
   }
+  if ((threadIdx.x & 31) == 0) atomicMin(reinterpret_cast<long long *>(slots + kMaxBlocks + 1), key);
 }
 
-__global__ void __launch_bounds__(1024) k_cfl_reduce(const double *block_min, int nb, double *dt_out) {
-  __shared__ double sm[32];
-  double b = INFINITY;
-  for (int q = threadIdx.x; q < nb; q += blockDim.x) b = nan_min(b, block_min[q]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) b = nan_min(b, __shfl_xor_sync(0xffffffffu, b, off));
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = b;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double m = sm[0];
-    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) m = nan_min(m, sm[q]);
-    *dt_out = m;
-  }
+__global__ void k_cfl_store(const double *slots, double *dt_out) {
+  *dt_out = key_bound(*reinterpret_cast<const long long *>(slots + kMaxBlocks + 1));
 }
 
 template <int DIM> cudaError_t launch_cfl(const Arrays &g, const Gas &G, double *slots, double *dt_out, cudaStream_t s) {
   const int nb = (g.n + kThreads - 1) / kThreads;
   cudaError_t e;
+  // 0x7f7f7f7f: an FP32 value above every finite upper end
+  if ((e = cudaMemsetAsync(slots + kMaxBlocks, 0x7f, sizeof(double), s)) != cudaSuccess) return e;
   k_cfl_bracket<DIM><<<nb, kThreads, 0, s>>>(g, G, slots);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_cfl_upper<<<1, 1024, 0, s>>>(slots, nb);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_cfl_exact<DIM><<<nb, kThreads, 0, s>>>(g, G, slots);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_cfl_reduce<<<1, 1024, 0, s>>>(slots, nb, dt_out);
+  k_cfl_store<<<1, 1, 0, s>>>(slots, dt_out);
   return cudaGetLastError();
 }
 
@@ -545,8 +549,8 @@ extern "C" eh_status eh_cfl_dt_noalloc(int32_t dim, double gamma, double cfl, in
   eh_status st = scratch_for_current_device(&scratch);
   if (st != EH_OK) return st;
   const Arrays g{n, nnz, row_ptr, col, cij, mi, is_boundary, U, gamma, cfl};
-  const Gas G{(float)gamma, (float)(0.5 * (gamma - 1.0)), (float)((gamma - 1.0) / (2.0 * gamma)),
-              (float)(2.0 * gamma / (gamma - 1.0)), (float)((gamma + 1.0) / (2.0 * gamma))};
+  const Gas G{(float)gamma, (float)(gamma - 1.0), (float)(0.5 * (gamma - 1.0)), (float)((gamma - 1.0) / (2.0 * gamma)),
+              (float)(2.0 * gamma / (gamma - 1.0)), (float)((gamma + 1.0) / (2.0 * gamma)), gamma == 1.4};
   // (an error here is this call's only: none was pending)
   const cudaError_t e = dim == 2 ? launch_cfl<2>(g, G, scratch, dt_out, (cudaStream_t)stream)
                                  : launch_cfl<3>(g, G, scratch, dt_out, (cudaStream_t)stream);

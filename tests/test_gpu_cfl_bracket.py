@@ -34,7 +34,7 @@ def _states(mesh, gamma):
     yield "large units", W.conserved(1e38 * (1.0 + hat), [1e9 * noise[1]] + zero, 1e55 * (1.0 + hat), gamma)
 
 
-@pytest.mark.parametrize("gamma", [1.4, 1.05, 5.0 / 3.0])
+@pytest.mark.parametrize("gamma", [1.4, 1.05, 1.001, 5.0 / 3.0])
 @pytest.mark.parametrize("kind", ["q1", "p1", "hex", "flat"])
 def test_bracketed_step_is_the_contexts(kind, gamma):
     torch = pytest.importorskip("torch")
