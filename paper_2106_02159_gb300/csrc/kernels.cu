@@ -2014,6 +2014,34 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     return;
   }
   const bool one_i = lone_in[i] != 0;
+  if (one_i && !lsym_trace) {
+    // a row whose limiters, and whose neighbours' limiters, are all 1 (most
+    // rows): no limiter is gathered, and nothing is left of P_ij -- the row is
+    // marked spent, its rem entries are neither written nor read again
+    bool all = true;
+    for (int64_t k = k0; k < k1; ++k) all &= lone_in[m.col[k]] != 0;
+    if (all) {
+      const bool before = slot > 1 && w.spent[i];
+      for (int64_t k = k0; k < k1 && !before; ++k) {
+        if (m.col[k] == i) continue;
+        double P[S];
+        load_vec<DIM>(w.P + k * SP, P);
+        if (slot > 1) {
+          const double r = w.rem[k];
+          if (dbits(r) == 0) continue;
+#pragma unroll
+          for (int s = 0; s < S; ++s) P[s] = r * P[s];
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) u[s] += lambda_i * P[s];  // l = 1
+      }
+      store_vec<DIM>(Uout + (int64_t)i * SP, u);
+      lone_out[i] = 1;
+      w.spent[i] = 1;
+      return;
+    }
+  }
+  const bool spent = slot > 1 && w.spent[i];  // nothing is left already: rem is not there to be read
   // slot = the pass (1, 2, ...): pass 1 starts from k_lim1's P_ij, a later
   // pass from the remainder rem[k] P[k] that the previous one left
   for (int64_t k = k0; k < k1; ++k) {
@@ -2029,7 +2057,7 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     double *Pk = w.P + k * SP;
     double P[S];
     if (slot > 1) {
-      const double r = w.rem[k];
+      const double r = spent ? 0.0 : w.rem[k];
       if (dbits(r) == 0) continue;  // nothing left of P_ij (rem stays 0)
 #pragma unroll
       for (int s = 0; s < S; ++s) P[s] = r * Pk[s];
@@ -2045,14 +2073,22 @@ __device__ __forceinline__ void pass_row(const MeshView &m, const Params &p, con
     w.rem[k] = 1.0 - l;
   }
   store_vec<DIM>(Uout + (int64_t)i * SP, u);
+  if (spent) {
+    lone_out[i] = 1;
+    return;
+  }
+  w.spent[i] = 0;
   bool long_deferred = false;
   const uint64_t defer = pass_search<DIM, 1>(m, p, w, u, lout, slot, i, 0, long_deferred);
   lim_finish<1>(m, w, lone_out, lout, slot, i, 0, defer, defer == 0 && !long_deferred);
 }
 
-// (bound by the latency of the limiters' gathers: at most 64 registers, so that
-// 1024 rows are in flight per SM; the pre-decision's second level alone would
-// take 92, with k_pass 142 -> 174 us on the 998k cylinder)
+// Bound by the latency of the limiters' gathers and by its reads of P: at most 64
+// registers, so that 1024 rows are in flight per SM (the pre-decision's second
+// level alone would take 92, with 142 -> 174 us on the 998k cylinder); 142 -> 107
+// us with the spent rows. Listing the rows that need a limiter, so that the
+// others run beside the queued searches on a second stream, measured the same
+// step time (5.17 against 5.19 ms) and slowed meshes below 0.4M rows.
 template <int DIM>
 __global__ void __launch_bounds__(TPB_MAX, 4) k_pass(MeshView m, Params p, Work w, const double *__restrict__ Uin,
                                               double *__restrict__ Uout, const double *__restrict__ lin,
@@ -2119,6 +2155,7 @@ __global__ void __launch_bounds__(32 * PARTS) k_pass_split(MeshView m, Params p,
   if (in && part == 0) store_vec<DIM>(Uout + (int64_t)i * SP, u);
   bool long_deferred = false;
   uint64_t defer = 0;
+  if (rough && part == 0) w.spent[i] = 0;
   if (rough) defer = pass_search<DIM, PARTS>(m, p, w, u, lout, 1, i, part, long_deferred);
   if (defer != 0 || long_deferred) queued[lane] = 1;
   __syncthreads();
@@ -2444,8 +2481,21 @@ __device__ __forceinline__ void apply_bc_node(const MeshView &m, const Params &p
   }
 }
 
+// rho > 0 and E - |m|^2/(2 rho) > 0; the division only where FP32 does not show
+// rho E - |m|^2/2 to be positive with a margin of 1e-5 rho E (its roundings: 12 x 2^-23)
 template <int DIM>
 __device__ __forceinline__ bool admissible(const double *u) {
+  {
+    const float r = trunc_f32(u[0]), e = trunc_f32(u[DIM + 1]);
+    float m2 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < DIM; ++q) {
+      const float mq = trunc_f32(u[1 + q]);
+      m2 += mq * mq;
+    }
+    const float re = r * e;
+    if (r > 1e-15f && r < 1e15f && e > 1e-15f && e < 1e15f && re - 0.5f * m2 > 1e-5f * re) return true;
+  }
   double m2 = 0.0;
 #pragma unroll
   for (int q = 0; q < DIM; ++q) m2 += u[1 + q] * u[1 + q];
@@ -2463,24 +2513,43 @@ __device__ __forceinline__ void final_row(const MeshView &m, const Params &p, co
   double u[S];
   load_vec<DIM>(Uin + (int64_t)i * SP, u);
   const unsigned char *lone = w.lone + (int64_t)((p.limiter_passes - 1) & 1) * m.n;  // of the last pass
-  if (w.rough2[i] && p.limiter_passes >= 2) {
+  if (w.rough2[i] && p.limiter_passes >= 2 && w.spent[i] && !lsym_trace) {
+    // nothing is left of P_ij
+  } else if (w.rough2[i] && p.limiter_passes >= 2) {
     // the remainder rem P that the last k_pass left: where rem = 0 (most
     // entries) the update adds nothing, and the symmetrised limiter -- a
-    // dependent gather of the transposed one -- is not needed
-    for (int64_t k = k0; k < k1; ++k) {
-      if (m.col[k] == i) {
-        if (lsym_trace) lsym_trace[k] = 1.0;
-        continue;
-      }
-      const double r = w.rem[k];
-      if (dbits(r) == 0 && !lsym_trace) continue;
-      const int j = m.col[k];
-      const double l = lmin(lone[i] ? 1.0 : lin[k], lone[j] ? 1.0 : lin[m.tr[k]]);
-      if (lsym_trace) lsym_trace[k] = l;
-      if (dbits(r) == 0) continue;
-      const double *Pk = w.P + k * SP;
+    // dependent gather of the transposed one -- is not needed. Four entries at a
+    // time, so that their loads overlap (with the admissibility test's division
+    // left out and the spent rows, k_final 71 -> 47 us on the 998k cylinder, 257 ->
+    // 194 us at 4.0M vertices).
+    const bool one_i = lone[i] != 0, spent = w.spent[i] != 0;
+    for (int64_t kb = k0; kb < k1; kb += 4) {
+      double r[4], l[4];
+      int c[4], t[4];
+      bool need[4];
 #pragma unroll
-      for (int s = 0; s < S; ++s) u[s] += lambda_i * l * (r * Pk[s]);
+      for (int q = 0; q < 4; ++q) {
+        c[q] = kb + q < k1 ? m.col[kb + q] : i;
+        r[q] = kb + q < k1 && !spent ? w.rem[kb + q] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        need[q] = c[q] != i && (lsym_trace || dbits(r[q]) != 0);
+        t[q] = need[q] ? m.tr[kb + q] : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        l[q] = need[q] ? lmin(one_i ? 1.0 : lin[kb + q], lone[c[q]] ? 1.0 : lin[t[q]]) : 1.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (kb + q >= k1) break;
+        if (lsym_trace) lsym_trace[kb + q] = l[q];
+        if (!need[q] || dbits(r[q]) == 0) continue;
+        double P[S];
+        load_vec<DIM>(w.P + (kb + q) * SP, P);
+#pragma unroll
+        for (int s = 0; s < S; ++s) u[s] += lambda_i * l[q] * (r[q] * P[s]);
+      }
     }
   } else if (w.rough2[i]) {  // else every P_ij is 0 (see lim1_row) and the update adds nothing
     for (int64_t kb = k0; kb < k1; kb += LCHUNK) {

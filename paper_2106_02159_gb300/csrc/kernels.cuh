@@ -132,6 +132,10 @@ struct Work {
   // k_pass of pass p (q = p & 1), read by the next pass, which then needs no
   // gather of the transposed limiter for an entry between two such rows
   unsigned char *lone;    // [2][n]
+  // spent[i] = 1 when a limiter pass left nothing of row i's P_ij (every limiter
+  // of the row and its neighbours was 1; written by k_pass for rows with
+  // rough2 = 1): rem is not written for such a row
+  unsigned char *spent;   // [n]
   double *w;       // [nnz][SP]  (f(U_j) - f(U_i)) c_ij
   double *inc;     // [n][SP]    sum_{j != i} d_ij (U_j - U_i) - w_ij
   double *FH;      // [n][SP]    F^H_i / m_i
