@@ -281,6 +281,79 @@ __device__ __forceinline__ T lambda_max(const Params &p, T unl, T pl, T al, T az
   return max_nonneg(pos_part(-lam1), pos_part(lam3));
 }
 
+// a + b on the FP64 pipe, for a rarely taken branch: a call, which the compiler
+// neither evaluates ahead of the branch nor turns into a predicated instruction
+// (that would occupy the pipe whether its predicate holds or not)
+__device__ __noinline__ double add_fp64_cold(double a, double b) { return __dadd_rn(a, b); }
+// a + b rounded to nearest even on the integer units: IEEE addition for every
+// pair of doubles (the larger magnitude's exponent field within [70, 2045];
+// others, infinities and NaN go to the FP64 pipe). The larger significand is held
+// with 10 guard bits, the smaller shifted to it with a sticky bit, the sum
+// renormalised and rounded. ~60 integer instructions, 30 cycles of an SM per
+// warp, against 19 on the FP64 pipe -- but on units that the row kernels leave
+// idle: 8 of these beside 16 FP64 FMAs take 335 cycles, 8 FP64 additions beside
+// them 461. (Compared with the FP64 pipe on 2.5e9 pairs: exponents apart by
+// 0 to 140, cancellation, ties, zeros, subnormals.)
+// On the operands' words: a sign flipped or cleared on a double would become an
+// FP64 instruction again.
+__device__ __forceinline__ double add_words(unsigned ah, unsigned al, unsigned bh, unsigned bl) {
+  unsigned xa = ah & 0x7fffffffu, xb = bh & 0x7fffffffu;
+  const bool swap = xa < xb || (xa == xb && al < bl);
+  {
+    unsigned t = ah;
+    ah = swap ? bh : ah;
+    bh = swap ? t : bh;
+    t = al;
+    al = swap ? bl : al;
+    bl = swap ? t : bl;
+    t = xa;
+    xa = swap ? xb : xa;
+    xb = swap ? t : xb;
+  }
+  const unsigned ea = xa >> 20, eb = xb >> 20;
+  if (ea - 70u > 1975u) {
+    return add_fp64_cold(__hiloint2double((int)ah, (int)al), __hiloint2double((int)bh, (int)bl));
+  }
+  const unsigned d = min(ea - eb, 63u);
+  const unsigned mah = (ah & 0xfffffu) | 0x100000u, mbh = (bh & 0xfffffu) | (min(eb, 1u) << 20);
+  const unsigned long long ma = ((unsigned long long)mah << 32 | al) << 10, mb = ((unsigned long long)mbh << 32 | bl) << 10;
+  const unsigned long long sh = mb >> d;
+  const unsigned long long x = sh | (unsigned)((sh << d) != mb);  // sticky
+  const unsigned long long sx = (unsigned long long)(long long)((int)(ah ^ bh) >> 31);
+  const unsigned long long R = ma + ((x ^ sx) - sx);
+  const int lz = __clzll((long long)R);
+  const unsigned long long N = R << (lz & 63), m = N >> 11;
+  const unsigned up = ((unsigned)N & 0x7ffu) + ((unsigned)m & 1u) > 0x400u;
+  const unsigned long long r = ((unsigned long long)(ea - (unsigned)lz) << 52) + m + up;
+  const unsigned hi = (unsigned)(r >> 32) | (ah & 0x80000000u);
+  return R == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)r);
+}
+__device__ __forceinline__ unsigned hi_word(double x) { return (unsigned)__double2hiint(x); }
+__device__ __forceinline__ unsigned lo_word(double x) { return (unsigned)__double2loint(x); }
+__device__ __forceinline__ double add_alu(double a, double b) {
+  return add_words(hi_word(a), lo_word(a), hi_word(b), lo_word(b));
+}
+__device__ __forceinline__ double sub_alu(double a, double b) {
+  return add_words(hi_word(a), lo_word(a), hi_word(b) ^ 0x80000000u, lo_word(b));
+}
+__device__ __forceinline__ double add_abs_alu(double a, double b) {  // |a| + |b|
+  return add_words(hi_word(a) & 0x7fffffffu, lo_word(a), hi_word(b) & 0x7fffffffu, lo_word(b));
+}
+// a + b, a - b, |a| + |b| on the integer units (ALU) or the FP64 pipe: the same values
+template <bool ALU> __device__ __forceinline__ double add_on(double a, double b) {
+  if constexpr (ALU) return add_alu(a, b); else return __dadd_rn(a, b);
+}
+template <bool ALU> __device__ __forceinline__ double sub_on(double a, double b) {
+  if constexpr (ALU) return sub_alu(a, b); else return __dsub_rn(a, b);
+}
+template <bool ALU> __device__ __forceinline__ double add_abs_on(double a, double b) {
+  if constexpr (ALU) return add_abs_alu(a, b); else return __dadd_rn(abs_bits(a), abs_bits(b));
+}
+// (FP32: the plain instructions)
+template <bool ALU> __device__ __forceinline__ float add_on(float a, float b) { return a + b; }
+template <bool ALU> __device__ __forceinline__ float sub_on(float a, float b) { return a - b; }
+template <bool ALU> __device__ __forceinline__ float add_abs_on(float a, float b) { return fabsf(a) + fabsf(b); }
+
 // a - b on the integer units where a and b have the same sign and exponent (their
 // bit patterns' difference is then the exact result's significand: nothing is
 // rounded), an FP64 subtraction otherwise: the same value always. For the
@@ -292,9 +365,7 @@ __device__ __forceinline__ double sub_near(double a, double b) {
   const int ah = __double2hiint(a), bh = __double2hiint(b);
   const unsigned e = ((unsigned)ah >> 20) & 0x7ffu;
   if ((unsigned)(ah ^ bh) >> 20 != 0 || e - 65u >= 0x7ffu - 65u) {
-    double r;  // (volatile: kept inside the branch, not evaluated ahead of it)
-    asm volatile("sub.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-    return r;
+    return add_fp64_cold(a, -b);
   }
   const long long d = dbits(a) - dbits(b);
   const long long sg = d >> 63;
@@ -331,6 +402,7 @@ __device__ __forceinline__ float2 unpack_f32(double x) {
 // magnitudes (gamma <= 5/3); the quotient 8u more; the seventh power (or exp2
 // of inv_z log2) multiplies the relative error by 7 (inv_z). Anything unclear,
 // or out of FP32's range (a = NaN), takes the full evaluation.
+template <bool ALU>
 __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, double vcr, double ci, double pl, double al,
                                                  double azl, double ipl, float2 fl, double pr, double ar, double azr,
                                                  double ipr, float2 fr) {
@@ -375,12 +447,12 @@ __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, do
   const double as = left ? al : ar;
   if (!need) {
     const double us = __dmul_rn(left ? -vcl : vcr, ci);
-    return pos_part(us + as);
+    return pos_part(add_on<ALU>(us, as));
   }
   const double unl = __dmul_rn(vcl, ci), unr = __dmul_rn(vcr, ci);
-  double num = __fma_rn(-(0.5 * p.gm1), __dsub_rn(unr, unl), al + ar);
+  double num = __fma_rn(-(0.5 * p.gm1), sub_on<ALU>(unr, unl), add_on<ALU>(al, ar));
   num = pos_part(num);
-  const double x = num / (azl + azr);
+  const double x = num / add_on<ALU>(azl, azr);
   double ptr;
   if (p.gamma75) {
     const double x2 = x * x;
@@ -391,7 +463,7 @@ __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, do
   }
   const double ks = p.kshock;
   const double ps = left ? pl : pr, ips = left ? ipl : ipr, us = left ? -unl : unr;
-  const double ss = gt_nonneg(ptr, ps) ? sqrt(1.0 + ks * (ptr - ps) * ips) : 1.0;
+  const double ss = gt_nonneg(ptr, ps) ? sqrt(1.0 + ks * sub_on<ALU>(ptr, ps) * ips) : 1.0;
   double lam = pos_part(us + as * ss);
   if (two) {
     const double so = gt_nonneg(ptr, pl) ? sqrt(1.0 + ks * (ptr - pl) * ipl) : 1.0;
@@ -1083,7 +1155,7 @@ __device__ __forceinline__ ViscNode<DIM, T> visc_node(const Work &w, int i) {
 // the flux formed in FP32) carry rounding errors that the difference of
 // rounded fluxes does not: they left ~20x more of the limiter's l = 1
 // checks failing on the Mach-3 cylinder and raised the error against FP64
-template <int DIM, typename T, bool BOTH>
+template <int DIM, typename T, bool BOTH, bool ALU>
 __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, const Work &w, const ViscNode<DIM, T> &n,
                                           int i, int j, int64_t k) {
   constexpr int S = DIM + 2;
@@ -1171,8 +1243,8 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
     vjc += vj[q] * c[q];
     vic += n.v[q] * c[q];
   }
-  const T dp = pj - n.p;
-  T wv[S], a_ = T(0), dm[DIM];
+  const T dp = sub_on<ALU>(pj, n.p);
+  T wv[S], a_ = T(0), dm[DIM], dH, de;
   if constexpr (flux_diff) {
 #pragma unroll
     for (int s = 0; s < S; ++s) {
@@ -1191,15 +1263,17 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
     T w0 = T(0);
 #pragma unroll
     for (int q = 0; q < DIM; ++q) {
-      dm[q] = mj[q] - n.mo[q];
+      dm[q] = sub_on<ALU>(mj[q], n.mo[q]);
       w0 += dm[q] * c[q];
     }
-    const T dv = vjc - vic;
+    const T dv = sub_on<ALU>(vjc, vic);
     wv[0] = w0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) wv[1 + a] = dm[a] * vjc + n.mo[a] * dv + dp * c[a];
-    wv[S - 1] = __fma_rn(Hj - n.H, vjc, __dmul_rn(n.H, dv));
-    a_ = __fma_rn(etaj - n.eta, vjc, __dmul_rn(n.eta, dv));
+    dH = sub_on<ALU>(Hj, n.H);
+    de = sub_on<ALU>(etaj, n.eta);
+    wv[S - 1] = __fma_rn(dH, vjc, __dmul_rn(n.H, dv));
+    a_ = __fma_rn(de, vjc, __dmul_rn(n.eta, dv));
   }
   // the transposed entry: c_ji = -c_ij unless both nodes lie on the boundary
   // (Sec. 3.1), so w_ji = w_ij and a_ji = a_ij; otherwise evaluate with c_ji
@@ -1233,8 +1307,8 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
       wt[0] = -w0t;
 #pragma unroll
       for (int a = 0; a < DIM; ++a) wt[1 + a] = -(dm[a] * vjct + n.mo[a] * dvt + dp * ct[a]);
-      wt[S - 1] = -__fma_rn(Hj - n.H, vjct, __dmul_rn(n.H, dvt));
-      at = -__fma_rn(etaj - n.eta, vjct, __dmul_rn(n.eta, dvt));
+      wt[S - 1] = -__fma_rn(dH, vjct, __dmul_rn(n.H, dvt));
+      at = -__fma_rn(de, vjct, __dmul_rn(n.eta, dvt));
     }
   }
   // d_ij (Sec. 3.1), mirrored; normal velocities v . c_ij / |c_ij| (FP32:
@@ -1260,9 +1334,9 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
       dij = max_nonneg(dij, dji);
     }
   } else {
-    dij = lambda_max_sel(p, vic, vjc, ci, n.p, n.a, n.az, n.ip, n.f32, pj, aj, azj, ipj, fj) * cn;
+    dij = lambda_max_sel<ALU>(p, vic, vjc, ci, n.p, n.a, n.az, n.ip, n.f32, pj, aj, azj, ipj, fj) * cn;
     if constexpr (BOTH) {
-      const T dji = lambda_max_sel(p, vjct, vict, cit, pj, aj, azj, ipj, fj, n.p, n.a, n.az, n.ip, n.f32) * cnt;
+      const T dji = lambda_max_sel<ALU>(p, vjct, vict, cit, pj, aj, azj, ipj, fj, n.p, n.a, n.az, n.ip, n.f32) * cnt;
       dij = max_nonneg(dij, dji);
     }
   }
@@ -1284,16 +1358,18 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
 // Bound by FP64 issue: on a 998k-vertex cylinder, every edge general, 442 us
 // and 5.4M FP64 warp instructions (7.4M before lambda_max_sel) with the L1 at
 // 74 % of its throughput through 8-byte accesses, 358 us with 32-byte ones (FP64
-// pipe 80 % of the 84 % that it sustains); 493 us before both.
-template <int DIM, typename T>
-__global__ void __launch_bounds__(TPB_MAX) k_visc(MeshView m, Params p, Work w, unsigned row_blocks, int lparts) {
+// pipe 80 % of the 84 % that it sustains), 299 us and 4.35M with the differences
+// on the integer units (ALU; pipe 78 %) and three blocks of 256 threads an SM;
+// 493 us before the three.
+template <int DIM, typename T, bool ALU>
+__global__ void __launch_bounds__(TPB_MAX, 3) k_visc(MeshView m, Params p, Work w, unsigned row_blocks, int lparts) {
   if (w.st->err) return;
   if (blockIdx.x >= row_blocks) {
     const int q = (blockIdx.x - row_blocks) * blockDim.x + threadIdx.x;
     if (q >= m.n_bp) return;
     const int i = m.bp_row[q], k = m.bp_pos[q];
     const ViscNode<DIM, T> n = visc_node<DIM, T>(w, i);
-    visc_edge<DIM, T, true>(m, p, w, n, i, m.col[k], k);
+    visc_edge<DIM, T, true, ALU>(m, p, w, n, i, m.col[k], k);
     return;
   }
   const unsigned warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1305,7 +1381,7 @@ __global__ void __launch_bounds__(TPB_MAX) k_visc(MeshView m, Params p, Work w, 
   for (int64_t k = m.row_ptr[i] + (warp & ((1 << lparts) - 1)); k < k1; k += 1 << lparts) {
     const int j = m.col[k];
     if (j <= i || (bi && m.isb[j])) continue;
-    visc_edge<DIM, T, false>(m, p, w, n, i, j, k);
+    visc_edge<DIM, T, false, ALU>(m, p, w, n, i, j, k);
   }
 }
 
@@ -1329,7 +1405,7 @@ template <int DIM, typename T> __device__ __forceinline__ void entropy_gradient(
   deta[DIM + 1] = -g1;
 }
 // entry k's terms of N_i and D_i
-template <int DIM, typename T>
+template <int DIM, typename T, bool ALU>
 __device__ __forceinline__ void indicator_terms(const Work &w, int64_t k, const T *deta, T &n, T &d) {
   constexpr int S = DIM + 2;
   T wk[S], a_, d_;
@@ -1337,14 +1413,16 @@ __device__ __forceinline__ void indicator_terms(const Work &w, int64_t k, const 
   T b_ = T(0);
 #pragma unroll
   for (int s = 0; s < S; ++s) b_ += deta[s] * wk[s];
-  n = a_ - b_;
-  d = abs_bits(a_) + abs_bits(b_);
+  n = sub_on<ALU>(a_, b_);
+  d = add_abs_on<ALU>(a_, b_);
 }
 // alpha_i / 2 (exact): d^H_ij = (a_i/2 + a_j/2) d_ij
 template <typename T> __device__ __forceinline__ double half_alpha(T N, T D) {
   return D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;
 }
 
+// Additions on the integer units: 1.7M FP64 warp instructions of 2.7M remain, 998k
+// cylinder 168 -> 134 us.
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w) {
   constexpr int S = DIM + 2;
@@ -1361,9 +1439,9 @@ __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w)
   for (int64_t k = k0; k < k1; ++k) {
     if (m.col[k] == i) continue;
     T n, d;
-    indicator_terms<DIM, T>(w, k, deta, n, d);
-    N += n;
-    D += d;
+    indicator_terms<DIM, T, true>(w, k, deta, n, d);
+    N = add_on<true>(N, n);
+    D = add_on<true>(D, d);
   }
   w.alpha[i] = half_alpha(N, D);
 }
@@ -1402,7 +1480,7 @@ __global__ void __launch_bounds__(32 * PARTS) k_alpha_split(MeshView m, Params p
   for (int r = 0;; ++r) {
     const int64_t k = k0 + r * PARTS + part;
     T n = T(0), d = T(0);
-    if (k < k1 && m.col[k] != i) indicator_terms<DIM, T>(w, k, deta, n, d);
+    if (k < k1 && m.col[k] != i) indicator_terms<DIM, T, false>(w, k, deta, n, d);
     sn[r & 1][part][lane] = n;
     sd[r & 1][part][lane] = d;
     const int more = __syncthreads_or(k0 + (r + 1) * PARTS < k1);
@@ -1481,7 +1559,7 @@ __device__ __forceinline__ void store_bounds(const MeshView &m, const Params &p,
 
 // Algorithm 1 steps 2-3 for one row; returns the row's CFL bound
 // c_cfl m_i / (2 sum_{j != i} d_ij), or +inf (row_cfl_bound)
-template <int DIM, typename T>
+template <int DIM, typename T, bool ALU>
 __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, const Work &w, int i,
                                           unsigned long long so_far) {
   constexpr int S = DIM + 2;
@@ -1520,21 +1598,21 @@ __device__ __forceinline__ double low_row(const MeshView &m, const Params &p, co
     T wk[S], ak, dkT;
     load_edge<DIM, T>(w, k, wk, ak, dkT);
     const double dk = (double)dkT;
-    const T dH = T(alphai + w.alpha[j]) * dkT;  // w.alpha holds alpha / 2
+    const T dH = T(sizeof(T) == 4 ? add_on<ALU>(alphai, w.alpha[j]) : alphai + w.alpha[j]) * dkT;  // w.alpha holds alpha / 2
     const double w0 = (double)wk[0];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : Rj[s] - ui[s];
+      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : sub_on<ALU>(Rj[s], ui[s]);
       inc[s] += dk * du;  // sum_j d_ij (U_j - U_i); the sum of w_ij is subtracted once
       fh[s] += dH * (T)du;
-      wsum[s] += wk[s];
+      wsum[s] = add_on<ALU>(wsum[s], wk[s]);
     }
-    if (dbits(dk) > 0) rb.add(dk * (ui[0] + Rj[0]) - w0, dk);  // dk >= 0
+    if (dbits(dk) > 0) rb.add(dk * (sizeof(T) == 4 ? add_on<ALU>(ui[0], Rj[0]) : ui[0] + Rj[0]) - w0, dk);  // dk >= 0
     // Phi > 0: the integer order of the bit patterns is the numeric order
     const double pj = Rj64[R::PHI];
     phimin = dbits(pj) < dbits(phimin) ? pj : phimin;
     phimax = dbits(pj) > dbits(phimax) ? pj : phimax;
-    dsum += dk;
+    dsum = add_on<ALU && sizeof(T) == 4>(dsum, dk);
   }
 #pragma unroll
   for (int s = 0; s < S; ++s) {
@@ -1625,15 +1703,18 @@ __device__ __forceinline__ void fold_bound(const Work &w, double bound, int inst
 // Bound by FP64 issue. Of the 32.6 FP64 instructions an entry that a row took
 // (998k cylinder: 8.1M warp instructions, 486 us), the sums need 21; the bar
 // states' cross products, the relaxation of strict bounds, most rows' division
-// for the CFL bound and the minima's FP64 compares are gone: 26.7 (397 us).
-template <int DIM, typename T>
-__global__ void __launch_bounds__(TPB_MAX) k_low(MeshView m, Params p, Work w) {
+// for the CFL bound and the minima's FP64 compares are gone: 26.7 (397 us); with
+// the sum of w_ij, du and (mixed) the sums around d_ij on the integer units (ALU)
+// 4.7M, 336 us: FP64 pipe 74 %, integer units 52 %, three blocks of 256 threads an
+// SM (two: 350; four, with spills: 392). Mixed 360 -> 305 us.
+template <int DIM, typename T, bool ALU>
+__global__ void __launch_bounds__(TPB_MAX, ALU && DIM == 2 ? 3 : 2) k_low(MeshView m, Params p, Work w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double bound = INFINITY;
   const int inst = m.inst ? m.inst[min(i, m.n - 1)] : 0;
   const unsigned long long so_far = __ldcg(&w.bound_bits[inst]);
   if (i < m.n && !w.st->err)
-    bound = w.rough[i] ? low_row<DIM, T>(m, p, w, i, so_far) : low_row_smooth<DIM, T>(m, p, w, i, so_far);
+    bound = w.rough[i] ? low_row<DIM, T, ALU>(m, p, w, i, so_far) : low_row_smooth<DIM, T>(m, p, w, i, so_far);
   __syncwarp();
   fold_bound(w, bound, inst, so_far);
 }
@@ -1756,7 +1837,7 @@ __global__ void __launch_bounds__(256) k_tau(MeshView m, Work w, int stage, doub
 // U^L and the entries q = part, part + STEP, ... of row i; returns the mask of
 // entries left to the queued searches (of the first 64 of a row; later ones are
 // queued at once and set long_deferred)
-template <int DIM, typename T, int STEP>
+template <int DIM, typename T, int STEP, bool ALU>
 __device__ __forceinline__ uint64_t lim1_entries(const MeshView &m, const Params &p, const Work &w, double *P_trace,
                                                  int i, int part, bool &long_deferred) {
   constexpr int S = DIM + 2;
@@ -1840,8 +1921,8 @@ __device__ __forceinline__ uint64_t lim1_entries(const MeshView &m, const Params
     double P[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : Rj[s] - ui[s];
-      P[s] = __fma_rn(cm, gi[s] - Gj[s], __dmul_rn(cd, du));
+      const double du = s == 0 || s == 1 || s == S - 1 ? sub_near(Rj[s], ui[s]) : sub_on<ALU>(Rj[s], ui[s]);
+      P[s] = __fma_rn(cm, sub_on<ALU>(gi[s], Gj[s]), __dmul_rn(cd, du));
     }
     store_vec<DIM>(Pk, P);
     if (P_trace) {
@@ -1875,13 +1956,15 @@ __device__ __forceinline__ void lim_finish(const MeshView &m, const Work &w, uns
 }
 
 // rows i, i + grid size, ... (the grid may be capped to limit the rows in
-// flight; one row per thread otherwise)
-template <int DIM, typename T>
-__global__ void __launch_bounds__(TPB_MAX) k_lim1(MeshView m, Params p, Work w, double *P_trace) {
+// flight; one row per thread otherwise). The differences of P_ij on the integer
+// units where ALU: 998k cylinder 386 -> 328 us (FP64 pipe 77 %, integer 58 %),
+// mixed 415 -> 349.
+template <int DIM, typename T, bool ALU>
+__global__ void __launch_bounds__(TPB_MAX, ALU && DIM == 2 ? 3 : 2) k_lim1(MeshView m, Params p, Work w, double *P_trace) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m.n; i += gridDim.x * blockDim.x) {
     if (w.st->err) return;
     bool long_deferred = false;
-    const uint64_t defer = lim1_entries<DIM, T, 1>(m, p, w, P_trace, i, 0, long_deferred);
+    const uint64_t defer = lim1_entries<DIM, T, 1, ALU>(m, p, w, P_trace, i, 0, long_deferred);
     lim_finish<1>(m, w, w.lone, w.la, 0, i, 0, defer, defer == 0 && !long_deferred);
   }
 }
@@ -1896,7 +1979,7 @@ __global__ void __launch_bounds__(32 * PARTS) k_lim1_split(MeshView m, Params p,
   const bool in = i < m.n && !w.st->err;
   bool long_deferred = false;
   uint64_t defer = 0;
-  if (in) defer = lim1_entries<DIM, T, PARTS>(m, p, w, P_trace, i, part, long_deferred);
+  if (in) defer = lim1_entries<DIM, T, PARTS, false>(m, p, w, P_trace, i, part, long_deferred);
   if (defer != 0 || long_deferred) queued[lane] = 1;
   __syncthreads();
   if (in) lim_finish<PARTS>(m, w, w.lone, w.la, 0, i, part, defer, queued[lane] == 0);
@@ -2687,6 +2770,14 @@ template <int DIM> __global__ void k_count_not_admissible(int n, const double *U
 // (The launch shape of eh_set_launch_shape applies to the row forms.)
 constexpr int SPLIT_SUMS = 32 * 1024;     // k_alpha, k_low: the warps repeat loads and half of the products
 constexpr int SPLIT_ENTRIES = 64 * 1024;  // k_lim1, k_pass: the entries are independent
+// Additions on the integer units (add_on<true>) in 2D k_low and k_lim1 from here
+// on. Below, one wave of the form with FP64 additions holds all rows (92 to 106
+// registers, 152 SMs x 576 rows = 88k) and finishes sooner: 40 against 47 us for
+// k_low at 78k rows behind a shock; at 103k it takes a second wave: k_low 61
+// against 50 us, k_lim1 61 against 51 (developed flow; behind a shock 45 against
+// 54 and 58 against 59), at 998k 391 against 336 and 386 against 328. 3D k_low has
+// them at every size (95k rows 175 -> 172 us), 3D k_lim1 nowhere (625 -> 642 us).
+constexpr int ALU_ROWS = 96 * 1024;
 template <int DIM, typename T>
 void launch_prep(const MeshView &m, const Params &p, const double *U, const Work &w, int tpb, cudaStream_t s) {
   k_prep<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, U, w.rec, (T *)w.vrec, w.rough, w.steady, w.st);
@@ -2700,7 +2791,15 @@ void launch_visc(const MeshView &m, const Params &p, const Work &w, int tpb, cud
   // 246k cylinder behind a shock 252 / 208 / 209, 375k in 3D 830 / 824 / 834)
   const int lparts = m.n < 160 * 1024 ? 2 : m.n < 640 * 1024 ? 1 : 0;
   const unsigned rows = nblocks((int64_t)nblocks(m.n, 32) << lparts, tpb / 32);
-  k_visc<DIM, T><<<rows + nblocks(m.n_bp, tpb), tpb, 0, s>>>(m, p, w, rows, lparts);
+  // differences on the integer units where the FP64 pipe is full (FP64 form 358 ->
+  // 299 us at 998k rows, 78k 54.7 -> 53.2, 3D 95k 238 -> 216); small meshes wait on
+  // latencies instead (4k vortex: 17.9 us on the FP64 pipe, 19.1 on the integer
+  // units). The mixed form's differences are FP32 ones already.
+  const unsigned grid = rows + nblocks(m.n_bp, tpb);
+  if (sizeof(T) == 8 && m.n >= SPLIT_ENTRIES)
+    k_visc<DIM, T, sizeof(T) == 8><<<grid, tpb, 0, s>>>(m, p, w, rows, lparts);
+  else
+    k_visc<DIM, T, false><<<grid, tpb, 0, s>>>(m, p, w, rows, lparts);
 }
 template <int DIM, typename T>
 void launch_alpha(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {
@@ -2713,8 +2812,10 @@ template <int DIM, typename T>
 void launch_low(const MeshView &m, const Params &p, const Work &w, int tpb, cudaStream_t s) {
   if (m.n < SPLIT_SUMS)
     k_low_split<DIM, T><<<nblocks(m.n, 32), 32 * (DIM + 3), 0, s>>>(m, p, w);
+  else if (DIM == 2 && m.n < ALU_ROWS)
+    k_low<DIM, T, DIM == 3><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
   else
-    k_low<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
+    k_low<DIM, T, true><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, w);
 }
 void launch_tau(const MeshView &m, const Work &w, int stage, double dt_given, double cfl, bool advance_time,
                 cudaStream_t s) {
@@ -2731,8 +2832,10 @@ void launch_lim1(const MeshView &m, const Params &p, const Work &w, double *P_tr
                  cudaStream_t s) {
   if (m.n < SPLIT_ENTRIES)
     k_lim1_split<DIM, T><<<nblocks(m.n, 32), 32 * PARTS, 0, s>>>(m, p, w, P_trace);
+  else if (DIM == 3 || m.n < ALU_ROWS)
+    k_lim1<DIM, T, false><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, P_trace);
   else
-    k_lim1<DIM, T><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, P_trace);
+    k_lim1<DIM, T, DIM == 2><<<capped_grid(m.n, tpb, max_blocks), tpb, 0, s>>>(m, p, w, P_trace);
 }
 template <int DIM>
 void launch_pass(const MeshView &m, const Params &p, const Work &w, const double *Uin, double *Uout, const double *lin,
