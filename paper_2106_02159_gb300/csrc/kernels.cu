@@ -19,6 +19,7 @@
 // neighbours differs has P_ij = 0 and every limiter 1; a limiter pass leaves
 // its remainder (1 - l) P_ij as the factor 1 - l (nothing is read where it is
 // 0); a row whose limiters are all 1 stores none and says so in a flag.
+#include "integer_fp64.cuh"
 #include "kernels.cuh"
 
 #include <cooperative_groups.h>
@@ -281,64 +282,6 @@ __device__ __forceinline__ T lambda_max(const Params &p, T unl, T pl, T al, T az
   return max_nonneg(pos_part(-lam1), pos_part(lam3));
 }
 
-// a + b on the FP64 pipe, for a rarely taken branch: a call, which the compiler
-// neither evaluates ahead of the branch nor turns into a predicated instruction
-// (that would occupy the pipe whether its predicate holds or not)
-__device__ __noinline__ double add_fp64_cold(double a, double b) { return __dadd_rn(a, b); }
-// a + b rounded to nearest even on the integer units: IEEE addition for every
-// pair of doubles (the larger magnitude's exponent field within [70, 2045];
-// others, infinities and NaN go to the FP64 pipe). The larger significand is held
-// with 10 guard bits, the smaller shifted to it with a sticky bit, the sum
-// renormalised and rounded. ~60 integer instructions, 30 cycles of an SM per
-// warp, against 19 on the FP64 pipe -- but on units that the row kernels leave
-// idle: 8 of these beside 16 FP64 FMAs take 335 cycles, 8 FP64 additions beside
-// them 461. (Compared with the FP64 pipe on 2.5e9 pairs: exponents apart by
-// 0 to 140, cancellation, ties, zeros, subnormals.)
-// On the operands' words: a sign flipped or cleared on a double would become an
-// FP64 instruction again.
-__device__ __forceinline__ double add_words(unsigned ah, unsigned al, unsigned bh, unsigned bl) {
-  unsigned xa = ah & 0x7fffffffu, xb = bh & 0x7fffffffu;
-  const bool swap = xa < xb || (xa == xb && al < bl);
-  {
-    unsigned t = ah;
-    ah = swap ? bh : ah;
-    bh = swap ? t : bh;
-    t = al;
-    al = swap ? bl : al;
-    bl = swap ? t : bl;
-    t = xa;
-    xa = swap ? xb : xa;
-    xb = swap ? t : xb;
-  }
-  const unsigned ea = xa >> 20, eb = xb >> 20;
-  if (ea - 70u > 1975u) {
-    return add_fp64_cold(__hiloint2double((int)ah, (int)al), __hiloint2double((int)bh, (int)bl));
-  }
-  const unsigned d = min(ea - eb, 63u);
-  const unsigned mah = (ah & 0xfffffu) | 0x100000u, mbh = (bh & 0xfffffu) | (min(eb, 1u) << 20);
-  const unsigned long long ma = ((unsigned long long)mah << 32 | al) << 10, mb = ((unsigned long long)mbh << 32 | bl) << 10;
-  const unsigned long long sh = mb >> d;
-  const unsigned long long x = sh | (unsigned)((sh << d) != mb);  // sticky
-  const unsigned long long sx = (unsigned long long)(long long)((int)(ah ^ bh) >> 31);
-  const unsigned long long R = ma + ((x ^ sx) - sx);
-  const int lz = __clzll((long long)R);
-  const unsigned long long N = R << (lz & 63), m = N >> 11;
-  const unsigned up = ((unsigned)N & 0x7ffu) + ((unsigned)m & 1u) > 0x400u;
-  const unsigned long long r = ((unsigned long long)(ea - (unsigned)lz) << 52) + m + up;
-  const unsigned hi = (unsigned)(r >> 32) | (ah & 0x80000000u);
-  return R == 0 ? 0.0 : __hiloint2double((int)hi, (int)(unsigned)r);
-}
-__device__ __forceinline__ unsigned hi_word(double x) { return (unsigned)__double2hiint(x); }
-__device__ __forceinline__ unsigned lo_word(double x) { return (unsigned)__double2loint(x); }
-__device__ __forceinline__ double add_alu(double a, double b) {
-  return add_words(hi_word(a), lo_word(a), hi_word(b), lo_word(b));
-}
-__device__ __forceinline__ double sub_alu(double a, double b) {
-  return add_words(hi_word(a), lo_word(a), hi_word(b) ^ 0x80000000u, lo_word(b));
-}
-__device__ __forceinline__ double add_abs_alu(double a, double b) {  // |a| + |b|
-  return add_words(hi_word(a) & 0x7fffffffu, lo_word(a), hi_word(b) & 0x7fffffffu, lo_word(b));
-}
 // a + b, a - b, |a| + |b| on the integer units (ALU) or the FP64 pipe: the same values
 template <bool ALU> __device__ __forceinline__ double add_on(double a, double b) {
   if constexpr (ALU) return add_alu(a, b); else return __dadd_rn(a, b);
@@ -353,28 +296,6 @@ template <bool ALU> __device__ __forceinline__ double add_abs_on(double a, doubl
 template <bool ALU> __device__ __forceinline__ float add_on(float a, float b) { return a + b; }
 template <bool ALU> __device__ __forceinline__ float sub_on(float a, float b) { return a - b; }
 template <bool ALU> __device__ __forceinline__ float add_abs_on(float a, float b) { return fabsf(a) + fabsf(b); }
-
-// a - b on the integer units where a and b have the same sign and exponent (their
-// bit patterns' difference is then the exact result's significand: nothing is
-// rounded), an FP64 subtraction otherwise: the same value always. For the
-// differences of neighbouring densities, streamwise momenta and energies, which
-// rarely cross a power of two: ~26 integer instructions run beside the FP64
-// pipe instead of one of its 19-cycle slots (k_low 397 -> 386 us, k_lim1 419 ->
-// 391 us on the 998k cylinder; 609 -> 485 and 679 -> 634 us in 3D).
-__device__ __forceinline__ double sub_near(double a, double b) {
-  const int ah = __double2hiint(a), bh = __double2hiint(b);
-  const unsigned e = ((unsigned)ah >> 20) & 0x7ffu;
-  if ((unsigned)(ah ^ bh) >> 20 != 0 || e - 65u >= 0x7ffu - 65u) {
-    return add_fp64_cold(a, -b);
-  }
-  const long long d = dbits(a) - dbits(b);
-  const long long sg = d >> 63;
-  const unsigned long long m = (unsigned long long)((d ^ sg) - sg);
-  const int sh = __clzll((long long)m) - 11;
-  const unsigned long long r = ((unsigned long long)(e - 1 - sh) << 52) + (m << sh);
-  const unsigned long long sign = ((unsigned long long)sg ^ (unsigned long long)dbits(a)) & 0x8000000000000000ull;
-  return m == 0 ? 0.0 : __longlong_as_double((long long)(r | sign));
-}
 
 // a and p of a node as an FP32 pair in one FP64 slot of its record (Rec::F32),
 // for lambda_max_sel; a = NaN when a, p or a p^-z could leave FP32's range
@@ -452,7 +373,7 @@ __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, do
   const double unl = __dmul_rn(vcl, ci), unr = __dmul_rn(vcr, ci);
   double num = __fma_rn(-(0.5 * p.gm1), sub_on<ALU>(unr, unl), add_on<ALU>(al, ar));
   num = pos_part(num);
-  const double x = num / add_on<ALU>(azl, azr);
+  const double x = div_alu(num, add_on<ALU>(azl, azr));
   double ptr;
   if (p.gamma75) {
     const double x2 = x * x;
@@ -463,7 +384,7 @@ __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, do
   }
   const double ks = p.kshock;
   const double ps = left ? pl : pr, ips = left ? ipl : ipr, us = left ? -unl : unr;
-  const double ss = gt_nonneg(ptr, ps) ? sqrt(1.0 + ks * sub_on<ALU>(ptr, ps) * ips) : 1.0;
+  const double ss = gt_nonneg(ptr, ps) ? sqrt_alu(1.0 + ks * sub_on<ALU>(ptr, ps) * ips) : 1.0;
   double lam = pos_part(us + as * ss);
   if (two) {
     const double so = gt_nonneg(ptr, pl) ? sqrt(1.0 + ks * (ptr - pl) * ipl) : 1.0;
@@ -520,7 +441,7 @@ __device__ __forceinline__ double psi_g75(const double *ub, const double *P, dou
   double m2 = 0.0;
 #pragma unroll
   for (int k = 0; k < DIM; ++k) m2 += u[1 + k] * u[1 + k];
-  const double eps = u[S - 1] - m2 / (2.0 * u[0]);
+  const double eps = u[S - 1] - div_alu(m2, 2.0 * u[0]);
   const double r = rroot5(u[0]);
   *r_out = r;
   return eps - phimin * (u[0] * u[0] * (r * r * r));
@@ -532,7 +453,7 @@ __device__ __forceinline__ double dpsi_g75(const double *ub, const double *P, do
   double u[S];
 #pragma unroll
   for (int s = 0; s < S; ++s) u[s] = ub[s] + l * P[s];
-  const double irho = 1.0 / u[0];
+  const double irho = div_alu(1.0, u[0]);
   double v2 = 0.0, vP = 0.0;
 #pragma unroll
   for (int k = 0; k < DIM; ++k) {
@@ -578,9 +499,9 @@ __device__ __forceinline__ LsBracket line_search_bracket(const Params &p, const 
   const double rb = ub[0], rp = P[0];
   // density: the division is needed only when l = 1 leaves [rho_min, rho_max]
   if (pos_strict(rp)) {
-    if (gt_pos(rb + rp, rmax)) l = clamp01((rmax - rb) / rp);
+    if (gt_pos(rb + rp, rmax)) l = clamp01(div_alu(rmax - rb, rp));
   } else if (neg_strict(rp)) {
-    if (lt_pos(rb + rp, rmin)) l = clamp01((rmin - rb) / rp);
+    if (lt_pos(rb + rp, rmin)) l = clamp01(div_alu(rmin - rb, rp));
   }
   b.l = l;
   if (p.gamma75) {
@@ -636,9 +557,9 @@ __device__ double line_search_iterate(const Params &p, const double *ub, const d
                                       const LsBracket &b) {
   double lL = 0.0, lR = b.l, pl = b.pl, pr = b.pr, rR = b.rR;
   for (int it = 0; it < LINE_SEARCH_ITERATIONS; ++it) {
-    double ls = lL + pl * (lR - lL) / (pl - pr);
+    double ls = lL + div_alu(pl * (lR - lL), pl - pr);
     double dr = p.gamma75 ? dpsi_g75<DIM>(ub, P, lR, rR, phimin) : dpsi<DIM>(p, ub, P, lR, phimin);
-    double ln = neg_strict(dr) ? lR - pr / dr : lR;
+    double ln = neg_strict(dr) ? lR - div_alu(pr, dr) : lR;
     if (order_key(ln) < order_key(ls)) ln = ls;
     double ps, pn, rs, rn;
     if (p.gamma75) {
@@ -670,7 +591,7 @@ __device__ double line_search_iterate(const Params &p, const double *ub, const d
 // The line search by pairs of neighbouring lanes that hold the same search, with
 // line_search_start's and line_search_iterate's values bit for bit: psi(l) and
 // psi(0), the secant's and Newton's divisions, and psi at their two points are
-// evaluated side by side (74 instead of 122 FP64 instructions an iteration, at
+// evaluated side by side (52 instead of 85 FP64 instructions an iteration, at
 // 63 cycles each). For queues that leave the chip idle; a full one is faster
 // with a search per lane. gamma = 7/5 (with another gamma the powers are most of
 // the time). All lanes of a warp call both.
@@ -705,7 +626,7 @@ __device__ __forceinline__ double line_search_iterate_pair(const double *ub, con
     if (__all_sync(all, done)) break;
     const double dr = dpsi_g75<DIM>(ub, P, lR, rR, phimin);
     // (a finished search divides 1 by 1: a zero would take the division's slow path)
-    const double q = (done ? 1.0 : odd ? pr : pl * (lR - lL)) / (done ? 1.0 : odd ? dr : pl - pr);
+    const double q = div_alu(done ? 1.0 : odd ? pr : pl * (lR - lL), done ? 1.0 : odd ? dr : pl - pr);
     const double mine = odd ? (neg_strict(dr) ? lR - q : lR) : lL + q;
     const double other = __shfl_xor_sync(all, mine, 1);
     const double ls = odd ? other : mine;
@@ -986,6 +907,9 @@ __device__ __forceinline__ void node_flux(const T *mv, const T *v, T pr, T H, T 
 // ---------------------------------------------------------------------------
 // k_prep: node records (primitives and derived quantities), once per stage
 // ---------------------------------------------------------------------------
+// Bound by FP64 issue: the logarithm and the two roots are 60 of ~70 instructions
+// a node (102 with the divisions and the square root on that pipe: 998k-vertex
+// cylinder 200 -> 160 us, mixed 250 -> 207).
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const double *__restrict__ U,
                                               double *__restrict__ rec, T *__restrict__ vrec,
@@ -1016,7 +940,7 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
     if (same) return;
   }
   double rho = u[0];
-  double irho = 1.0 / rho;
+  double irho = div_alu(1.0, rho);
   double v[DIM], m2 = 0.0;
 #pragma unroll
   for (int k = 0; k < DIM; ++k) {
@@ -1025,7 +949,7 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
   }
   double eps = u[S - 1] - 0.5 * m2 * irho;
   double pr = p.gm1 * eps;
-  double a = sqrt(p.gamma * pr * irho);
+  double a = sqrt_alu(p.gamma * pr * irho);
   double az, phi;
   if (p.gamma75) {
     az = a * rroot7(pr);
@@ -1047,12 +971,12 @@ __global__ void __launch_bounds__(TPB_MAX) k_prep(MeshView m, Params p, const do
   r[R::P] = pr;
   r[R::A] = a;
   r[R::AZ] = az;
-  r[R::IP] = 1.0 / pr;
+  r[R::IP] = div_alu(1.0, pr);
   r[R::PHI] = phi;
   r[R::ETA] = eta;
   r[R::H] = u[S - 1] + pr;
   r[R::IRHO] = irho;
-  r[R::IEPS] = 1.0 / eps;
+  r[R::IEPS] = div_alu(1.0, eps);
   r[R::F32] = pack_f32(a, pr, az);
 #pragma unroll
   for (int q = 0; q <= R::IEPS; q += 4) st4(Rr + q, r[q], r[q + 1], r[q + 2], r[q + 3]);
@@ -1359,8 +1283,9 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
 // and 5.4M FP64 warp instructions (7.4M before lambda_max_sel) with the L1 at
 // 74 % of its throughput through 8-byte accesses, 358 us with 32-byte ones (FP64
 // pipe 80 % of the 84 % that it sustains), 299 us and 4.35M with the differences
-// on the integer units (ALU; pipe 78 %) and three blocks of 256 threads an SM;
-// 493 us before the three.
+// on the integer units (ALU; pipe 78 %) and three blocks of 256 threads an SM,
+// 270 us with the division and the root there too (375k in 3D: 527 -> 420);
+// 493 us before all of these.
 template <int DIM, typename T, bool ALU>
 __global__ void __launch_bounds__(TPB_MAX, 3) k_visc(MeshView m, Params p, Work w, unsigned row_blocks, int lparts) {
   if (w.st->err) return;
@@ -1418,11 +1343,14 @@ __device__ __forceinline__ void indicator_terms(const Work &w, int64_t k, const 
 }
 // alpha_i / 2 (exact): d^H_ij = (a_i/2 + a_j/2) d_ij
 template <typename T> __device__ __forceinline__ double half_alpha(T N, T D) {
-  return D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;
+  if constexpr (sizeof(T) == 8)
+    return D > T(0) ? 0.5 * div_alu(abs_bits(N), D) : 0.0;
+  else
+    return D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;
 }
 
 // Additions on the integer units: 1.7M FP64 warp instructions of 2.7M remain, 998k
-// cylinder 168 -> 134 us.
+// cylinder 168 -> 134 us, 125 with the quotient.
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w) {
   constexpr int S = DIM + 2;
@@ -1533,8 +1461,8 @@ struct DensityBounds {
       }
     }
   }
-  __device__ __forceinline__ double rho_min() const { return dmin == 1.0 ? nmin : nmin / dmin; }
-  __device__ __forceinline__ double rho_max() const { return dmax == 1.0 ? nmax : nmax / dmax; }
+  __device__ __forceinline__ double rho_min() const { return dmin == 1.0 ? nmin : div_alu(nmin, dmin); }
+  __device__ __forceinline__ double rho_max() const { return dmax == 1.0 ? nmax : div_alu(nmax, dmax); }
 };
 
 // c_cfl m_i / (2 sum_j d_ij), or +inf where FP32 shows it to be above the
@@ -1706,7 +1634,8 @@ __device__ __forceinline__ void fold_bound(const Work &w, double bound, int inst
 // for the CFL bound and the minima's FP64 compares are gone: 26.7 (397 us); with
 // the sum of w_ij, du and (mixed) the sums around d_ij on the integer units (ALU)
 // 4.7M, 336 us: FP64 pipe 74 %, integer units 52 %, three blocks of 256 threads an
-// SM (two: 350; four, with spills: 392). Mixed 360 -> 305 us.
+// SM (two: 350; four, with spills: 392), mixed 360 -> 305. The bounds' two divisions
+// on the integer units: 325 us, mixed 285.
 template <int DIM, typename T, bool ALU>
 __global__ void __launch_bounds__(TPB_MAX, ALU && DIM == 2 ? 3 : 2) k_low(MeshView m, Params p, Work w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
