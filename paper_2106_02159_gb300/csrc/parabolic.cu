@@ -8,6 +8,7 @@
 // the final update (eqs. vel_parabolic_discrete, energy_parabolic_discrete).
 // The CG iterations are queued by the host (capi.cu) in batches; their scalars
 // live on the device. State layout [S][n] with S = 4; velocity vectors [n][2].
+#include "integer_fp64.cuh"
 #include "parabolic.cuh"
 
 #include <cmath>
@@ -18,17 +19,18 @@ namespace {
 constexpr int kT = 256;
 inline unsigned grid_for(int64_t m) { return (unsigned)((m + kT - 1) / kT); }
 
+// (divisions on the integer units: 247k nodes 28 -> 15 us)
 __global__ void k_par_init(ParView v, ParWork w, const double *__restrict__ U, double dt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= v.n) return;
   const int n = v.n;
   const double rho = U[i];
   const double D = rho * v.mi[i];
-  const double vx = U[n + i] / rho, vy = U[2 * n + i] / rho;
+  const double vx = div_alu(U[n + i], rho), vy = div_alu(U[2 * n + i], rho);
   w.D[i] = D;
   w.V[2 * i] = vx;
   w.V[2 * i + 1] = vy;
-  w.en[i] = U[3 * n + i] / rho - 0.5 * (vx * vx + vy * vy);
+  w.en[i] = div_alu(U[3 * n + i], rho) - 0.5 * (vx * vx + vy * vy);
   const bool wl = v.wall[i] != 0;
   const int64_t kd = v.diag[i];
   const double c = 0.5 * dt;
@@ -37,7 +39,7 @@ __global__ void k_par_init(ParView v, ParWork w, const double *__restrict__ U, d
   for (int a = 0; a < 2; ++a) {
     w.b[2 * i + a] = wl ? 0.0 : D * vv[a];
     w.x[2 * i + a] = wl ? 0.0 : vv[a];
-    w.iPd[2 * i + a] = wl ? 1.0 : 1.0 / (D + c * v.A[4 * kd + 3 * a]);
+    w.iPd[2 * i + a] = wl ? 1.0 : div_alu(1.0, D + c * v.A[4 * kd + 3 * a]);
   }
 }
 
@@ -62,7 +64,9 @@ __global__ void k_vel_coef(ParView v, const double *__restrict__ G, double *__re
   }
 }
 
-// y = D x + coef A x; wall rows are the identity
+// y = D x + coef A x; wall rows are the identity. FP64 issue is most of it (6
+// instructions an entry: 39 us at 247k rows); with the sums on the integer units 4
+// remain: 35 us, of which reading 115 MB takes 17.
 __global__ void k_vel_apply(ParView v, ParWork w, double coef, const double *__restrict__ x, double *__restrict__ y,
                             const int *skip) {
   if (skip && *skip) return;
@@ -78,8 +82,8 @@ __global__ void k_vel_apply(ParView v, ParWork w, double coef, const double *__r
     const int j = v.col[k];
     const double2 r0 = *(const double2 *)(v.A + 4 * k), r1 = *(const double2 *)(v.A + 4 * k + 2);
     const double2 xj = *(const double2 *)(x + 2 * j);
-    a0 += r0.x * xj.x + r0.y * xj.y;
-    a1 += r1.x * xj.x + r1.y * xj.y;
+    a0 = add_alu(a0, __fma_rn(r0.x, xj.x, __dmul_rn(r0.y, xj.y)));
+    a1 = add_alu(a1, __fma_rn(r1.x, xj.x, __dmul_rn(r1.y, xj.y)));
   }
   const double D = w.D[i];
   *(double2 *)(y + 2 * i) = make_double2(D * xi.x + coef * a0, D * xi.y + coef * a1);
@@ -218,10 +222,13 @@ __global__ void k_min_partial(const double *__restrict__ a, int64_t m, double *_
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// one warp (one thread: 49 us for the 608 partials, a warp: 5)
 __global__ void k_min_partials(const double *__restrict__ part, int np, double *out) {
   double acc = INFINITY;
-  for (int q = 0; q < np; ++q) acc = fmin(acc, part[q]);
-  *out = acc;
+  for (int q = threadIdx.x; q < np; q += 32) acc = fmin(acc, part[q]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc = fmin(acc, __shfl_xor_sync(0xffffffffu, acc, o));
+  if (threadIdx.x == 0) *out = acc;
 }
 
 // every cell's share of int sigma(v):eps(v) phi_a for its nv nodes a, by the
@@ -268,7 +275,7 @@ __global__ void k_source(ParView v, ParWork w) {
   if (i >= v.n) return;
   double acc = 0.0;
   for (int64_t t = v.nc_ptr[i]; t < v.nc_ptr[i + 1]; ++t) acc += w.ce[(int64_t)v.nc_cell[t] * v.nv + v.nc_local[t]];
-  w.K[i] = acc / v.mi[i];
+  w.K[i] = div_alu(acc, v.mi[i]);
 }
 
 __global__ void k_en_rhs(ParView v, ParWork w, double src, double coefL) {
@@ -277,7 +284,7 @@ __global__ void k_en_rhs(ParView v, ParWork w, double src, double coefL) {
   const double D = w.D[i];
   w.b[i] = D * w.en[i] + src * v.mi[i] * w.K[i];
   w.x[i] = w.en[i];
-  w.iPd[i] = 1.0 / (D + coefL * v.L[v.diag[i]]);
+  w.iPd[i] = div_alu(1.0, D + coefL * v.L[v.diag[i]]);
 }
 
 __global__ void k_en_extrapolate(ParView v, ParWork w) {
@@ -381,7 +388,7 @@ void par_final(const ParView &v, const ParWork &w, double *U, cudaStream_t s) {
 }
 void par_min_e(const ParView &v, const ParWork &w, int slot, cudaStream_t s) {
   k_min_partial<<<kRedBlocks, kT, 0, s>>>(w.eH, v.n, w.part);
-  k_min_partials<<<1, 1, 0, s>>>(w.part, kRedBlocks, w.scal + slot);
+  k_min_partials<<<1, 32, 0, s>>>(w.part, kRedBlocks, w.scal + slot);
 }
 
 }  // namespace eh
