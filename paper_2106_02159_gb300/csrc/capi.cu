@@ -624,28 +624,14 @@ eh_status eh_create(const eh_config *cfg, eh_ctx **out) {
   cudaMemset(c->st, 0, sizeof(DevStatus));
   c->mesh_err = (unsigned long long *)(c->st + 1);
   if (cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) c->nsm = 0;
-  if (cfg->dim == 3) {
-    // 3D: eh_autotune on a 6.0M-vertex extruded cylinder (after 100 steps
-    // and on a perturbed state, FP64 and mixed), with k_pass reading P only
-    // where a limiter is below 1: every kernel uncapped (2-3% over a cap of
-    // 512 rows in flight per SM on k_pass, which kept a 27-entry row's lines
-    // of P in L1 while its second walk still re-read all of them)
-    c->tpb[EH_KERNEL_PREP] = 64;
-    c->tpb[EH_KERNEL_VISC] = 128;
-    c->tpb[EH_KERNEL_LOW] = 64;
-    c->tpb[EH_KERNEL_LIM1] = 128;
-    c->tpb[EH_KERNEL_PASS] = 256;
-    c->tpb[EH_KERNEL_FINAL] = 64;
-    c->tpb[EH_KERNEL_LSEARCH] = 64;
-  } else {
-    // 2D: eh_autotune on the 4.0M cylinder (bench window and a perturbed
-    // state, FP64 and mixed) picks 64 rows per block and no cap on the rows
-    // in flight for the row kernels (1-2% faster than 128 with caps)
-    for (int k = 0; k < EH_KERNEL_COUNT; ++k)
-      if (k != EH_KERNEL_TAU) c->tpb[k] = 64;
-    c->tpb[EH_KERNEL_LSEARCH] = 128;
-    c->tpb[EH_KERNEL_VISC] = 128;
-  }
+  // 64 threads per block and no cap on the rows in flight for every row kernel.
+  // A block's registers are freed when its slowest warp ends: 128 and 256 threads
+  // against 64 take 1-2 and 4-10 % more on large meshes (k_lim1 of the 998k
+  // cylinder 331, 335, 348 us; k_pass of a 375k 3D one 307, 314, 334), the queued
+  // searches 3-14 and 20-35 % (246k cylinder, gamma = 1.3: 193, 219, 256 us). Caps
+  // lost 2-3 % where k_pass reads P only for limiters below 1 (6.0M vertices in 3D).
+  for (int k = 0; k < EH_KERNEL_COUNT; ++k)
+    if (k != EH_KERNEL_TAU) c->tpb[k] = 64;
   Params &p = c->prm;
   p.gamma = cfg->gamma;
   p.cfl = cfg->cfl;
