@@ -336,7 +336,8 @@ eh_status eh_get_rows_per_sm(const eh_ctx *ctx, int32_t *rows);
  * 256; rows_per_sm 0 (one thread per row) or, for EH_KERNEL_LIM1, _PASS and
  * _FINAL only, a cap of 1..2048 rows in flight per SM (the kernel then loops
  * over rows with a grid stride). EH_ERR_INVALID_ARG otherwise. Results do not
- * depend on the shape. */
+ * depend on the shape. Meshes below 64k rows run forms of some kernels (rows
+ * split over warps) whose blocks these calls do not change. */
 eh_status eh_set_launch_shape(eh_ctx *ctx, int32_t kernel, int32_t threads_per_block, int32_t rows_per_sm);
 
 /* Number of kernel launches one eh_step issues (for accounting). */
