@@ -1349,8 +1349,10 @@ template <typename T> __device__ __forceinline__ double half_alpha(T N, T D) {
     return D > T(0) ? 0.5 * (double)(fabs(N) / D) : 0.0;
 }
 
-// Additions on the integer units: 1.7M FP64 warp instructions of 2.7M remain, 998k
-// cylinder 168 -> 134 us, 125 with the quotient.
+// Three of an entry's four additions on the integer units: 998k cylinder 168 -> 134
+// us with all four there, 132 with the quotient too (integer units 73 % busy, FP64
+// pipe 58 %), and with the sum of D back on the FP64 pipe k_visc and k_alpha 399 ->
+// 392 us (375k in 3D 578 -> 560). 643 MB are read, 95 us at the memory's rate.
 template <int DIM, typename T>
 __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w) {
   constexpr int S = DIM + 2;
@@ -1369,7 +1371,7 @@ __global__ void __launch_bounds__(TPB_MAX) k_alpha(MeshView m, Params p, Work w)
     T n, d;
     indicator_terms<DIM, T, true>(w, k, deta, n, d);
     N = add_on<true>(N, n);
-    D = add_on<true>(D, d);
+    D = add_on<false>(D, d);
   }
   w.alpha[i] = half_alpha(N, D);
 }
