@@ -369,6 +369,63 @@ eh_status setup_instances(eh_ctx *c, int ninst, const int64_t *off, const double
   return EH_OK;
 }
 
+// The boundary list's checks; isb (n values) = 1 for its nodes.
+eh_status check_boundary(eh_ctx *c, int32_t n, int32_t n_bnd, const int32_t *node, const int32_t *kind,
+                         const double *state, std::vector<unsigned char> &isb) {
+  isb.assign(n, 0);
+  for (int b = 0; b < n_bnd; ++b) {
+    const int i = node[b];
+    if (i < 0 || i >= n || isb[i]) return fail(c, EH_ERR_BAD_MESH, "boundary node %d invalid or repeated", i);
+    if (kind[b] < EH_BC_SLIP || kind[b] > EH_BC_GODUNOV)
+      return fail(c, EH_ERR_BAD_MESH, "boundary kind %d invalid", kind[b]);
+    if (kind[b] != EH_BC_SLIP && kind[b] != EH_BC_DO_NOTHING && !state)
+      return fail(c, EH_ERR_BAD_MESH, "boundary kind %d needs a Dirichlet state", kind[b]);
+    isb[i] = 1;
+  }
+  return EH_OK;
+}
+
+// The first error of a mesh, entry by entry: rows, then the pattern, then the
+// coefficients, then the boundary list; EH_OK if there is none. The device
+// decides whether a mesh is taken (eh_upload_mesh); this names what is wrong
+// with one that is not, or for which there is no room.
+eh_status first_mesh_error(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_ptr, const int32_t *col,
+                           const double *cij, const double *mij, const double *mi, int32_t n_bnd, const int32_t *node,
+                           const int32_t *kind, const double *state) {
+  if (row_ptr[0] != 0 || row_ptr[n] != nnz) return fail(c, EH_ERR_BAD_MESH, "row_ptr must start at 0 and end at nnz");
+  for (int i = 0; i < n; ++i) {
+    if (row_ptr[i + 1] - row_ptr[i] < 2) return fail(c, EH_ERR_BAD_MESH, "row %d has fewer than 2 entries", i);
+    if (row_ptr[i + 1] > nnz) continue;  // (a later row is too short)
+    bool diag = false;
+    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
+      if (col[k] < 0 || col[k] >= n) return fail(c, EH_ERR_BAD_MESH, "column out of range in row %d", i);
+      if (k > row_ptr[i] && col[k] <= col[k - 1]) return fail(c, EH_ERR_BAD_MESH, "row %d not sorted/unique", i);
+      if (col[k] == i) diag = true;
+    }
+    if (!diag) return fail(c, EH_ERR_BAD_MESH, "row %d has no diagonal entry", i);
+    if (!(mi[i] > 0.0)) return fail(c, EH_ERR_BAD_MESH, "m_%d <= 0", i);
+  }
+  const auto transposed = [&](int i, int j) {  // the position of entry (j, i), -1 if there is none
+    const int32_t *e = col + row_ptr[j + 1], *f = std::lower_bound(col + row_ptr[j], e, i);
+    return f == e || *f != i ? (int64_t)-1 : (int64_t)(f - col);
+  };
+  for (int i = 0; i < n; ++i)
+    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k)
+      if (transposed(i, col[k]) < 0) return fail(c, EH_ERR_BAD_MESH, "pattern not symmetric at (%d,%d)", i, col[k]);
+  for (int i = 0; i < n; ++i)
+    for (int64_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) {
+      double s2 = 0.0;
+      for (int d = 0; d < c->cfg.dim; ++d) s2 += cij[(int64_t)d * nnz + k] * cij[(int64_t)d * nnz + k];
+      if (col[k] != i && !(std::sqrt(s2) > 0.0))
+        return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry");
+      const double a = mij[k], b = mij[transposed(i, col[k])];
+      if (std::fabs(a - b) > 1e-12 * std::max(std::fabs(a), std::fabs(b)))
+        return fail(c, EH_ERR_BAD_MESH, "consistent mass not symmetric at (%d,%d)", i, col[k]);
+    }
+  std::vector<unsigned char> isb;
+  return check_boundary(c, n, n_bnd, node, kind, state, isb);
+}
+
 // Device arrays of the static mesh data for (up to) n nodes, nnz entries,
 // n_bnd boundary nodes and n_bp edges between two of them; sets the MeshView
 // pointers (contents not written).
@@ -679,21 +736,16 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   free_mesh(c);
   const int dim = c->cfg.dim, S = S_of(c);
   // ---- checks on the host: what the device's checks index by ----
-  if (row_ptr[0] != 0 || row_ptr[n] != nnz) return fail(c, EH_ERR_BAD_MESH, "row_ptr must start at 0 and end at nnz");
-  for (int i = 0; i < n; ++i)
-    if (row_ptr[i + 1] - row_ptr[i] < 2) return fail(c, EH_ERR_BAD_MESH, "row %d has fewer than 2 entries", i);
-  std::vector<unsigned char> isb(n, 0);
+  const auto refused = [&] {
+    return first_mesh_error(c, n, nnz, row_ptr, col, cij, mij, mi, n_bnd, bnd_node, bnd_kind, bnd_state);
+  };
+  std::vector<unsigned char> isb;
+  bool rows = row_ptr[0] == 0 && row_ptr[n] == nnz;
+  for (int i = 0; i < n; ++i) rows &= row_ptr[i + 1] - row_ptr[i] >= 2;
+  if (!rows || check_boundary(c, n, n_bnd, bnd_node, bnd_kind, bnd_state, isb) != EH_OK) return refused();
   int nonreflecting = 0;
-  for (int b = 0; b < n_bnd; ++b) {
-    const int i = bnd_node[b];
-    if (i < 0 || i >= n || isb[i]) return fail(c, EH_ERR_BAD_MESH, "boundary node %d invalid or repeated", i);
-    if (bnd_kind[b] < EH_BC_SLIP || bnd_kind[b] > EH_BC_GODUNOV)
-      return fail(c, EH_ERR_BAD_MESH, "boundary kind %d invalid", bnd_kind[b]);
-    if (bnd_kind[b] != EH_BC_SLIP && bnd_kind[b] != EH_BC_DO_NOTHING && !bnd_state)
-      return fail(c, EH_ERR_BAD_MESH, "boundary kind %d needs a Dirichlet state", bnd_kind[b]);
-    if (bnd_kind[b] == EH_BC_CHARACTERISTIC || bnd_kind[b] == EH_BC_GODUNOV) ++nonreflecting;
-    isb[i] = 1;
-  }
+  for (int b = 0; b < n_bnd; ++b)
+    nonreflecting += bnd_kind[b] == EH_BC_CHARACTERISTIC || bnd_kind[b] == EH_BC_GODUNOV;
   // edges between two boundary nodes, from the smaller one's row (columns are
   // not checked yet; a mesh with a bad one is rejected below)
   std::vector<int32_t> bprow, bppos;
@@ -716,7 +768,8 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   if ((st = alloc_static(c, n, nnz, n_bnd, (int64_t)bprow.size())) != EH_OK ||
       (st = alloc_work(c, n, nnz)) != EH_OK) {
     free_mesh(c);
-    return st;
+    const eh_status bad = refused();  // (a bad mesh is reported as such, whether there is room for it or not)
+    return bad ? bad : st;
   }
   // the caller's c_ij and m_ij, needed until the static arrays are made from
   // them: in work arrays where there are some
@@ -727,7 +780,8 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
     if (cudaMalloc(&tmp, sizeof(double) * (size_t)(dim + 1) * nnz) != cudaSuccess) {
       cudaGetLastError();
       free_mesh(c);
-      return fail(c, EH_ERR_OOM, "cudaMalloc of %zu bytes", sizeof(double) * (size_t)(dim + 1) * nnz);
+      const eh_status bad = refused();
+      return bad ? bad : fail(c, EH_ERR_OOM, "cudaMalloc of %zu bytes", sizeof(double) * (size_t)(dim + 1) * nnz);
     }
     cij_d = (double *)tmp;
     mij_d = cij_d + (size_t)dim * nnz;
@@ -797,16 +851,8 @@ eh_status eh_upload_mesh(eh_ctx *c, int32_t n, int64_t nnz, const int64_t *row_p
   }
   if (key != ~0ull) {
     free_mesh(c);
-    const int row = (int)((key >> 16) & 0xFFFFFFFFu);
-    switch (key & 0xFFFF) {
-      case MESH_ERR_COL: return fail(c, EH_ERR_BAD_MESH, "column out of range in row %d", row);
-      case MESH_ERR_ORDER: return fail(c, EH_ERR_BAD_MESH, "row %d not sorted/unique", row);
-      case MESH_ERR_DIAG: return fail(c, EH_ERR_BAD_MESH, "row %d has no diagonal entry", row);
-      case MESH_ERR_MASS: return fail(c, EH_ERR_BAD_MESH, "m_%d <= 0", row);
-      case MESH_ERR_PATTERN: return fail(c, EH_ERR_BAD_MESH, "pattern not symmetric in row %d", row);
-      case MESH_ERR_CIJ: return fail(c, EH_ERR_BAD_MESH, "c_ij = 0 at an off-diagonal entry of row %d", row);
-      default: return fail(c, EH_ERR_BAD_MESH, "consistent mass not symmetric in row %d", row);
-    }
+    const eh_status bad = refused();
+    return bad ? bad : fail(c, EH_ERR_BAD_MESH, "row %d refused", (int)(key & 0xFFFFFFFFu));
   }
   c->n = n;
   c->nnz = nnz;

@@ -2869,34 +2869,35 @@ template <int DIM> void launch_count_not_admissible(int n, const double *U, DevS
 // binary search an entry) and the norms took most of an upload (998k vertices,
 // 9.0M entries: 104 ms; here 8.5 ms, bound by the copies of the caller's arrays)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void mesh_error(unsigned long long *err, int phase, int row, int code) {
-  atomicMin(err, (unsigned long long)phase << 56 | (unsigned long long)(unsigned)row << 16 | (unsigned)code);
+__device__ __forceinline__ void mesh_error(unsigned long long *err, int phase, int row) {
+  atomicMin(err, (unsigned long long)phase << 32 | (unsigned)row);
 }
-__device__ __forceinline__ bool mesh_failed(const unsigned long long *err) { return *err != ~0ull; }
+// an error of an earlier phase (one of the same phase leaves the other rows
+// running: the smallest row counts, not the first thread)
+__device__ __forceinline__ bool mesh_failed(const unsigned long long *err, int phase) {
+  return (*(const volatile unsigned long long *)err >> 32) < (unsigned)phase;
+}
 
 __global__ void k_mesh_rows(MeshView m, double *inv_mi, double *lam, unsigned long long *err) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m.n) return;
   const int64_t k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
-  bool diag = false;
-  int prev = -1, code = 0;
-  for (int64_t k = k0; k < k1 && !code; ++k) {
+  bool diag = false, ok = m.mi[i] > 0.0;
+  int prev = -1;
+  for (int64_t k = k0; k < k1; ++k) {
     const int c = m.col[k];
-    if (c < 0 || c >= m.n) code = MESH_ERR_COL;
-    else if (k > k0 && c <= prev) code = MESH_ERR_ORDER;
-    if (c == i) diag = true;
+    ok &= c > prev && c < m.n;
+    diag |= c == i;
     prev = c;
   }
-  if (!code && !diag) code = MESH_ERR_DIAG;
-  if (!code && !(m.mi[i] > 0.0)) code = MESH_ERR_MASS;
-  if (code) mesh_error(err, 0, i, code);
+  if (!ok || !diag) mesh_error(err, 0, i);
   inv_mi[i] = 1.0 / m.mi[i];
   lam[i] = 1.0 / (double)(k1 - k0 - 1);
 }
 
 __global__ void k_mesh_transpose(MeshView m, int32_t *tr, unsigned long long *err) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.n || mesh_failed(err)) return;
+  if (i >= m.n || mesh_failed(err, 1)) return;
   for (int64_t k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
     const int j = m.col[k];
     int64_t lo = m.row_ptr[j], hi = m.row_ptr[j + 1];
@@ -2906,7 +2907,7 @@ __global__ void k_mesh_transpose(MeshView m, int32_t *tr, unsigned long long *er
       if (m.col[mid] < i) lo = mid + 1; else hi = mid;
     }
     if (lo == end || m.col[lo] != i) {
-      mesh_error(err, 1, i, MESH_ERR_PATTERN);
+      mesh_error(err, 1, i);
       return;
     }
     tr[k] = (int32_t)lo;
@@ -2917,9 +2918,7 @@ template <int DIM, typename T>
 __global__ void k_mesh_entries(MeshView m, const double *cij, const double *mij, T *geo, T *geo_inv, double *betat,
                                unsigned long long *err) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m.n) return;
-  // (an error of this phase leaves the other rows running: the smallest key counts)
-  if ((*(volatile unsigned long long *)err >> 56) < 2) return;
+  if (i >= m.n || mesh_failed(err, 2)) return;
   for (int64_t k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
     double c[DIM], s2 = 0.0;
 #pragma unroll
@@ -2929,7 +2928,7 @@ __global__ void k_mesh_entries(MeshView m, const double *cij, const double *mij,
     }
     const double cn = sqrt(s2), ci = cn > 0.0 ? 1.0 / cn : 0.0;
     if (m.col[k] != i && !(cn > 0.0)) {
-      mesh_error(err, 2, i, MESH_ERR_CIJ);
+      mesh_error(err, 2, i);
       return;
     }
 #pragma unroll
@@ -2940,7 +2939,7 @@ __global__ void k_mesh_entries(MeshView m, const double *cij, const double *mij,
     // k_lim1 relies on it, with the mean of the two entries
     const double a = mij[k], b = mij[m.tr[k]];
     if (fabs(a - b) > 1e-12 * fmax(fabs(a), fabs(b))) {
-      mesh_error(err, 2, i, MESH_ERR_MIJ);
+      mesh_error(err, 2, i);
       return;
     }
     betat[k] = 0.5 * (a + b) / m.mi[i];

@@ -235,12 +235,11 @@ template <int DIM>
 void launch_state_stats(int n, const double *U, const double *mi, double *part, double *out, cudaStream_t s);
 
 // Mesh checks and static arrays of eh_upload_mesh, from the caller's arrays
-// copied to the device. *err (all-ones before) receives the smallest error
-// key found, row-major: phase << 56 | row << 16 | code (MESH_ERR_*); a kernel
-// whose predecessor found an error does nothing, so no index is used before it
-// is checked (row_ptr itself is checked by the caller).
-enum { MESH_ERR_COL = 1, MESH_ERR_ORDER = 2, MESH_ERR_DIAG = 3, MESH_ERR_MASS = 4, MESH_ERR_PATTERN = 5,
-       MESH_ERR_CIJ = 6, MESH_ERR_MIJ = 7 };
+// copied to the device. *err (all-ones before) receives the smallest of
+// phase << 32 | row over the rows with an error (phase: the kernels below in
+// order; the host names the error). A kernel whose predecessor found one does
+// nothing, so no index is used before it is checked (row_ptr itself is checked
+// by the caller).
 // sorted unique columns in range, a diagonal, m_i > 0; 1/m_i and lambda_i
 void launch_mesh_rows(const MeshView &m, double *inv_mi, double *lam, unsigned long long *err, cudaStream_t s);
 // the transpose index
