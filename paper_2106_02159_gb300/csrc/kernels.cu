@@ -2968,6 +2968,14 @@ void launch_mesh_boundary(const MeshView &m, int32_t *bnd_index, unsigned char *
   if (m.n_bnd > 0) k_mesh_boundary<<<nblocks(m.n_bnd, 256), 256, 0, s>>>(m, bnd_index, isb);
 }
 
+__global__ void k_gather_second(double *dst, const double *pairs, int64_t count) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < count) dst[k] = pairs[2 * k + 1];
+}
+void launch_gather_second(double *dst, const double *pairs, int64_t count, cudaStream_t s) {
+  k_gather_second<<<nblocks(count, 256), 256, 0, s>>>(dst, pairs, count);
+}
+
 // dst[i] = src[i] + add (nonneg_only: only where src[i] >= 0; -1 entries
 // stay): the index arrays of one instance placed into a block-diagonal union
 template <typename I> __global__ void k_offset_copy(I *dst, const I *src, int64_t count, I add, int nonneg_only) {

@@ -251,6 +251,9 @@ void launch_mesh_entries(const MeshView &m, const double *cij, const double *mij
 // bnd_index (-1 before) and isb (0 before) of the boundary nodes
 void launch_mesh_boundary(const MeshView &m, int32_t *bnd_index, unsigned char *isb, cudaStream_t s);
 
+// dst[k] = pairs[2 k + 1] over count pairs
+void launch_gather_second(double *dst, const double *pairs, int64_t count, cudaStream_t s);
+
 // dst[i] = src[i] + add over count entries (nonneg_only: negative entries
 // copied unchanged); int32_t and int64_t
 template <typename I>
