@@ -47,11 +47,15 @@ struct Slot {
 // line-search queues), with 10% and 1 MiB of headroom
 uint64_t estimate_bytes(int dim, int precision, int64_t n, int64_t nnz) {
   const int64_t S = dim + 2, SP = dim == 2 ? 4 : 6;
-  int64_t per_entry = 4 + 4 + 8 * dim + 8 * 4 + 8 * SP * 2 + 8 * 3 + 8 + 5;
-  int64_t per_node = 8 * (24 + 8 * SP + 3 * S + 13);
+  // every entry: P, three limiters, the search queues
+  int64_t per_entry = 8 * SP + 8 * 3 + 8 + 5, per_node;
   if (precision == EH_PRECISION_MIXED) {
-    per_entry += 4 * (dim + 2 + SP + 1);
-    per_node += 4 * (40 + SP);
+    // col, tr, m_ij/m_i, c_ij with its norms in FP32, the 8-value FP32 slot
+    per_entry += 4 + 4 + 8 + 4 * (dim == 2 ? 4 : 5) + 4 * 8;
+    per_node = 8 + 8 * 4 + 1 + 4 + 8 * 24 + 4 * 40 + 8 + 6 + 8 * 4 + (8 * 5 + 4) * SP + 8 * 3 * S;
+  } else {
+    per_entry += 4 + 4 + 8 * dim + 8 * 4 + 8 * SP;
+    per_node = 8 * (24 + 8 * SP + 3 * S + 13);
   }
   return (uint64_t)(1.1 * (double)(per_entry * nnz + per_node * n)) + (1u << 20);
 }

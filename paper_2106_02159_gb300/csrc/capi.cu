@@ -1643,8 +1643,10 @@ cudaStream_t stream_of(const eh_ctx *c) { return c->stream; }
 
 uint64_t part_bytes(int dim, int precision, int64_t n, int64_t nnz, int64_t n_bnd) {
   const int64_t S = dim + 2;
-  int64_t per_entry = 4 + 4 + 8 * dim + 8 * 3, per_node = 8 + 8 * 4 + 1 + 4 + 8 * S + 8 * 4;
-  if (precision == EH_PRECISION_MIXED) per_entry += 4 * (dim + 2);
+  // col, tr, m_ij/m_i, and c_ij with its norms in the viscosity precision; the
+  // boundary pairs (8 bytes each) are within the last 32 bytes a node
+  const int64_t per_entry = 4 + 4 + 8 + (precision == EH_PRECISION_MIXED ? 4 : 8) * (dim == 2 ? 4 : 5);
+  const int64_t per_node = 8 + 8 * 4 + 1 + 4 + 8 * S + 8 * 4;
   return (uint64_t)(per_entry * nnz + per_node * n + (8 + 8 * dim + 8 * S) * n_bnd) + (1u << 16);
 }
 
