@@ -320,15 +320,16 @@ eh_status eh_get_instance_steps(eh_ctx *ctx, int64_t *steps);
  * every candidate -- 64, 128 and 256 rows per block, and for the grid-stride
  * kernels (EH_KERNEL_LIM1, _PASS, _FINAL) one thread per row or at most 256,
  * 512 or 768 rows in flight per SM -- times every kernel with CUDA events and
- * keeps the fastest shape per kernel kind. The state and the instance times
- * are restored afterwards. chosen (may be NULL) receives EH_KERNEL_COUNT
+ * keeps the fastest shape per kernel kind (the current shape of a kind whose
+ * launches do not depend on it, see eh_set_launch_shape). The state and the
+ * instance times are restored afterwards. chosen (may be NULL) receives EH_KERNEL_COUNT
  * block sizes. */
 eh_status eh_autotune(eh_ctx *ctx, int32_t steps_per_candidate, int32_t *chosen);
 
-/* Current block size of every kernel kind (EH_KERNEL_COUNT values). */
+/* Block size set for every kernel kind (EH_KERNEL_COUNT values). */
 eh_status eh_get_block_sizes(const eh_ctx *ctx, int32_t *tpb);
 
-/* Rows in flight per SM of every kernel kind (EH_KERNEL_COUNT values; 0 = one
+/* Rows in flight per SM set for every kernel kind (EH_KERNEL_COUNT values; 0 = one
  * thread per row, the grid covering all rows at once). */
 eh_status eh_get_rows_per_sm(const eh_ctx *ctx, int32_t *rows);
 
@@ -336,8 +337,10 @@ eh_status eh_get_rows_per_sm(const eh_ctx *ctx, int32_t *rows);
  * 256; rows_per_sm 0 (one thread per row) or, for EH_KERNEL_LIM1, _PASS and
  * _FINAL only, a cap of 1..2048 rows in flight per SM (the kernel then loops
  * over rows with a grid stride). EH_ERR_INVALID_ARG otherwise. Results do not
- * depend on the shape. Meshes below 64k rows run forms of some kernels (rows
- * split over warps) whose blocks these calls do not change. */
+ * depend on the shape. On small meshes some kernels run in forms that split rows
+ * over warps, with blocks of their own: k_alpha (timed as EH_KERNEL_VISC) and
+ * EH_KERNEL_LOW below 32768 rows, EH_KERNEL_LIM1 and the first limiter pass of
+ * EH_KERNEL_PASS below 65536. The shape is kept there, but has no effect. */
 eh_status eh_set_launch_shape(eh_ctx *ctx, int32_t kernel, int32_t threads_per_block, int32_t rows_per_sm);
 
 /* Number of kernel launches one eh_step issues (for accounting). */

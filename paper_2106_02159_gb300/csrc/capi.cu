@@ -1440,7 +1440,8 @@ eh_status eh_autotune(eh_ctx *c, int32_t steps_per_candidate, int32_t *chosen) {
       CUDA_TRY(c, cudaGetLastError());
       flush_profile(c);
       for (int k = 0; k < EH_KERNEL_COUNT; ++k)
-        if (k != EH_KERNEL_TAU && c->prof_count[k] && c->prof_ms[k] < best_ms[k]) {
+        if (k != EH_KERNEL_TAU && launch_shape_used(k, c->n, c->cfg.limiter_passes) && c->prof_count[k] &&
+            c->prof_ms[k] < best_ms[k]) {
           best_ms[k] = c->prof_ms[k];
           best[k] = cands[q];
           best_cap[k] = c->rows_per_sm[k];

@@ -20,6 +20,7 @@
 // its remainder (1 - l) P_ij as the factor 1 - l (nothing is read where it is
 // 0); a row whose limiters are all 1 stores none and says so in a flag.
 #include "integer_fp64.cuh"
+#include "../../include/euler_hyp.h"
 #include "kernels.cuh"
 
 #include <cooperative_groups.h>
@@ -2709,6 +2710,14 @@ constexpr int SPLIT_ENTRIES = 64 * 1024;  // k_lim1, k_pass: the entries are ind
 // 54 and 58 against 59), at 998k 391 against 336 and 386 against 328. 3D k_low has
 // them at every size (95k rows 175 -> 172 us), 3D k_lim1 nowhere (625 -> 642 us).
 constexpr int ALU_ROWS = 96 * 1024;
+bool launch_shape_used(int kernel, int64_t n, int limiter_passes) {
+  switch (kernel) {
+    case EH_KERNEL_LOW: return n >= SPLIT_SUMS;
+    case EH_KERNEL_LIM1: return n >= SPLIT_ENTRIES;
+    case EH_KERNEL_PASS: return n >= SPLIT_ENTRIES || limiter_passes > 2;  // the first of the passes is split
+    default: return true;
+  }
+}
 template <int DIM, typename T>
 void launch_prep(const MeshView &m, const Params &p, const double *U, const Work &w, int tpb, cudaStream_t s) {
   k_prep<DIM, T><<<nblocks(m.n, tpb), tpb, 0, s>>>(m, p, U, w.rec, (T *)w.vrec, w.rough, w.steady, w.st);

@@ -192,6 +192,9 @@ constexpr int LSQ_SLOTS = 8;  // limiter passes per stage, at most
 // 'tpb' is the block size: 64, 128 or 256 threads, a thread per row (k_visc: a
 // lane per row, the row's entries dealt out to one, two or four warps).
 constexpr int TPB_MAX = 256;
+// false where every launch of a kernel kind (EH_KERNEL_*) on a mesh of n rows is
+// of a split form, whose blocks are fixed
+bool launch_shape_used(int kernel, int64_t n, int limiter_passes);
 template <int DIM, typename T>
 void launch_prep(const MeshView &m, const Params &p, const double *U, const Work &w, int tpb, cudaStream_t s);
 template <int DIM, typename T>
