@@ -1469,10 +1469,13 @@ struct DensityBounds {
 };
 
 // c_cfl m_i / (2 sum_j d_ij), or +inf where FP32 shows it to be above the
-// instance's minimum so far (which only ever falls): the division is then left out
+// instance's minimum so far (which only ever falls): the division is then left
+// out. Numerator and minimum well within FP32's normal range: a minimum below it
+// would be truncated to 0, above which every row's estimate lies.
 __device__ __forceinline__ double row_cfl_bound(const Params &p, double m, double dsum, unsigned long long so_far) {
-  const float est = __fdividef(0.5f * p.cfl_f * trunc_f32(m), trunc_f32(dsum));
-  if (est > trunc_f32(__longlong_as_double((long long)so_far)) * (1.0f + 4e-6f) && est < 1e30f) return INFINITY;
+  const float num = 0.5f * p.cfl_f * trunc_f32(m), est = __fdividef(num, trunc_f32(dsum));
+  const float low = trunc_f32(__longlong_as_double((long long)so_far));
+  if (num > 1e-30f && low > 1e-30f && est > low * (1.0f + 4e-6f) && est < 1e30f) return INFINITY;
   return p.cfl * m / (2.0 * dsum);
 }
 

@@ -1,0 +1,43 @@
+"""The FP32 pre-decisions at the ends of FP32's range: a change of units by powers
+of two (lengths, densities, velocities) scales the method's quantities by powers
+of two, so what the solver gives in one system of units it has to give in another,
+however small the numbers are. Needs a GPU."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2106_02159_gb300 import binding as B
+from paper_2106_02159_gb300 import meshes as M
+from paper_2106_02159_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _units(mesh, U, length, density, velocity):
+    """Mesh and state in units in which lengths, densities and velocities are so many times larger."""
+    d = mesh.dim
+    mesh = dataclasses.replace(mesh, cij=mesh.cij * length ** (d - 1), mij=mesh.mij * length**d, mi=mesh.mi * length**d)
+    scale = np.array([1.0] + [velocity] * d + [velocity**2]) * density
+    return mesh, np.ascontiguousarray(U * scale[:, None])
+
+
+@pytest.mark.parametrize("length,density,velocity", [(1.0, 1.0, 1.0), (2.0**-50, 2.0**-30, 2.0**70),
+                                                     (2.0**-60, 2.0**-20, 2.0**62)])
+def test_cfl_step_below_the_fp32_range(length, density, velocity):
+    """A mesh of several waves of blocks whose last part has the smallest bound:
+    the step is that of the part alone (bounds of 1e-38 and less are not brushed
+    aside by the FP32 comparison with the minimum so far)."""
+    part = M.cylinder_channel_q1(20)
+    copies = 150
+    slow, fast = (W.perturbed_state(part, 1, base=dict(rho=1.4, vel=(v, 0.0), p=1.0), amplitude=0.1) for v in (0.5, 9.0))
+    dt = []
+    for states in ([fast], [slow] * (copies - 1) + [fast]):
+        mesh, _, bs = M.concatenate([part] * len(states), [np.ones((4, part.n_bnd))] * len(states))
+        mesh, U = _units(mesh, np.concatenate(states, axis=1), length, density, velocity)
+        s = B.Solver()
+        s.upload_mesh(mesh, bs)
+        s.set_state(U)
+        dt.append(s.cfl_dt())
+        s.close()
+    assert dt[0] == dt[1], dt
