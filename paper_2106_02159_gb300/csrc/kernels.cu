@@ -322,8 +322,10 @@ __device__ __forceinline__ float2 unpack_f32(double x) {
 // Errors, u = 2^-24: a and p are rounded (u), a p^-z, v.c and 1/|c| truncated
 // (2u); normal velocities 5u; the numerator of p_tr 6u of its terms'
 // magnitudes (gamma <= 5/3); the quotient 8u more; the seventh power (or exp2
-// of inv_z log2) multiplies the relative error by 7 (inv_z). Anything unclear,
-// or out of FP32's range (a = NaN), takes the full evaluation.
+// of inv_z log2) multiplies the relative error by 7 (inv_z). A v.c below 2^-126 is
+// truncated to 0, which moves a normal velocity by up to 2^-126 / |c|: that has to
+// stay below u of the speeds. Anything unclear, or out of FP32's range (a = NaN),
+// takes the full evaluation.
 template <bool ALU>
 __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, double vcr, double ci, double pl, double al,
                                                  double azl, double ipl, float2 fl, double pr, double ar, double azr,
@@ -346,7 +348,8 @@ __device__ __forceinline__ double lambda_max_sel(const Params &p, double vcl, do
     rel = 1.2f * p.inv_z_f * (en + 12.0f * u + 4.0f * u * fabsf(lg)) + 24.0f * u;
   }
   bool left = false, two = true, need = true;
-  if (num_f > 0.0f && en < 0.01f && rel < 0.05f && ptr_f > 1e-30f && ptr_f < 1e30f && mag < 1e18f) {
+  if (num_f > 0.0f && en < 0.01f && rel < 0.05f && ptr_f > 1e-30f && ptr_f < 1e30f && mag < 1e18f &&
+      4e-31f * cif < mag) {
     const float plo = ptr_f * (1.0f - rel), phi = ptr_f * (1.0f + rel);
     const float ql = __fdividef(1.0f, fl.y), qr = __fdividef(1.0f, fr.y);
     constexpr float r8 = 8.0f * u;

@@ -41,3 +41,26 @@ def test_cfl_step_below_the_fp32_range(length, density, velocity):
         dt.append(s.cfl_dt())
         s.close()
     assert dt[0] == dt[1], dt
+
+
+@pytest.mark.parametrize("nv,dim", [(24, 2), (270, 2), (0, 3)])  # (270: 72900 rows, the integer forms)
+def test_viscosity_on_very_small_meshes(nv, dim):
+    """Slow flow on meshes whose v.c_ij are below FP32's range: d_ij scales with
+    |c_ij| to the last bit (no product with a velocity is taken for 0 where the
+    FP32 intervals choose the outer wave)."""
+    mesh = M.periodic_p1_square(nv) if dim == 2 else M.structured_q1_3d(9, 8, 10, periodic=(True, True, True))
+    rng = np.random.default_rng(4)
+    rho, p = 1.0 + 1e-5 * rng.random(mesh.n), (1.0 + 1e-5 * rng.random(mesh.n)) / 1.4
+    vel = 2e-5 * rng.standard_normal((dim, mesh.n))
+    U = np.concatenate([rho[None], rho * vel, (p / 0.4 + 0.5 * rho * (vel * vel).sum(0))[None]])
+    c_scale = 2.0**-112  # |c_ij| about 1e-35
+    d = []
+    for length in (1.0, c_scale if dim == 2 else c_scale**0.5):
+        m, V = _units(mesh, U, length, 1.0, 1.0)
+        s = B.Solver(dim=dim)
+        s.upload_mesh(m)
+        s.set_state(V)
+        s.stage()
+        d.append(s.trace(B.EH_TRACE_D_IJ))
+        s.close()
+    assert np.array_equal(d[0] * c_scale, d[1]), np.max(np.abs(d[1] / c_scale / d[0] - 1.0))
