@@ -277,16 +277,16 @@ template <int DIM> struct NodeF {
 template <int DIM> __device__ inline bool node_f32(const Arrays &g, const Gas &G, int i, NodeF<DIM> &w) {
   const float rho = trunc_f32(g.U[i]), E = trunc_f32(g.U[(int64_t)(DIM + 1) * g.n + i]);
   const float ir = __fdividef(1.0f, rho);
-  float m2 = 0.0f;
+  float ke = 0.0f;  // as m v: the squares of small momenta would leave FP32's range
   w.V = 0.0f;
 #pragma unroll
   for (int q = 0; q < DIM; ++q) {
     const float m = trunc_f32(g.U[(int64_t)(1 + q) * g.n + i]);
-    m2 += m * m;
     w.v[q] = m * ir;
+    ke += 0.5f * m * w.v[q];
     w.V += fabsf(w.v[q]);
   }
-  const float ke = 0.5f * m2 * ir, eps = E - ke;
+  const float eps = E - ke;
   const float ee = __fdividef(10.0f * kU * (E + ke), eps);  // relative error of eps
   w.p = G.gm1 * eps;
   w.ip = __fdividef(1.0f, w.p);
@@ -387,8 +387,8 @@ template <int DIM> __device__ inline Bracket row_bracket(const Arrays &g, const 
     err += e;
   }
   const float m = trunc_f32(g.mi[i]), e = ((float)(k1 - k0) + 16.0f) * kU;
-  if (!ok || !(m > 1e-30f && m < 1e30f && sum > 1e-30f && sum < 1e30f && e < 0.1f && err < 0.5f * sum)) return unknown;
   const float t = 0.5f * (float)g.cfl * m;
+  if (!ok || !(t > 1e-30f && m < 1e30f && sum > 1e-30f && sum < 1e30f && e < 0.1f && err < 0.5f * sum)) return unknown;
   const float lo = t / (sum + err) * (1.0f - e), hi = t / (sum - err) * (1.0f + e);
   if (!(lo > 1e-30f && hi < 1e30f)) return unknown;
   return Bracket{lo, hi};

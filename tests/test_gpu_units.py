@@ -64,3 +64,27 @@ def test_viscosity_on_very_small_meshes(nv, dim):
         d.append(s.trace(B.EH_TRACE_D_IJ))
         s.close()
     assert np.array_equal(d[0] * c_scale, d[1]), np.max(np.abs(d[1] / c_scale / d[0] - 1.0))
+
+
+@pytest.mark.parametrize("density,velocity", [(1.0, 1.0), (2.0**-90, 2.0**17), (2.0**-95, 2.0**20)])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_allocation_free_cfl_step_of_thin_gases(dim, density, velocity):
+    """Momenta of 1e-22, whose squares are below FP32's range (a gas of 1e-27 kg/m^3
+    at 1e5 m/s): the brackets still hold the bounds, and the step is eh_cfl_dt's to
+    the tolerance of the parity tests."""
+    torch = pytest.importorskip("torch")
+    mesh = M.cylinder_channel_q1(30) if dim == 2 else M.structured_q1_3d(9, 8, 10, kinds=(M.BC_SLIP,) * 6)
+    dev = lambda a, t: torch.as_tensor(np.ascontiguousarray(a, dtype=t), device="cuda")  # noqa: E731
+    isb = np.zeros(mesh.n, dtype=np.uint8)
+    isb[mesh.bnd_node] = 1
+    args = (dev(mesh.row_ptr, np.int64), dev(mesh.col, np.int32), dev(mesh.cij, np.float64), dev(mesh.mi, np.float64),
+            dev(isb, np.uint8))
+    out = torch.zeros(1, dtype=torch.float64, device="cuda")
+    s = B.Solver(dim=dim)
+    s.upload_mesh(mesh, np.ones((dim + 2, mesh.n_bnd)))
+    for seed in range(6):
+        _, U = _units(mesh, W.perturbed_state(mesh, seed), 1.0, density, velocity)
+        s.set_state(U)
+        expect = s.cfl_dt()
+        B.cfl_dt_noalloc(dim, 1.4, 0.5, *args, dev(U, np.float64), out)
+        assert abs(float(out.item()) - expect) <= 1e-13 * expect, (seed, float(out.item()), expect)
