@@ -47,8 +47,7 @@ KERNEL_NAMES = ("prep", "visc", "low", "tau", "lim1", "pass", "final", "lsearch"
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile libeuler_hyp.so for sm_103a (nvcc; no GPU needed)."""
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(CSRC, h) for h in ("kernels.cuh", "integer_fp64.cuh")] + [
-        os.path.join(_ROOT, "include", "euler_hyp.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(_ROOT, "include", "euler_hyp.h")]
     if not force and os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= max(os.path.getmtime(d) for d in deps):
         return LIB_PATH
     os.makedirs(BUILD_DIR, exist_ok=True)
