@@ -361,10 +361,11 @@ def run_reference(args, dist):
 
 
 # DRAM bytes (read + write) per CSR entry of each kernel kind, from one ncu
-# capture of the kernels as they stand (dram__bytes_read.sum +
-# dram__bytes_write.sum, 2D Q1 cylinder, FP64, 4.0M vertices, the bench's own
-# timed window; k_visc + k_alpha as "visc"); a launch moves about this times
-# nnz. None where a kernel changed after the capture.
+# capture (dram__bytes_read.sum + dram__bytes_write.sum, 2D Q1 cylinder, FP64,
+# 4.0M vertices, the bench's own timed window; k_visc + k_alpha as "visc"); a
+# launch moves about this times nnz. None where a kernel's traffic changed after
+# the capture (since it, k_alpha has one addition on another unit and k_visc and
+# k_low have one more FP32 comparison: the same bytes).
 NCU_DRAM_BYTES_PER_ENTRY_2D_FP64 = {
     "prep": 24.3, "visc": 87.2, "low": 69.6, "lim1": 53.7, "pass": 26.6, "final": 14.2,
 }

@@ -3,10 +3,11 @@
 //
 // GB300 issues an FP64 warp instruction per 19 cycles and SM (per 63 cycles and
 // warp); a division takes 7.4 and a square root 7.5 of them. The row kernels are
-// held by that pipe while the integer units, 38 times as fast, idle. With the
-// divisions and roots of k_prep, k_visc, k_alpha, k_low and the line searches here,
-// a step takes 4.21 instead of 4.50 ms (998k-vertex cylinder), 6.91 instead of 7.48
-// (375k in 3D), 0.755 instead of 0.823 (62k); the additions, 4.50 instead of 5.11.
+// held by that pipe while the integer units, 38 times as fast, idle. A step of the
+// 998k-vertex cylinder took 5.11 ms with all of it on the FP64 pipe, 4.50 with the
+// additions of k_visc, k_alpha, k_low and k_lim1 here, 4.21 with the divisions and
+// roots of k_prep, k_visc, k_alpha, k_low and the line searches too (375k in 3D 7.93,
+// 7.48, 6.91; 62k 0.823 and, with the divisions, 0.755).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -75,12 +76,13 @@ static __device__ __noinline__ double sqrt_fp64_cold(double a) { return __dsqrt_
 // a / b rounded to nearest even on the integer units, for every pair of doubles
 // (subnormal, zero, infinite or NaN operands and quotients near the range's ends go
 // to the FP64 pipe): a long division of the significands with digits of 18, 18 and
-// 17 bits. 1/D from an FP32 reciprocal (1 ulp, of D's leading 24 bits) lessened by
-// 2^-21 never exceeds it, so each digit is at most the true one and short of it by
-// less than 1.2: the remainder stays in [0, 1.2 D) and fits 64 bits, and one
-// comparison completes the 54-bit quotient, whose last bit rounds (a quotient of
-// doubles is never halfway between two). ~65 integer instructions, against 7.4
-// slots of 19 cycles on the FP64 pipe. (Compared with the FP64 division on 3e8
+// 17 bits. With D in [1, 2), the FP32 reciprocal of D's leading 24 bits is above 1/D
+// by less than 2^-23 through the bits left out and by at most 2^-24 (1 ulp) through
+// its own error; lessened by 2^-22 it never exceeds 1/D, so each digit is at most the
+// true one, and short of it by less than 1.2: the remainder stays in [0, 1.2 D) and
+// fits 64 bits, and one comparison completes the 54-bit quotient, whose last bit
+// rounds (a quotient of doubles is never halfway between two). ~65 integer
+// instructions, against 7.4 slots of 19 cycles on the FP64 pipe. (Compared with the FP64 division on 3e8
 // pairs on the CPU, the reciprocal off by up to one ulp either way, and 1.2e9 on
 // the GPU; the square root likewise.)
 __device__ __forceinline__ double div_alu(double a, double b) {

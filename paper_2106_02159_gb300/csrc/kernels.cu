@@ -87,8 +87,9 @@ __device__ __forceinline__ float trunc_f32(double x) {
 // Lanes of a row kernel read sectors of different lines (rows are 64 to 288
 // bytes apart), so L1 serves one lane's line at a time whatever the width:
 // with 8-byte loads and stores the viscosity kernel ran its L1 at 74-81 % and
-// wrote five times the sectors it had values for. The loads are of data that
-// the kernel does not write.
+// wrote five times the sectors it had values for. The compiler may move a load
+// across stores: each is of data that the kernel does not write, or (k_prep's
+// old record) its values decide a branch that the stores lie behind.
 __device__ __forceinline__ void ld4(const double *p, double &a, double &b, double &c, double &d) {
   asm("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
 }
@@ -722,8 +723,10 @@ __device__ __forceinline__ Pair operator*(const Pair &a, const Pair &b) {
   e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, e));
   return quick_pair(q, e);
 }
-// x as a pair (relative error 2^-47; exact down to 2^-126): the upper 24
-// significant bits, and the other 29 as an integer scaled by x's exponent
+// x as a pair: the upper 24 significant bits, and the other 29 as an integer
+// scaled by x's exponent. Relative error 2^-47 down to |x| = 2^-74, 2^-23 below,
+// where the low part is left out (at most 2^-97, beside tested magnitudes of 2^-12
+// and bounds of 2^-44 of them: nothing) and x itself is 0 below 2^-126
 __device__ __forceinline__ Pair split_f32(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const float h = trunc_f32(x);
@@ -1283,13 +1286,13 @@ __device__ __forceinline__ void visc_edge(const MeshView &m, const Params &p, co
 // list: in the row blocks a single such lane (a wall every few rows on small
 // meshes) would make its warp evaluate both directions (sweep of 256 small
 // cylinders: 238 -> 179 us with k_alpha).
-// Bound by FP64 issue: on a 998k-vertex cylinder, every edge general, 442 us
-// and 5.4M FP64 warp instructions (7.4M before lambda_max_sel) with the L1 at
-// 74 % of its throughput through 8-byte accesses, 358 us with 32-byte ones (FP64
-// pipe 80 % of the 84 % that it sustains), 299 us and 4.35M with the differences
-// on the integer units (ALU; pipe 78 %) and three blocks of 256 threads an SM,
-// 270 us with the division and the root there too (375k in 3D: 527 -> 420);
-// 493 us before all of these.
+// Bound by FP64 issue beside integer issue: on a 998k-vertex cylinder, every edge
+// general, 254 us and 3.21M FP64 warp instructions (FP64 pipe 67 % of the 84 % that
+// it sustains, integer units 59 %; 375k in 3D 403 us), 493 us and 7.4M before. Of
+// these, the choice of the outer wave took 7.4M to 5.4M (442 us), 32-byte accesses
+// the L1 from 74 % of its throughput (358 us), the differences on the integer units
+// (ALU) 4.35M (299 us), the division and the root there the rest. 80 registers a
+// thread, so that 768 rows run on an SM (64-thread blocks, 12 of them).
 template <int DIM, typename T, bool ALU>
 __global__ void __launch_bounds__(TPB_MAX, 3) k_visc(MeshView m, Params p, Work w, unsigned row_blocks, int lparts) {
   if (w.st->err) return;
@@ -1640,11 +1643,11 @@ __device__ __forceinline__ void fold_bound(const Work &w, double bound, int inst
 // Bound by FP64 issue. Of the 32.6 FP64 instructions an entry that a row took
 // (998k cylinder: 8.1M warp instructions, 486 us), the sums need 21; the bar
 // states' cross products, the relaxation of strict bounds, most rows' division
-// for the CFL bound and the minima's FP64 compares are gone: 26.7 (397 us); with
-// the sum of w_ij, du and (mixed) the sums around d_ij on the integer units (ALU)
-// 4.7M, 336 us: FP64 pipe 74 %, integer units 52 %, three blocks of 256 threads an
-// SM (two: 350; four, with spills: 392), mixed 360 -> 305. The bounds' two divisions
-// on the integer units: 325 us, mixed 285.
+// for the CFL bound and the minima's FP64 compares are gone (26.7, 397 us), and the
+// sum of w_ij, du, the bounds' two divisions and (mixed) the sums around d_ij are on
+// the integer units: 4.19M, 323 us, mixed 285 (FP64 pipe 68 %, integer units 55 %).
+// ALU: 80 registers a thread, 768 rows an SM (512 rows 350 us, 1024 with spills 392,
+// when 768 took 336).
 template <int DIM, typename T, bool ALU>
 __global__ void __launch_bounds__(TPB_MAX, ALU && DIM == 2 ? 3 : 2) k_low(MeshView m, Params p, Work w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2700,12 +2703,21 @@ template <int DIM> __global__ void k_count_not_admissible(int n, const double *U
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// rows below which the split forms run. Microseconds a launch, row form ->
-// split form: 4k-vertex vortex k_visc + k_alpha 22.3 -> 17.8, k_low 19.0 -> 13.6,
-// k_lim1 18.8 -> 12.1, k_pass 13.5 -> 12.7; 6.6k vortex in a box with queued
-// searches 25.6 -> 23.1, 21.4 -> 17.4, 38.5 -> 20.7, 32.0 -> 20.5; 62k cylinder
-// 53.5 -> 56.1, 38.3 -> 46.6, 55.0 -> 49.9, 41.2 -> 40.3; 196k rows: all slower.
-// (The launch shape of eh_set_launch_shape applies to the row forms.)
+// rows below which the split forms run. Microseconds a launch, row form / split
+// form, FP64, flow behind a shock (perturbed flow):
+//   2D rows           8k          24k          40k          62k          77k
+//   k_visc + k_alpha  27/21       33/29        38/38 (40/41) 46/48        50/53
+//   k_low             26/20       27/27 (23/27) 29/35       35/43        40/48
+//   k_lim1            40/20       41/29        44/39        51/49 (41/46) 56/54 (44/52)
+//   k_pass            39/22       39/24        40/28        42/38 (27/27) 43/44 (28/32)
+//   3D rows           5k          16k          29k          35k          62k          76k
+//   k_visc + k_alpha  57/35       73/53        95/75        107/88       140/130      147/141
+//   k_low             74/33       79/54        87/78 (73/64) 90/95 (76/79) 115/136     123/158
+//   k_lim1            127/40      135/60       150/95       157/107      190/153 (128/128) 215/183 (142/146)
+//   k_pass            124/57      139/64       153/78       155/112      174/156 (104/122) 193/190 (110/147)
+// In 3D the lines are where k_low and k_lim1 cross; in 2D k_low crosses earlier,
+// between 16k and 24k rows, and k_alpha later. (The launch shape of
+// eh_set_launch_shape applies to the row forms.)
 constexpr int SPLIT_SUMS = 32 * 1024;     // k_alpha, k_low: the warps repeat loads and half of the products
 constexpr int SPLIT_ENTRIES = 64 * 1024;  // k_lim1, k_pass: the entries are independent
 // Additions on the integer units (add_on<true>) in 2D k_low and k_lim1 from here
@@ -2714,7 +2726,7 @@ constexpr int SPLIT_ENTRIES = 64 * 1024;  // k_lim1, k_pass: the entries are ind
 // k_low at 78k rows behind a shock; at 103k it takes a second wave: k_low 61
 // against 50 us, k_lim1 61 against 51 (developed flow; behind a shock 45 against
 // 54 and 58 against 59), at 998k 391 against 336 and 386 against 328. 3D k_low has
-// them at every size (95k rows 175 -> 172 us), 3D k_lim1 nowhere (625 -> 642 us).
+// them from SPLIT_SUMS on (95k rows 175 -> 172 us), 3D k_lim1 nowhere (625 -> 642 us).
 constexpr int ALU_ROWS = 96 * 1024;
 bool launch_shape_used(int kernel, int64_t n, int limiter_passes) {
   switch (kernel) {
