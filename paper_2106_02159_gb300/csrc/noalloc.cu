@@ -134,7 +134,7 @@ struct Arrays {
 // orientation (from the row of min(i, j)), with the maximum over both
 // directions when both nodes are boundary nodes; 'own' is node i, derived. For
 // two states equal bit for bit the two-rarefaction pressure is the common
-// pressure, both outer waves are rarefactions and the bound is |v.n| + a: no
+// pressure, both outer waves are rarefactions and the bound is max(a - v.n, v.n + a): no
 // root, power or division (a uniform flow, where every row ties for the
 // minimum and is evaluated here, then costs a few operations an entry).
 template <int DIM>
@@ -163,8 +163,9 @@ __device__ inline double graph_viscosity(const Arrays &g, int i, int j, int64_t 
     const double cn = sqrt(s2);
     double lam;
     if (same) {
-      const double ci = 1.0 / cn;
-      lam = fabs(normal_velocity(own, c, ci)) + own.a;
+      // (as wave_bound: fmax drops the NaN of an entry with c = 0, whose d_ij is 0)
+      const double ci = 1.0 / cn, un = normal_velocity(own, c, ci);
+      lam = fmax(fmax(own.a - un, 0.0), fmax(un + own.a, 0.0));
     } else {
       const double ci = 1.0 / cn;
       const double ul = normal_velocity(l, c, ci), ur = normal_velocity(r, c, ci);
